@@ -103,6 +103,9 @@ struct hlbm {
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fv = nullptr, ev_force = nullptr, ev_move = nullptr, ev_cls = nullptr;
     bool force_pending = false;
+    // tag of the last exchange of a deep-tile FV launch: only ever grows (a
+    // restored or abandoned step never meets packets with its own tags)
+    unsigned xtag = 0;
 
     int64_t t = 0;
     double Xprev = 0, Yprev = 0;
@@ -513,6 +516,10 @@ int step_fv(hlbm* h, cudaStream_t s, PendingStep& ps, cudaEvent_t ev0 = nullptr,
         d.spin_limit = h->inject_spin_limit;
         h->inject_stall_tile = -1;
     }
+    if (h->fv_kind == HLBM_FV_DEEP) {
+        ps.a.xtag = h->xtag;
+        h->xtag += (unsigned)((d.n_sub + d.deep_k - 1) / d.deep_k);
+    }
     cudaError_t fe = h->fv_kind == HLBM_FV_DEEP   ? launch_fv_deep<T>(d, ps.a, use_far ? &far : nullptr, s)
                      : h->fv_kind == HLBM_FV_TMEM ? launch_fv_tmem<T>(d, ps.a, s)
                      : h->fv_kind == HLBM_FV_SMEM ? launch_fv_smem<T>(d, ps.a, s)
@@ -522,10 +529,9 @@ int step_fv(hlbm* h, cudaStream_t s, PendingStep& ps, cudaEvent_t ev0 = nullptr,
     if (ev1) cudaEventRecord(ev1, s);
     if (fe != cudaSuccess) return cuda_check(h, fe, "FV sub-step launch");
     h->far_ready = use_far;
-    // the state after the last sub-step is in the record buffer of the last
-    // exchange: fu_out when the number of exchanges is odd
-    const int n_exch = h->fv_kind == HLBM_FV_DEEP ? (d.n_sub + d.deep_k - 1) / d.deep_k : d.n_sub;
-    if (n_exch & 1) h->ui = 1 - h->ui;
+    // the state after the last sub-step is in fu_out (deep tiles), or in the
+    // record buffer of the last sub-step: fu_out when their number is odd
+    if (h->fv_kind == HLBM_FV_DEEP || (d.n_sub & 1)) h->ui = 1 - h->ui;
     bind(h, d);
     phase_end(h, HLBM_PHASE_FV, ev, 2, s);
     return HLBM_OK;
@@ -614,14 +620,15 @@ int step_impl(hlbm* h, int64_t nsteps) {
 // in the caller's node order (on meshes built layer by layer consecutive
 // slots then run along a layer, which spreads a warp's gathers over the
 // shared-memory banks).  Sub-step s of a block computes the own nodes and
-// layers 1 .. K-1-s.  The tiles a tile waits for are the owners of its
-// ghosts and the tiles that hold its nodes as ghosts (symmetric, so that no
-// tile can overwrite an exchange buffer a neighbour still reads).  Returns
+// layers 1 .. K-1-s.  A tile waits for the packets of its ghosts, and for the
+// progress counters of the tiles that hold its nodes as ghosts without owning
+// any of its ghosts (no tile then overwrites packets a neighbour still
+// reads).  Returns
 // false when a tile's computed slots exceed comp_cap.
 struct DeepTables {
     int K = 0, slot_cap = 0, ocap = 0;
     std::vector<int32_t> ptr, cnt, gid, optr, rptr, row_gid, lcol, nb_ptr, nb;
-    std::vector<int8_t> send;
+    std::vector<int8_t> send, pub;
     std::vector<uint16_t> oslot;
 };
 
@@ -712,18 +719,23 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
     D.send.assign(D.gid.size(), 0);
     for (int k = 0; k < n_tiles; ++k)
         for (int x = 0; x < tile_start[k + 1] - tile_start[k]; ++x) D.send[D.ptr[k] + x] = held[D.gid[D.ptr[k] + x]];
-    // symmetric neighbour sets
-    std::vector<std::vector<int32_t>> sym(n_tiles);
+    // tiles that read tile k while k does not read them: k waits for their
+    // progress counters before it overwrites packets, and they publish theirs
+    for (auto& v : nbs) {
+        std::sort(v.begin(), v.end());
+        v.erase(std::unique(v.begin(), v.end()), v.end());
+    }
+    std::vector<std::vector<int32_t>> wait(n_tiles);
+    D.pub.assign(n_tiles, 0);
     for (int k = 0; k < n_tiles; ++k)
-        for (int32_t o : nbs[k]) {
-            sym[k].push_back(o);
-            sym[o].push_back(k);
-        }
+        for (int32_t o : nbs[k])
+            if (!std::binary_search(nbs[o].begin(), nbs[o].end(), (int32_t)k)) {
+                wait[o].push_back(k);
+                D.pub[k] = 1;
+            }
     D.nb_ptr.assign(n_tiles + 1, 0);
     for (int k = 0; k < n_tiles; ++k) {
-        std::sort(sym[k].begin(), sym[k].end());
-        sym[k].erase(std::unique(sym[k].begin(), sym[k].end()), sym[k].end());
-        D.nb.insert(D.nb.end(), sym[k].begin(), sym[k].end());
+        D.nb.insert(D.nb.end(), wait[k].begin(), wait[k].end());
         D.nb_ptr[k + 1] = (int32_t)D.nb.size();
     }
     return true;
@@ -842,7 +854,7 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
     d.n_tiles = n_tiles;
     d.tile_start = (int32_t*)track(upload(h, tile_start.data(), tile_start.size(), &rc));
     if (h->fv_kind == HLBM_FV_DEEP) {
-        // the deep kernel waits for the symmetric neighbour sets of its K-deep ghost layers
+        // the counters the deep kernel waits for besides its ghosts' packets
         tile_nb_ptr = deep.nb_ptr;
         tile_nb = deep.nb;
         if (tile_nb.empty()) tile_nb.push_back(0);
@@ -864,6 +876,12 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
         if (rc != HLBM_OK) return rc;
         if (!rows || !d_rgid || !d_lcol) return fail(h, HLBM_ENOMEM, "device allocation failed");
         d.deep_rows = rows;
+        d.deep_pub = (int8_t*)track(upload(h, deep.pub.data(), deep.pub.size(), &rc));
+        const size_t xbytes = fv_deep_packet_bytes<T>(n);
+        d.deep_x = (unsigned char*)track(dev_alloc(h, xbytes));
+        if (rc != HLBM_OK) return rc;
+        if (!d.deep_x) return fail(h, HLBM_ENOMEM, "device allocation failed");
+        cudaMemsetAsync(d.deep_x, 0, xbytes, s);
         launch_build_deep_rows<T>(d, d_rgid, d_lcol, nrow, rows, s);
         cudaError_t e3 = cudaStreamSynchronize(s);
         dev_free(h, d_rgid);

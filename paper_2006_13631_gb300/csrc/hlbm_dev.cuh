@@ -151,6 +151,7 @@ struct StepArgs {
     int pbx0, pby0; // window of the previous step (previous class and state)
     int first;      // 1 at t == 0
     double v0, v1;  // INDUCED motion: lamina velocity at t and t+1
+    unsigned xtag;  // deep tiles: exchange b of this step's FV launch carries the tag xtag + b
 };
 
 // The next lattice step's stream-collide outside a rectangle, run by the
@@ -230,6 +231,8 @@ struct Dev {
     const uint16_t* deep_oslot;
     const int32_t* deep_rptr;   // [n_tiles + 1]: first computed slot of each tile in deep_rows
     const uint32_t* deep_rows;  // per computed slot: its FV row as stored in tensor memory
+    unsigned char* deep_x;      // exchange packets, two buffers of every node's record
+    const int8_t* deep_pub;     // per tile: some tile waits for its progress counter
     // shared-memory tiles: halo node lists, ELL matrices with tile-local
     // columns (own nodes first, then halo), and the nodes other tiles read
     int ell_width;            // entries per row (rows padded)
@@ -607,6 +610,7 @@ constexpr int kDeepMaxK = 4;  // most sub-steps between exchanges
 constexpr int kDeepCnt = 3 + kDeepMaxK;
 template <typename T> int fv_deep_tmem_slots();          // computed slots a tile may have
 template <typename T> int fv_deep_row_words();           // words of one row image
+template <typename T> size_t fv_deep_packet_bytes(int n); // exchange packets of n nodes
 template <typename T> size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap);
 template <typename T> int fv_deep_tile_capacity(size_t smem);
 template <typename T>

@@ -9,54 +9,12 @@
 
 #include <algorithm>
 
+#include "fv_node.cuh"
 #include "hlbm_dev.cuh"
 
 namespace hk {
 
 constexpr int kMaxRow = 64;
-
-// Patch record: f'[0..8] and the quadratic equilibrium terms
-// z = (jx^2 / rho, jx jy / rho, jy^2 / rho) at [9..11].  With j = sum_i c_i f'_i
-// and drho = sum_i f'_i,
-//   f_i^eq - w_i rho0 = w_i (drho - 1.5 (z0 + z2) + 3 c_i.j + 4.5 (cx^2 z0 + 2 cx cy z1 + cy^2 z2)),
-// linear in (drho, j, z).  For sum_k C_Pk f^eq(P_k) the drho and j parts
-// are sums of Cf_i = sum_k C_Pk f'_k,i, so only z has to be carried.
-template <typename T>
-__device__ __forceinline__ void z_of(const T (&f)[9], T rho0, T (&z)[3]) {
-    T dr = T(0), jx = T(0), jy = T(0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        dr += f[i];
-        jx = add_cx(i, jx, f[i]);
-        jy = add_cy(i, jy, f[i]);
-    }
-    T inv = T(1) / (rho0 + dr);
-    z[0] = jx * jx * inv;
-    z[1] = jx * jy * inv;
-    z[2] = jy * jy * inv;
-}
-
-// sum_k C_Pk (f^eq_k,i - w_i rho0) from Cf_i and Z = sum_k C_Pk z_k
-template <typename T>
-__device__ __forceinline__ void ceq_of(const T (&Cf)[9], const T (&Z)[3], T (&ceq)[9]) {
-    T dr = T(0), jx = T(0), jy = T(0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        dr += Cf[i];
-        jx = add_cx(i, jx, Cf[i]);
-        jy = add_cy(i, jy, Cf[i]);
-    }
-    const T q0 = dr - T(1.5) * (Z[0] + Z[2]);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        // (c_i . j) and c_i c_i : Z, i.e. Z0, Z2 or Z0 +- 2 Z1 + Z2
-        const T quad = cx_of(i) == 0 ? (cy_of(i) == 0 ? T(0) : Z[2])
-                                     : (cy_of(i) == 0 ? Z[0]
-                                                      : (cx_of(i) * cy_of(i) > 0 ? Z[0] + T(2) * Z[1]
-                                                                                 : Z[0] - T(2) * Z[1]) + Z[2]);
-        ceq[i] = w_of<T>(i) * (q0 + T(3) * cdot(i, jx, jy) + T(4.5) * quad);
-    }
-}
 
 template <typename T>
 __device__ __forceinline__ void load_f(const T* rec, T (&f)[9]) {
@@ -279,98 +237,7 @@ void launch_feed(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // Wall nodes then take the lamina velocity: f += f^eq(rho, U) - f^eq(rho, u).
 // Outer nodes take the lattice state, linear in time at theta = (m+1)/n:
 //   f = f^eq(rho, u) + (1 - 1/(2 tau_s)) f^neq   (eq. postcollision2_u).
-// The FV update of one node (eq. ulbe), shared by both FV kernels so that
-// the result of a node does not depend on the kernel or the tiling: the
-// off-diagonal entries k != P in row order, then the pivot.  With the
-// exact zero row sum g_PP = -sum_k g_Pk the streaming sums are written
-// S_i = sum_{k != P} (c_i . g_Pk) (f_k,i - f_P,i): the same number in exact
-// arithmetic, but the differences are small next to f_k, so that in FP32 the
-// products no longer round at the scale of |g| |f| (|g| ~ 1/h, h down to 0.1
-// at the wall).  c_i . g_Pk is gx, gy, gx + gy or gx - gy up to its sign.
-template <typename T>
-struct FvAcc {
-    T S[9], Cf[9], Z[3];  // S[0] stays 0 (c_0 = 0)
-};
-
-template <typename T>
-__device__ __forceinline__ void fv_acc_init(FvAcc<T>& a) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.S[i] = a.Cf[i] = T(0);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) a.Z[j] = T(0);
-}
-
-// entry (g_Pk, C_Pk) of row P with the neighbour's state f, z; fP is the
-// pivot's state
-template <typename T>
-__device__ __forceinline__ void fv_acc_entry(FvAcc<T>& a, T gx, T gy, T c, const T (&f)[9], const T (&z)[3],
-                                             const T (&fP)[9]) {
-    const T gp = gx + gy, gm = gx - gy;
-    a.S[1] += gx * (f[1] - fP[1]);
-    a.S[2] += gy * (f[2] - fP[2]);
-    a.S[3] -= gx * (f[3] - fP[3]);
-    a.S[4] -= gy * (f[4] - fP[4]);
-    a.S[5] += gp * (f[5] - fP[5]);
-    a.S[6] -= gm * (f[6] - fP[6]);
-    a.S[7] -= gp * (f[7] - fP[7]);
-    a.S[8] += gm * (f[8] - fP[8]);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.Cf[i] += c * f[i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) a.Z[k] += c * z[k];
-}
-
-// The update of eq. ulbe from the sums.  The collision sums Cf_i - ceq_i
-// carry no mass and no momentum in exact arithmetic (ceq is built from the
-// moments of Cf); their rounding residues m0 = sum_i n_i, m = sum_i c_i n_i
-// are removed by subtracting w_i (m0 + 3 c_i.m), which leaves exact values
-// unchanged and stops the residues from acting, sub-step after sub-step, as
-// spurious sources of mass and momentum.
-template <typename T>
-__device__ __forceinline__ void fv_acc_finish(const Dev<T>& d, FvAcc<T>& a, T cP, const T (&fP)[9], const T (&zP)[3],
-                                              T (&fn)[9]) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.Cf[i] += cP * fP[i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) a.Z[k] += cP * zP[k];
-    T ceq[9];
-    ceq_of(a.Cf, a.Z, ceq);
-    T nq[9], m0 = T(0), mx = T(0), my = T(0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        nq[i] = a.Cf[i] - ceq[i];
-        m0 += nq[i];
-        mx = add_cx(i, mx, nq[i]);
-        my = add_cy(i, my, nq[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        nq[i] -= w_of<T>(i) * (m0 + T(3) * cdot(i, mx, my));
-        fn[i] = fP[i] + d.dt_u * (a.S[i] - nq[i] * d.inv_tau_u);
-    }
-}
-
-// wall nodes: impose the lamina velocity, keep the non-equilibrium part
-template <typename T>
-__device__ __forceinline__ void fv_wall(const Dev<T>& d, T U, T V, T (&fn)[9]) {
-    T dr, rr, ux, uy;
-    moments_dev(fn, d.rho0, dr, rr, ux, uy);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) fn[i] += feq_dev<T>(i, dr, rr, U, V) - feq_dev<T>(i, dr, rr, ux, uy);
-}
-
-// outer nodes: the lattice state interpolated linearly in time (eq. 182,
-// Dirichlet reading); sn[j * stride], j < 12, is the state at t and
-// sn[(12 + j) * stride] the one at t + 1
-template <typename T>
-__device__ __forceinline__ void fv_outer_from(const Dev<T>& d, const T* sn, int64_t stride, int m, T (&fn)[9]) {
-    const T th = T(m + 1) / T(d.n_sub);
-    T st[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) st[j] = (T(1) - th) * sn[j * stride] + th * sn[(12 + j) * stride];
-    f_from_state(d, st, fn);
-}
-
+// The arithmetic of a node is in fv_node.cuh, shared by every FV kernel.
 template <typename T>
 __device__ __forceinline__ void fv_outer(const Dev<T>& d, int P, int m, T (&fn)[9]) {
     fv_outer_from(d, d.snap + d.outer_of[P], (int64_t)d.n_outer, m, fn);
@@ -1359,29 +1226,37 @@ cudaError_t launch_fv_tmem(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // that the updates of layer j-1 read and that are not in earlier layers
 // (outer nodes read nothing).  Sub-step s of a block of K recomputes the
 // own nodes and ghost layers 1 .. K-1-s from the tile's own data, so the
-// tile needs its neighbours' records only once per block: the own nodes
-// other tiles hold as ghosts are written to the global record buffer at the
-// end of a block, the tile releases its progress counter, and at the start
-// of the next block each tile fetches its ghost layers after acquiring its
-// neighbour tiles' counters.  Meanwhile the threads update the own nodes
-// whose rows read only own nodes (slots [0, n_a)); then one block barrier
-// per sub-step.  The arithmetic of a node is that of the other FV kernels
-// (fv_acc_*, same entry order), so the results are the same bit for bit.
+// tile needs its neighbours' records only once per block.  The arithmetic of
+// a node is that of the other FV kernels (fv_node.cuh, same entry order), so
+// the results are the same bit for bit.
+//
+// Exchange.  An own node that other tiles hold as a ghost is sent at the end
+// of a block as packets of 16 bytes, three FP32 values (one FP64 value) and
+// a tag, each stored and loaded as one 128-bit access: a reader polls the
+// packet itself, so that neither a fence, nor a flag, nor a second round
+// trip for the data stands between the sender's store and the reader's copy
+// (with the counters and cp.async copies of the other kernels, 3.8 us per
+// sub-step on a 2588-node FP32 patch at K = 2, 3.7 on 45 304 nodes and 28 on
+// 3008 FP64 nodes; with the packets and the pair arithmetic 2.4, 2.6 and
+// 17.7).  Tags are unique over the solver's life
+// (StepArgs::xtag), so a packet left by an earlier launch is never taken for
+// a new one.  Packets alternate between two buffers; a tile overwrites the
+// packets of exchange e when it sends exchange e + 2, after having received
+// exchange e + 1 of every tile it reads, which that tile sent after its reads
+// of exchange e.  A tile read by one that it does not itself read (outer
+// nodes read nothing) waits for that tile's progress counter instead.
 //
 // Slots: own nodes (those reading only own nodes first), then the ghost
 // layers in order.  Records of all slots are double-buffered in shared
-// memory; the FV rows of the computed slots live in tensor memory, one row
-// image per slot (header cP, ne, then per off-diagonal entry gx, gy, C and
-// the local slot of the column; FP64 values take two words).  Slot x is
-// updated by thread x % kDeepThreads, which reads its row image from its
-// own TMEM lane: FP32 runs 768 FV threads of two slots and loads a row
-// entry by entry (64 registers), FP64 512 threads of two slots that load a
-// row in two halves.  The FP32 block has 256 more threads (8 warps) that run
-// the next lattice step's stream-collide away from the patch (FarArgs)
-// while the FV warps step the patch: the FV work is latency-bound and the
-// lattice work bandwidth-bound, so they share the SM.  On the 4096^2
-// workload 768 FV threads of exactly two slots each also beat 1024 of one
-// or two (0.416 against 0.423 ms per step).
+// memory (pair order: f1 .. f8, f0, z0 .. z2); the FV rows of the computed
+// slots live in tensor memory, one row image per slot (header cP, ne, then
+// per off-diagonal entry gx, gy, C and the local slot of the column; FP64
+// values take two words).  Slot x is updated by thread x % kDeepFv, which
+// reads its row image from its own TMEM lane: FP32 runs 768 FV threads of
+// two slots and loads a row two entries at a time (64 registers), FP64 512
+// threads of two slots that load a row in two halves.  The FP32 block has
+// 256 more threads (8 warps) that run the next lattice step's stream-collide
+// away from the patch (FarArgs) while the FV warps step the patch.
 template <typename T>
 constexpr int kDeepThreads = sizeof(T) == 4 ? 1024 : 512;  // block size
 template <typename T>
@@ -1398,6 +1273,10 @@ static_assert(kDeepSlotWords<float> * (kDeepGroups<float> * kDeepFv<float> / 128
                   kDeepSlotWords<double> * (kDeepGroups<double> * kDeepFv<double> / 128) <= 512,
               "row images of all slots within the 512 TMEM columns");
 static_assert(1 + kTmemMaxEntries <= 8, "row image: header and 7 entries");
+template <typename T>
+constexpr int kPktValues = sizeof(T) == 4 ? 3 : 1;  // values of a 16-byte packet
+template <typename T>
+constexpr int kPkts = kSR / kPktValues<T>;  // packets of a record
 
 template <typename T>
 int fv_deep_tmem_slots() {
@@ -1406,6 +1285,10 @@ int fv_deep_tmem_slots() {
 template <typename T>
 int fv_deep_row_words() {
     return kDeepSlotWords<T>;
+}
+template <typename T>
+size_t fv_deep_packet_bytes(int n) {
+    return (size_t)2 * n * kPkts<T> * 16;
 }
 
 struct DeepSmem {
@@ -1442,68 +1325,131 @@ size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap) {
     return deep_smem_layout<T>(slot_cap, n_sub, ocap).total;
 }
 
+// ---- packets: one relaxed 128-bit access each (value bits low, tag on top)
+struct Packet {
+    unsigned long long lo, hi;
+};
+__device__ __forceinline__ void st_packet(void* p, unsigned long long lo, unsigned long long hi) {
+    asm volatile(
+        "{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p), "l"(lo),
+        "l"(hi)
+        : "memory");
+}
+__device__ __forceinline__ Packet ld_packet(const void* p) {
+    Packet k;
+    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
+                 : "=l"(k.lo), "=l"(k.hi)
+                 : "l"(p)
+                 : "memory");
+    return k;
+}
+__device__ __forceinline__ unsigned packet_tag(const Packet& k) { return (unsigned)(k.hi >> 32); }
+
+// the packets of a record of pairs (order of the shared-memory records)
+__device__ __forceinline__ void send_record(unsigned char* p, const RecP<float>& r, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    auto w = [](float v) { return (unsigned long long)__float_as_uint(v); };
+    st_packet(p, r.A.v, t | w(px(r.B)));
+    st_packet(p + 16, w(py(r.B)) | (w(px(r.C)) << 32), t | w(py(r.C)));
+    st_packet(p + 32, r.D.v, t | w(px(r.E)));
+    st_packet(p + 48, w(py(r.E)) | (w(px(r.F)) << 32), t | w(py(r.F)));
+}
+__device__ __forceinline__ void send_record(unsigned char* p, const RecP<double>& r, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    const double v[12] = {r.A.a, r.A.b, r.B.a, r.B.b, r.C.a, r.C.b, r.D.a, r.D.b, r.E.a, r.E.b, r.F.a, r.F.b};
+#pragma unroll
+    for (int k = 0; k < 12; ++k) st_packet(p + 16 * k, (unsigned long long)__double_as_longlong(v[k]), t);
+}
+// a packet's values into the record at dst (packet c of it)
+__device__ __forceinline__ void take_packet(float* dst, int c, const Packet& k) {
+    dst[3 * c] = __uint_as_float((unsigned)k.lo);
+    dst[3 * c + 1] = __uint_as_float((unsigned)(k.lo >> 32));
+    dst[3 * c + 2] = __uint_as_float((unsigned)k.hi);
+}
+__device__ __forceinline__ void take_packet(double* dst, int c, const Packet& k) {
+    dst[c] = __longlong_as_double((long long)k.lo);
+}
+
+// ---- records of pairs in shared memory (16-byte accesses)
+__device__ __forceinline__ RecP<float> ld_rec(const float* p) {
+    RecP<float> r;
+    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(p), b = *reinterpret_cast<const ulonglong2*>(p + 4),
+                     c = *reinterpret_cast<const ulonglong2*>(p + 8);
+    r.A.v = a.x, r.B.v = a.y, r.C.v = b.x, r.D.v = b.y, r.E.v = c.x, r.F.v = c.y;
+    return r;
+}
+__device__ __forceinline__ RecP<double> ld_rec(const double* p) {
+    const double2* q = reinterpret_cast<const double2*>(p);
+    RecP<double> r;
+    auto get = [&](int k) {
+        const double2 v = q[k];
+        return pk(v.x, v.y);
+    };
+    r.A = get(0), r.B = get(1), r.C = get(2), r.D = get(3), r.E = get(4), r.F = get(5);
+    return r;
+}
+__device__ __forceinline__ void st_rec(float* p, const RecP<float>& r) {
+    *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(r.A.v, r.B.v);
+    *reinterpret_cast<ulonglong2*>(p + 4) = make_ulonglong2(r.C.v, r.D.v);
+    *reinterpret_cast<ulonglong2*>(p + 8) = make_ulonglong2(r.E.v, r.F.v);
+}
+__device__ __forceinline__ void st_rec(double* p, const RecP<double>& r) {
+    double2* q = reinterpret_cast<double2*>(p);
+    auto put = [&](int k, const Pr<double>& v) { q[k] = make_double2(v.a, v.b); };
+    put(0, r.A), put(1, r.B), put(2, r.C), put(3, r.D), put(4, r.E), put(5, r.F);
+}
+template <typename T>
+__device__ __forceinline__ RecP<T> rec_of(const Pops<T>& p, const T (&z)[3]) {
+    return RecP<T>{p.A, p.B, p.C, p.D, pk(p.f0, z[0]), pk(z[1], z[2])};
+}
+
 // 16 or 32 words of this thread's TMEM lane, complete on return
 template <int N>
 __device__ __forceinline__ void tmem_ldn(uint32_t taddr, uint32_t (&v)[N]) {
-    if constexpr (N == 16) {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15}, [%16];\n\t"
-            "tcgen05.wait::ld.sync.aligned;"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(taddr)
-            : "memory");
-    } else {
-        static_assert(N == 32, "x16 or x32");
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
-            "tcgen05.wait::ld.sync.aligned;"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-              "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
-              "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
-              "=r"(v[30]), "=r"(v[31])
-            : "r"(taddr)
-            : "memory");
-    }
+    static_assert(N == 32, "x32");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
 }
 
 // entry (gx, gy, C, column) at word w of a row image half
 template <typename T, int N>
 __device__ __forceinline__ void deep_entry(const uint32_t (&v)[N], int w, T& gx, T& gy, T& c, int& col) {
-    if constexpr (sizeof(T) == 4) {
-        gx = __uint_as_float(v[w]);
-        gy = __uint_as_float(v[w + 1]);
-        c = __uint_as_float(v[w + 2]);
-        col = (int)v[w + 3];
-    } else {
-        gx = from_words<T>(v[w], v[w + 1]);
-        gy = from_words<T>(v[w + 2], v[w + 3]);
-        c = from_words<T>(v[w + 4], v[w + 5]);
-        col = (int)v[w + 6];
-    }
+    gx = from_words<T>(v[w], v[w + 1]);
+    gy = from_words<T>(v[w + 2], v[w + 3]);
+    c = from_words<T>(v[w + 4], v[w + 5]);
+    col = (int)v[w + 6];
 }
 
 // The update of slot x (warp-uniform call: lanes with valid = false take
 // part in the TMEM loads only), written into the next record buffer and,
-// when out is set, into the global record of its node.  Both halves of the
-// row image are loaded by every lane of the warp at points where the warp
-// is converged (tcgen05.ld is .sync.aligned); only the arithmetic between
-// them is predicated.
+// when pkt is set, sent to the tiles that hold the node as a ghost.  The row
+// image is loaded by every lane of the warp at points where the warp is
+// converged (tcgen05.ld is .sync.aligned); only the arithmetic between the
+// loads is predicated.
 template <typename T>
 __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* sm, const DeepSmem& L, const T* cur,
-                                          T* nxt, uint32_t tslot, bool valid, int x, int m, T* gout, bool out) {
+                                          T* nxt, uint32_t tslot, bool valid, int x, int m, unsigned char* pkt,
+                                          unsigned tag) {
     constexpr int EW = kDeepEntryWords<T>;
     const int8_t kind = valid ? reinterpret_cast<const int8_t*>(sm + L.kind)[x] : (int8_t)HLBM_NODE_OUTER;
-    T fP[9] = {};
-    if (valid && kind != HLBM_NODE_OUTER) read_rec9(cur + (size_t)kSR * x, fP);
-    FvAcc<T> acc;
-    fv_acc_init(acc);
+    Pops<T> P{};
+    if (valid && kind != HLBM_NODE_OUTER) {
+        const RecP<T> own = ld_rec(cur + (size_t)kSR * x);
+        P.A = own.A, P.B = own.B, P.C = own.C, P.D = own.D;
+    }
+    FvSums<T> acc;
+    fv_sums_init(acc);
     T cP;
     if constexpr (sizeof(T) == 4) {
-        // header, then the entries one by one up to the warp's longest row
+        // header, then the entries two by two up to the warp's longest row
         uint32_t hdr[4];
         tmem_ld4(tslot, hdr);
         cP = __uint_as_float(hdr[0]);
@@ -1516,16 +1462,12 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
             if (j >= nem) break;
             uint32_t e[8];
             tmem_ld8(tslot + EW * (j + 1), e);
-            if (j < ne) {
-                T f[9], z[3];
-                read_rec12(cur + (size_t)kSR * (int)e[3], f, z);
-                fv_acc_entry(acc, __uint_as_float(e[0]), __uint_as_float(e[1]), __uint_as_float(e[2]), f, z, fP);
-            }
-            if (j + 1 < ne) {
-                T f[9], z[3];
-                read_rec12(cur + (size_t)kSR * (int)e[7], f, z);
-                fv_acc_entry(acc, __uint_as_float(e[4]), __uint_as_float(e[5]), __uint_as_float(e[6]), f, z, fP);
-            }
+            if (j < ne)
+                fv_sums_entry(acc, __uint_as_float(e[0]), __uint_as_float(e[1]), __uint_as_float(e[2]),
+                              ld_rec(cur + (size_t)kSR * (int)e[3]), P);
+            if (j + 1 < ne)
+                fv_sums_entry(acc, __uint_as_float(e[4]), __uint_as_float(e[5]), __uint_as_float(e[6]),
+                              ld_rec(cur + (size_t)kSR * (int)e[7]), P);
         }
     } else {
         constexpr int H = kDeepHalf<T>;
@@ -1540,9 +1482,7 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
                 T gx, gy, c;
                 int col;
                 deep_entry<T, H>(v, EW * (j + 1), gx, gy, c, col);
-                T f[9], z[3];
-                read_rec12(cur + (size_t)kSR * col, f, z);
-                fv_acc_entry(acc, gx, gy, c, f, z, fP);
+                fv_sums_entry(acc, gx, gy, c, ld_rec(cur + (size_t)kSR * col), P);
             }
         }
         __syncwarp();
@@ -1553,21 +1493,17 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
                 T gx, gy, c;
                 int col;
                 deep_entry<T, H>(v, EW * (j - E0), gx, gy, c, col);
-                T f[9], z[3];
-                read_rec12(cur + (size_t)kSR * col, f, z);
-                fv_acc_entry(acc, gx, gy, c, f, z, fP);
+                fv_sums_entry(acc, gx, gy, c, ld_rec(cur + (size_t)kSR * col), P);
             }
         }
     }
     if (!valid) return;
-    T fn[9];
+    Pops<T> fn;
     if (kind == HLBM_NODE_OUTER) {
         const int q = reinterpret_cast<const int16_t*>(sm + L.omap)[x];
-        fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m, fn);
+        fn = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m);
     } else {
-        T zP[3];
-        read_z3(cur + (size_t)kSR * x, zP);
-        fv_acc_finish(d, acc, cP, fP, zP, fn);
+        fn = fv_sums_finish(d, acc, cP, ld_rec(cur + (size_t)kSR * x));
         if (kind == HLBM_NODE_WALL) {
             const T* uv = reinterpret_cast<const T*>(sm + L.uv);
             fv_wall(d, uv[m], uv[d.n_sub + m], fn);
@@ -1575,16 +1511,9 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
     }
     T z[3];
     z_of(fn, d.rho0, z);
-    T* o = nxt + (size_t)kSR * x;
-    st4(o, fn[0], fn[1], fn[2], fn[3]);
-    st4(o + 4, fn[4], fn[5], fn[6], fn[7]);
-    st4(o + 8, fn[8], z[0], z[1], z[2]);
-    if (out) {
-        T* rec = gout + (int64_t)kRec * reinterpret_cast<const int32_t*>(sm + L.gid)[x];
-        st4(rec, fn[0], fn[1], fn[2], fn[3]);
-        st4(rec + 4, fn[4], fn[5], fn[6], fn[7]);
-        st4(rec + 8, fn[8], z[0], z[1], z[2]);
-    }
+    const RecP<T> r = rec_of(fn, z);
+    st_rec(nxt + (size_t)kSR * x, r);
+    if (pkt) send_record(pkt, r, tag);
 }
 
 // One chunk of the next lattice step's stream-collide (FarArgs, FP32
@@ -1655,6 +1584,41 @@ __device__ __forceinline__ void fv_bar() {
     asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
 }
 
+// Receives the ghost records of one exchange into the ghost slots of buffer
+// cur: thread k of N (counted from the last FV thread, whose warps have the
+// fewest nodes) takes packets k, k + N, ...  Each is polled until its tag is
+// the exchange's, a bounded number of times; false when a wait ran out or
+// another tile gave up.
+template <typename T, int N>
+__device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned char* xb, const int32_t* gid, T* cur,
+                                             int n_own, int n_slot, unsigned tag, int k) {
+    constexpr int PK = kPkts<T>;
+    const int np = (n_slot - n_own) * PK;
+    bool ok = true;
+    for (int p = k; p < np && ok; p += N) {
+        const int g = p / PK, c = p - g * PK;
+        const int sl = n_own + g;
+        const unsigned char* src = xb + ((int64_t)gid[sl] * PK + c) * 16;
+        Packet v = ld_packet(src);
+        long spins = 0;
+        while (packet_tag(v) != tag) {
+            if ((spins & 63) == 63 && *(volatile unsigned*)d.abort_flag) {
+                ok = false;
+                break;
+            }
+            if (++spins > d.spin_limit) {
+                atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
+                atomicExch(d.abort_flag, 1u);
+                ok = false;
+                break;
+            }
+            v = ld_packet(src);
+        }
+        take_packet(cur + (size_t)kSR * sl, c, v);
+    }
+    return ok;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -1693,13 +1657,14 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
         kd[x] = d.kind[g];
         sd[x] = d.deep_send[s0 + x];
         om[x] = -1;
+        const T* r = g0 + (int64_t)kRec * g;
+        T* o = buf0 + (size_t)kSR * x;
+        const Vec4<T> v0 = ld4(r), v1 = ld4(r + 4), v2 = ld4(r + 8);
+        st4(o, v0.y, v0.z, v0.w, v1.x);
+        st4(o + 4, v1.y, v1.z, v1.w, v2.x);
+        st4(o + 8, v0.x, v2.y, v2.z, v2.w);
     }
     __syncthreads();
-    for (int x = tid; x < 3 * n_slot; x += BT) {
-        const int sl = x / 3, c = x - 3 * sl;
-        const Vec4<T> v = ld4(g0 + (int64_t)kRec * gid[sl] + 4 * c);
-        st4(buf0 + (size_t)kSR * sl + 4 * c, v.x, v.y, v.z, v.w);
-    }
     {
         const int o0 = d.deep_optr[tile], on = d.deep_optr[tile + 1] - o0;
         T* osn = reinterpret_cast<T*>(sm + L.osnap);
@@ -1734,98 +1699,90 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
     const unsigned long long base = (unsigned long long)a.t * (unsigned long long)d.n_sub;
     if (tid < NT) {
         const int nb0 = d.tile_nb_ptr[tile], nb1 = d.tile_nb_ptr[tile + 1];
+        const int64_t xhalf = (int64_t)d.n * kPkts<T> * 16;
+        // own nodes that read only own nodes are updated while the ghosts are on
+        // their way when they fill the FV warps; fewer are left for after the
+        // wait, since one pass over all slots then takes no longer than over a part
+        const int n_early = n_a >= NT ? n_a : 0;
         int m = 0;
         bool aborted = false;
         for (int b = 0; m < d.n_sub && !aborted; ++b) {
             const int kb = min(K, d.n_sub - m);
             const bool final_block = (m + kb == d.n_sub);
-            T* gout = (b & 1) ? g0 : g1;  // the state at the end of block b is exchange b + 1
+            // block b receives exchange b (b > 0) and sends exchange b + 1
+            unsigned char* xout = d.deep_x + ((b + 1) & 1) * xhalf;
+            const unsigned tag_out = a.xtag + (unsigned)(b + 1);
             for (int s = 0; s < kb; ++s, ++m) {
                 T* cur = (m & 1) ? buf1 : buf0;
                 T* nxt = (m & 1) ? buf0 : buf1;
-                const bool last = (s == kb - 1);
+                const bool send = (s == kb - 1) && !final_block && tile != d.stall_tile;
                 const int cs = cnt[3 + s];
                 int lo = 0;
                 if (s == 0 && b > 0) {
-                    // own nodes that read only own nodes, while warp 0 waits for
-                    // the neighbour tiles' exchange b and copies the ghost layers
-    #pragma unroll
+#pragma unroll
                     for (int j = 0; j < G; ++j) {
                         const int x = j * NT + tid;
-                        const bool v = x < n_a;
+                        const bool v = x < n_early;
                         if (__any_sync(0xffffffffu, v))
-                            deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m, gout, false);
+                            deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u);
                     }
-                    if (warp == 0) {
-                        bool ok = true;
-                        for (int e = nb0 + tid; e < nb1 && ok; e += 32) {
-                            const unsigned long long* pc = d.progress + d.tile_nb[e];
-                            long spins = 0;
-                            while (ld_acquire(pc) < base + m) {
-                                if (*(volatile unsigned*)d.abort_flag) {
-                                    ok = false;
-                                    break;
-                                }
-                                if (++spins > d.spin_limit) {
-                                    atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
-                                    atomicExch(d.abort_flag, 1u);
-                                    ok = false;
-                                    break;
-                                }
-                                __nanosleep(32);
+                    bool ok = deep_receive<T, NT>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
+                                                  a.xtag + (unsigned)b, NT - 1 - tid);
+                    // tiles that read this one but are not read by it: their reads of
+                    // the packets about to be overwritten are behind their counter
+                    for (int e = nb0 + tid; e < nb1 && ok; e += NT) {
+                        const unsigned long long* pc = d.progress + d.tile_nb[e];
+                        long spins = 0;
+                        while (ld_acquire(pc) < base + m) {
+                            if (*(volatile unsigned*)d.abort_flag) {
+                                ok = false;
+                                break;
+                            }
+                            if (++spins > d.spin_limit) {
+                                atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
+                                atomicExch(d.abort_flag, 1u);
+                                ok = false;
+                                break;
                             }
                         }
-                        __syncwarp();
-                        ok = __all_sync(0xffffffffu, ok);
-                        if (ok) {
-                            const T* gin = (b & 1) ? g1 : g0;
-                            constexpr int kChunks = kSR * (int)sizeof(T) / 16;
-                            for (int x = tid; x < kChunks * (n_slot - n_own); x += 32) {
-                                const int hs = x / kChunks, c = x - kChunks * hs;
-                                const int sl = n_own + hs;
-                                cp_async16(reinterpret_cast<unsigned char*>(cur + (size_t)kSR * sl) + 16 * c,
-                                           reinterpret_cast<const unsigned char*>(gin + (int64_t)kRec * gid[sl]) + 16 * c);
-                            }
-                        }
-                        cp_async_wait_all();
-                        if (tid == 0 && !ok) abort_sh = 1;
                     }
+                    if (!ok) abort_sh = 1;
                     fv_bar<NT>();
                     if (abort_sh) {
                         aborted = true;
                         break;
                     }
-                    // a block of one sub-step ends here: the records of those nodes go
-                    // to the exchange buffer only now, after the neighbours' counters
-                    // were acquired (a neighbour may still have been reading that
-                    // buffer's previous contents, two exchanges back, before)
-                    if (last) {
-                        for (int x = tid; x < n_a; x += NT) {
-                            if (!final_block && !sd[x]) continue;
-                            const T* r = nxt + (size_t)kSR * x;
-                            T* rec = gout + (int64_t)kRec * gid[x];
-                            const Vec4<T> a0 = ld4(r), a1 = ld4(r + 4), a2 = ld4(r + 8);
-                            st4(rec, a0.x, a0.y, a0.z, a0.w);
-                            st4(rec + 4, a1.x, a1.y, a1.z, a1.w);
-                            st4(rec + 8, a2.x, a2.y, a2.z, a2.w);
-                        }
+                    // a block of one sub-step ends here: the nodes updated early are sent
+                    // only now, after the receive (which frees the packets they overwrite)
+                    if (send) {
+                        for (int x = tid; x < n_early; x += NT)
+                            if (sd[x])
+                                send_record(xout + (int64_t)gid[x] * kPkts<T> * 16, ld_rec(nxt + (size_t)kSR * x), tag_out);
                     }
-                    lo = n_a;
+                    lo = n_early;
                 }
-    #pragma unroll
+#pragma unroll
                 for (int j = 0; j < G; ++j) {
                     const int x = j * NT + tid;
                     const bool v = x >= lo && x < cs;
                     if (__any_sync(0xffffffffu, v))
-                        deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m, gout,
-                                  last && x < n_own && (final_block || sd[x]));
+                        deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m,
+                                  send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out);
                 }
                 fv_bar<NT>();
             }
-            if (!aborted && !final_block && tid == 0 && tile != d.stall_tile) {
-                __threadfence();
+            if (!aborted && !final_block && d.deep_pub[tile] && tid == NT - 1 && tile != d.stall_tile)
                 st_release(d.progress + tile, base + m);
-            }
+        }
+        // the state after the last completed sub-step, in index order
+        const T* fin = (m & 1) ? buf1 : buf0;
+        for (int x = tid; x < n_own; x += NT) {
+            const T* r = fin + (size_t)kSR * x;
+            T* o = g1 + (int64_t)kRec * gid[x];
+            const Vec4<T> v0 = ld4(r), v1 = ld4(r + 4), v2 = ld4(r + 8);
+            st4(o, v2.x, v0.x, v0.y, v0.z);
+            st4(o + 4, v0.w, v1.x, v1.y, v1.z);
+            st4(o + 8, v1.w, v2.y, v2.z, v2.w);
         }
     } else if constexpr (sizeof(T) == 4) {
         // lattice warps: chunks of the next step's stream-collide until none is left
@@ -2836,6 +2793,7 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template cudaError_t launch_fv_tmem_pack<T>(const FvPack<T>&, int, size_t, cudaStream_t);                 \
     template int fv_deep_tmem_slots<T>();                                                                     \
     template int fv_deep_row_words<T>();                                                                      \
+    template size_t fv_deep_packet_bytes<T>(int);                                                             \
     template size_t fv_deep_smem_bytes<T>(int, int, int);                                                     \
     template int fv_deep_tile_capacity<T>(size_t);                                                            \
     template cudaError_t launch_fv_deep<T>(const Dev<T>&, const StepArgs&, const FarArgs<T>*, cudaStream_t);  \
