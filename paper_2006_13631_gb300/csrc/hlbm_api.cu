@@ -626,7 +626,7 @@ int step_impl(hlbm* h, int64_t nsteps) {
 // reads).  Returns
 // false when a tile's computed slots exceed comp_cap.
 struct DeepTables {
-    int K = 0, slot_cap = 0, ocap = 0;
+    int K = 0, slot_cap = 0, ocap = 0, comp_cap = 0;
     std::vector<int32_t> ptr, cnt, gid, optr, rptr, row_gid, lcol, nb_ptr, nb;
     std::vector<int8_t> send, pub;
     std::vector<uint16_t> oslot;
@@ -695,6 +695,7 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
         }
         const int n_comp = c[3];
         if (n_comp > comp_cap) return false;
+        D.comp_cap = std::max(D.comp_cap, n_comp);
         // computed slots: row images (columns as local slots; outer nodes
         // read none of theirs), outer slots for the staged feed
         for (int x = 0; x < n_comp; ++x) {
@@ -741,12 +742,30 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
     return true;
 }
 
+// The default number of FV tiles: one per SM, of at least 64 nodes in FP32 and
+// 16 in FP64.  An FP32 tile's sub-step is bound by latencies that do not
+// shrink with the tile below that; an FP64 one by the SM's FP64 issue rate
+// (k_fv_deep, quads), so that its nodes go to as many SMs as there are: at
+// least 64, 32, 24 and 16 nodes per tile give 13.0, 8.2, 7.7 and 7.2 us per
+// sub-step on 3008 nodes, 13.0, 8.8, 7.4 and 6.8 on 1072; 8 is no better.
+template <typename T>
+int default_tiles(int n, int sms) {
+    const int least = sizeof(T) == 8 ? 16 : 64;
+    return std::max(1, std::min(sms, (n + least - 1) / least));
+}
+
+// Computed slots of an FP64 tile up to which four lanes share a node (K = 2;
+// FV us per sub-step with quads / with a node per lane: 7.2 / 15.5 on 3008
+// nodes (152 tiles of at most 76 slots), 9.0 / 15.6 on 5464, 11.7 / 15.6 on
+// 9096, 16.8 / 18.1 on 13 188 (205 slots, about 150 computed); beyond, a quad
+// warp's larger total of FP64 instructions costs more than it hides).
+constexpr int kDeepQuadMax = 160;
+
 // FV tiles: equal ranges of the Morton-ordered nodes.  The shared-memory
 // kernel runs one block per tile, all co-resident; when a tile and its halo
 // do not fit in shared memory the global-memory kernel runs instead, with
 // as many tiles as it has co-resident blocks.  Neighbour tiles own a column
-// of a tile's rows.  n_tiles_req <= 0 picks one tile per SM (at least 64
-// nodes each).  Builds the tile tables, halo lists, ELL matrices with
+// of a tile's rows.  n_tiles_req <= 0 picks default_tiles.  Builds the tile tables, halo lists, ELL matrices with
 // tile-local columns, node orders and send flags; previous tables are
 // released.  Needs the FV matrices (d.coef).
 template <typename T>
@@ -795,7 +814,7 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
             halo_cap = std::max(halo_cap, (int)hl.size());
         }
     };
-    int n_tiles = n_tiles_req > 0 ? std::min(n_tiles_req, n) : std::max(1, std::min(sms, (n + 63) / 64));
+    int n_tiles = n_tiles_req > 0 ? std::min(n_tiles_req, n) : default_tiles<T>(n, sms);
     make_tiles(n_tiles);
     // outer nodes per tile (their feed is staged in shared memory)
     auto outer_cap = [&]() {
@@ -814,12 +833,15 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
     // deep tiles: the deepest exchange interval up to fv_depth that fits
     DeepTables deep;
     bool deep_ok = false;
+    int deep_quads = 0;
     if ((want == HLBM_FV_AUTO || want == HLBM_FV_DEEP) && max_row - 1 <= 7 && h->patch.outer_fv == 0) {
         for (int K = std::min(h->fv_depth, kDeepMaxK); K >= 1 && !deep_ok; --K) {
             if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), deep)) continue;
+            // FP64, few computed slots: four lanes per node
+            deep_quads = sizeof(T) == 8 && deep.comp_cap <= kDeepQuadMax ? deep.comp_cap : 0;
             deep_ok = deep.slot_cap < 65536 &&
                       fv_deep_tile_capacity<T>(fv_deep_smem_bytes<T>(deep.slot_cap, h->patch.n_sub,
-                                                                       std::max(deep.ocap, 1))) >= n_tiles;
+                                                                       std::max(deep.ocap, 1), deep_quads)) >= n_tiles;
         }
     }
     const size_t smem = fv_smem_bytes<T>(tile_cap, std::max(halo_cap, 1), std::max(max_row - 1, 0),
@@ -861,6 +883,7 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
         d.deep_k = deep.K;
         d.deep_slot_cap = deep.slot_cap;
         d.deep_ocap = std::max(deep.ocap, 1);
+        d.deep_quads = deep_quads;
         if (deep.oslot.empty()) deep.oslot.push_back(0);
         d.deep_ptr = (int32_t*)track(upload(h, deep.ptr.data(), deep.ptr.size(), &rc));
         d.deep_cnt = (int32_t*)track(upload(h, deep.cnt.data(), deep.cnt.size(), &rc));
@@ -1055,7 +1078,7 @@ int create_impl(hlbm* h, const hlbm_grid_t* g) {
         int devi = 0, sms = 1;
         cudaGetDevice(&devi);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, devi);
-        const int parts = std::max(1, std::min(sms, (n + 63) / 64));
+        const int parts = default_tiles<T>(n, sms);
         std::vector<int32_t> order;
         partition_order(n, h->tri.data(), nt, mkey.data(), parts, order, h->part_start);
         h->perm.assign(order.begin(), order.end());

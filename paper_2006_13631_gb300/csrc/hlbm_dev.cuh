@@ -223,6 +223,7 @@ struct Dev {
     int deep_k;
     int deep_slot_cap;          // most slots of a tile (own nodes and every ghost layer)
     int deep_ocap;              // most outer nodes among a tile's slots
+    int deep_quads;             // FP64: four lanes per node, rows in shared memory for this many computed slots (0: off)
     const int32_t* deep_ptr;    // [n_tiles + 1]: first slot of each tile in the slot arrays
     const int32_t* deep_cnt;    // [n_tiles][kDeepCnt]: n_a, n_own, n_slot, then the slots computed at block sub-step s
     const int32_t* deep_gid;    // per slot: node id
@@ -611,7 +612,7 @@ constexpr int kDeepCnt = 3 + kDeepMaxK;
 template <typename T> int fv_deep_tmem_slots();          // computed slots a tile may have
 template <typename T> int fv_deep_row_words();           // words of one row image
 template <typename T> size_t fv_deep_packet_bytes(int n); // exchange packets of n nodes
-template <typename T> size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap);
+template <typename T> size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows);
 template <typename T> int fv_deep_tile_capacity(size_t smem);
 template <typename T>
 cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>* far, cudaStream_t s);

@@ -1291,12 +1291,26 @@ size_t fv_deep_packet_bytes(int n) {
     return (size_t)2 * n * kPkts<T> * 16;
 }
 
-struct DeepSmem {
-    size_t buf0, buf1, uv, osnap, gid, kind, send, omap, total;
+// Quads (FP64, small tiles; rows in shared memory instead of tensor memory):
+// one row is 7 entries (g.c of the four axes, C, column) and a header
+struct alignas(16) QuadEntry {
+    double k[4];  // gx, gy, gx + gy, gx - gy
+    double c;
+    int32_t col, pad;
+};
+struct alignas(16) QuadRow {
+    QuadEntry e[kTmemMaxEntries];
+    double cP;
+    int32_t ne, pad;
 };
 
+struct DeepSmem {
+    size_t buf0, buf1, uv, osnap, rows, gid, kind, send, omap, total;
+};
+
+// quad_rows: computed slots whose rows are kept in shared memory (0: none)
 template <typename T>
-__host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int ocap) {
+__host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int ocap, int quad_rows) {
     auto up = [](size_t x) { return (x + 15) / 16 * 16; };
     DeepSmem L;
     size_t o = 0;
@@ -1308,6 +1322,8 @@ __host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int oca
     o = up(o + sizeof(T) * 2 * (size_t)n_sub);
     L.osnap = o;
     o = up(o + sizeof(T) * kSnap * (size_t)ocap);
+    L.rows = o;
+    o = up(o + sizeof(QuadRow) * (size_t)quad_rows);
     L.gid = o;
     o = up(o + sizeof(int32_t) * (size_t)cap);
     L.kind = o;
@@ -1321,8 +1337,8 @@ __host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int oca
 }
 
 template <typename T>
-size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap) {
-    return deep_smem_layout<T>(slot_cap, n_sub, ocap).total;
+size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows) {
+    return deep_smem_layout<T>(slot_cap, n_sub, ocap, quad_rows).total;
 }
 
 // ---- packets: one relaxed 128-bit access each (value bits low, tag on top)
@@ -1516,6 +1532,137 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
     if (pkt) send_record(pkt, r, tag);
 }
 
+// ---- FP64 quads.  FP64 instructions issue at one per 64 cycles from a warp
+// and one per 19 from an SM (measured; however many lanes are active), so a
+// warp that updates a node per lane (some 400 FP64 instructions) takes 12 us
+// even when it is alone on its SM, while the other three partitions idle.
+// On small tiles four lanes share a node: lane q of a quad holds the pair of
+// opposite directions q (x, y, (1,1), (-1,1)) and one of f0, z0, z1, z2,
+// some 110 instructions, and the sums over directions go through shuffles
+// within the quad: 7.2 us per sub-step against 17.7 on a 3008-node patch
+// (with tiles of at least 16 nodes instead of 64).  Every value is formed by the expression of fv_node.cuh,
+// so the bits are those of a node per lane.
+struct Quad {
+    int q;              // lane in the quad
+    double w;           // weight of the lane's directions
+    double sgn;         // +1 on odd lanes, -1 on even ones
+};
+__device__ __forceinline__ double qshfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src, 4); }
+
+// moments of the set whose pair (a, b) each lane holds, f0 in lane 0's e
+__device__ __forceinline__ void quad_moments(const Quad& Q, double a, double b, double e, double& m0, double& mx,
+                                             double& my) {
+    const double s = __dadd_rn(a, b), dd = __dsub_rn(a, b);
+    const double s2 = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 1));
+    const double s4 = __dadd_rn(s2, __shfl_xor_sync(0xffffffffu, s2, 2));
+    m0 = __dadd_rn(qshfl(e, 0), s4);
+    const double v = __dadd_rn(dd, __fma_rn(Q.sgn, qshfl(dd, 3), qshfl(dd, 2)));
+    mx = qshfl(v, 0);
+    my = qshfl(v, 1);
+}
+// c . (x, y) of the lane's first direction
+__device__ __forceinline__ double quad_dot(const Quad& Q, double x, double y) {
+    const double v = __fma_rn(Q.q == 3 ? -1.0 : 1.0, x, y);
+    return Q.q == 0 ? x : Q.q == 1 ? y : v;
+}
+
+// the update of the quad's slot x (every lane of the warp takes part)
+__device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned char* sm, const DeepSmem& L,
+                                          const double* cur, double* nxt, const Quad& Q, bool valid, int x, int m,
+                                          unsigned char* pkt, unsigned tag) {
+    const int q = Q.q, ia = q < 2 ? q : q + 2, ib = ia + 2, ie = 8 + q;
+    const int8_t kind = valid ? reinterpret_cast<const int8_t*>(sm + L.kind)[x] : (int8_t)HLBM_NODE_OUTER;
+    const bool row = kind != HLBM_NODE_OUTER;
+    double a = 0.0, b = 0.0, e = 0.0;
+    if (__any_sync(0xffffffffu, row)) {
+        const QuadRow* R = reinterpret_cast<const QuadRow*>(sm + L.rows) + (row ? x : 0);
+        const double* own = cur + (size_t)kSR * (row ? x : 0);
+        const double Pa = own[ia], Pb = own[ib], Pe = own[ie];
+        const int ne = row ? R->ne : 0;
+        double Sa = 0.0, Sb = 0.0, Ca = 0.0, Cb = 0.0, Ce = 0.0;
+#pragma unroll 2
+        for (int j = 0; j < ne; ++j) {
+            const double k = R->e[j].k[q], c = R->e[j].c;
+            const double* o = cur + (size_t)kSR * R->e[j].col;
+            const double fa = o[ia], fb = o[ib], fe = o[ie];
+            Sa = __fma_rn(k, __dsub_rn(fa, Pa), Sa);
+            Sb = __fma_rn(k, __dsub_rn(fb, Pb), Sb);
+            Ca = __fma_rn(c, fa, Ca);
+            Cb = __fma_rn(c, fb, Cb);
+            Ce = __fma_rn(c, fe, Ce);
+        }
+        __syncwarp();
+        Ca = __fma_rn(R->cP, Pa, Ca);
+        Cb = __fma_rn(R->cP, Pb, Cb);
+        Ce = __fma_rn(R->cP, Pe, Ce);
+        double dr, jx, jy;
+        quad_moments(Q, Ca, Cb, Ce, dr, jx, jy);
+        const double Z0 = qshfl(Ce, 1), Z1 = qshfl(Ce, 2), Z2 = qshfl(Ce, 3);
+        const double zs = __dadd_rn(Z0, Z2), q0 = __fma_rn(-1.5, zs, dr);
+        const double zd = __fma_rn(q == 3 ? -2.0 : 2.0, Z1, zs);
+        const double G = __fma_rn(4.5, q == 0 ? Z0 : q == 1 ? Z2 : zd, q0), H = __dmul_rn(3.0, quad_dot(Q, jx, jy));
+        Ca = __fma_rn(-Q.w, __dadd_rn(G, H), Ca);
+        Cb = __fma_rn(-Q.w, __dsub_rn(G, H), Cb);
+        Ce = __fma_rn(-w_of<double>(0), q0, Ce);
+        double m0, mx, my;
+        quad_moments(Q, Ca, Cb, Ce, m0, mx, my);
+        const double H2 = __dmul_rn(3.0, quad_dot(Q, mx, my));
+        Ca = __fma_rn(-Q.w, __dadd_rn(m0, H2), Ca);
+        Cb = __fma_rn(-Q.w, __dsub_rn(m0, H2), Cb);
+        Ce = __fma_rn(-w_of<double>(0), m0, Ce);
+        const double iv = q == 3 ? -d.inv_tau_u : d.inv_tau_u, dt = q == 3 ? -d.dt_u : d.dt_u;
+        a = __fma_rn(dt, __fma_rn(-iv, Ca, Sa), Pa);
+        b = __fma_rn(-dt, __fma_rn(iv, Cb, Sb), Pb);
+        e = __fma_rn(d.dt_u, __dmul_rn(-d.inv_tau_u, Ce), Pe);
+        const bool wall = kind == HLBM_NODE_WALL;
+        if (__any_sync(0xffffffffu, wall)) {
+            const double* uv = reinterpret_cast<const double*>(sm + L.uv);
+            const double U = uv[m], V = uv[d.n_sub + m];
+            quad_moments(Q, a, b, e, dr, jx, jy);
+            const double rho = __dadd_rn(d.rho0, dr), inv = 1.0 / rho;
+            const double ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
+            const double dx = __dsub_rn(U, ux), dy = __dsub_rn(V, uy), sx = __dadd_rn(U, ux), sy = __dadd_rn(V, uy);
+            const double bb = __dmul_rn(-1.5, __fma_rn(dx, sx, __dmul_rn(dy, sy)));
+            const double cd = quad_dot(Q, dx, dy);
+            const double Gw = __fma_rn(__dmul_rn(4.5, cd), quad_dot(Q, sx, sy), bb), Hw = __dmul_rn(3.0, cd);
+            const double wr = __dmul_rn(Q.w, rho);
+            if (wall) {
+                a = __fma_rn(wr, __dadd_rn(Gw, Hw), a);
+                b = __fma_rn(wr, __dsub_rn(Gw, Hw), b);
+                e = __fma_rn(__dmul_rn(w_of<double>(0), rho), bb, e);
+            }
+        }
+    }
+    if (valid && !row) {
+        const double* sn = reinterpret_cast<const double*>(sm + L.osnap) +
+                           kSnap * reinterpret_cast<const int16_t*>(sm + L.omap)[x];
+        const double th = double(m + 1) / double(d.n_sub), t0 = __dsub_rn(1.0, th);
+        auto at = [&](int j) { return __fma_rn(t0, sn[j], __dmul_rn(th, sn[12 + j])); };
+        const double dr = at(0), ux = at(1), uy = at(2), rho = __dadd_rn(d.rho0, dr);
+        const double qq = __dmul_rn(-1.5, __fma_rn(ux, ux, __dmul_rn(uy, uy))), c = quad_dot(Q, ux, uy);
+        const double G = __fma_rn(rho, __fma_rn(__dmul_rn(4.5, c), c, qq), dr), H = __dmul_rn(rho, __dmul_rn(3.0, c));
+        a = __fma_rn(d.kneq, at(4 + ia), __dmul_rn(Q.w, __dadd_rn(G, H)));
+        b = __fma_rn(d.kneq, at(4 + ib), __dmul_rn(Q.w, __dsub_rn(G, H)));
+        e = __fma_rn(d.kneq, at(3), __dmul_rn(w_of<double>(0), __fma_rn(rho, qq, dr)));
+    }
+    __syncwarp();
+    double dr, jx, jy;
+    quad_moments(Q, a, b, e, dr, jx, jy);
+    const double inv = 1.0 / __dadd_rn(d.rho0, dr), ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
+    if (q != 0) e = __dmul_rn(q == 3 ? jy : jx, q == 1 ? ux : uy);
+    if (!valid) return;
+    double* o = nxt + (size_t)kSR * x;
+    o[ia] = a;
+    o[ib] = b;
+    o[ie] = e;
+    if (pkt) {
+        const unsigned long long t = (unsigned long long)tag << 32;
+        st_packet(pkt + 16 * ia, (unsigned long long)__double_as_longlong(a), t);
+        st_packet(pkt + 16 * ib, (unsigned long long)__double_as_longlong(b), t);
+        st_packet(pkt + 16 * ie, (unsigned long long)__double_as_longlong(e), t);
+    }
+}
+
 // One chunk of the next lattice step's stream-collide (FarArgs, FP32
 // storage) on the lattice warps: row y = c / n_seg, nodes [64 seg,
 // 64 seg + 64), two per lane.  The pull and BGK arithmetic of a node is that
@@ -1630,7 +1777,8 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
     const int32_t* cnt = d.deep_cnt + kDeepCnt * tile;
     const int n_a = cnt[0], n_own = cnt[1], n_slot = cnt[2];
     const int K = d.deep_k;
-    const DeepSmem L = deep_smem_layout<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap);
+    const bool quads = sizeof(T) == 8 && d.deep_quads > 0;
+    const DeepSmem L = deep_smem_layout<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, quads ? d.deep_quads : 0);
     T* buf0 = reinterpret_cast<T*>(sm + L.buf0);
     T* buf1 = reinterpret_cast<T*>(sm + L.buf1);
     T* uv = reinterpret_cast<T*>(sm + L.uv);
@@ -1678,8 +1826,30 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
         // FV warps only)
         const int n_comp = cnt[3];
         const uint4* rows = reinterpret_cast<const uint4*>(d.deep_rows) + (int64_t)(SW / 4) * d.deep_rptr[tile];
+        if constexpr (sizeof(T) == 8) {
+            // quads: rows into shared memory, an entry per thread
+            const uint32_t* img = d.deep_rows + (int64_t)SW * d.deep_rptr[tile];
+            for (int x = tid; x < 8 * n_comp && quads; x += BT) {
+                const int sl = x >> 3, j = (x & 7) - 1;
+                QuadRow& R = reinterpret_cast<QuadRow*>(sm + L.rows)[sl];
+                const uint32_t* w = img + (int64_t)SW * sl + kDeepEntryWords<T> * (j + 1);
+                if (j < 0) {
+                    R.cP = from_words<double>(w[0], w[1]);
+                    R.ne = (int)w[2];
+                } else {
+                    const double gx = from_words<double>(w[0], w[1]), gy = from_words<double>(w[2], w[3]);
+                    QuadEntry& E = R.e[j];
+                    E.k[0] = gx;
+                    E.k[1] = gy;
+                    E.k[2] = __dadd_rn(gx, gy);
+                    E.k[3] = __dsub_rn(gx, gy);
+                    E.c = from_words<double>(w[4], w[5]);
+                    E.col = (int)w[6];
+                }
+            }
+        }
 #pragma unroll 1
-        for (int j = 0; j < G && tid < NT; ++j) {
+        for (int j = 0; j < G && tid < NT && !quads; ++j) {
             const int x = j * NT + tid;
             const bool have = x < n_comp;
             const uint32_t ts = tslot_of(j);
@@ -1703,7 +1873,11 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
         // own nodes that read only own nodes are updated while the ghosts are on
         // their way when they fill the FV warps; fewer are left for after the
         // wait, since one pass over all slots then takes no longer than over a part
-        const int n_early = n_a >= NT ? n_a : 0;
+        const int n_early = n_a >= NT && !quads ? n_a : 0;
+        Quad Q;
+        Q.q = tid & 3;
+        Q.w = w_of<double>(Q.q < 2 ? 1 : 5);
+        Q.sgn = (Q.q & 1) ? 1.0 : -1.0;
         int m = 0;
         bool aborted = false;
         for (int b = 0; m < d.n_sub && !aborted; ++b) {
@@ -1761,8 +1935,16 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                     }
                     lo = n_early;
                 }
+                if constexpr (sizeof(T) == 8) {
+                    for (int x0 = 8 * warp; x0 < cs && quads; x0 += NT / 4) {
+                        const int x = x0 + ((tid & 31) >> 2);
+                        const bool v = x < cs;
+                        quad_node(d, sm, L, cur, nxt, Q, v, x, m,
+                                  send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out);
+                    }
+                }
 #pragma unroll
-                for (int j = 0; j < G; ++j) {
+                for (int j = 0; j < G && !quads; ++j) {
                     const int x = j * NT + tid;
                     const bool v = x >= lo && x < cs;
                     if (__any_sync(0xffffffffu, v))
@@ -1835,7 +2017,7 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
     FarArgs<T> fa{};
     if (far && sizeof(T) == 4) fa = *far;
     void* args[] = {&dd, &aa, &b0, &b1, &fa};
-    const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap);
+    const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads);
     return cudaLaunchCooperativeKernel((const void*)k_fv_deep<T>, dim3(d.n_tiles), dim3(kDeepThreads<T>), args, smem,
                                        s);
 }
@@ -2794,7 +2976,7 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template int fv_deep_tmem_slots<T>();                                                                     \
     template int fv_deep_row_words<T>();                                                                      \
     template size_t fv_deep_packet_bytes<T>(int);                                                             \
-    template size_t fv_deep_smem_bytes<T>(int, int, int);                                                     \
+    template size_t fv_deep_smem_bytes<T>(int, int, int, int);                                                \
     template int fv_deep_tile_capacity<T>(size_t);                                                            \
     template cudaError_t launch_fv_deep<T>(const Dev<T>&, const StepArgs&, const FarArgs<T>*, cudaStream_t);  \
     template void launch_build_deep_rows<T>(const Dev<T>&, const int32_t*, const int32_t*, int64_t, uint32_t*, \
