@@ -126,18 +126,20 @@ __device__ __forceinline__ void pops_sub_lin(Pops<T>& p, Pr<T> ga, Pr<T> gd, T x
 // linear in (drho, j, z).  For sum_k C_Pk f^eq(P_k) the drho and j parts
 // are sums of Cf_i = sum_k C_Pk f'_k,i, so only z has to be carried.
 template <typename T>
-__device__ __forceinline__ void z_of(const Pops<T>& p, T rho0, T (&z)[3]) {
+__device__ __forceinline__ void z_of(const Pops<T>& p, T rho0, T (&z)[3], T& ux, T& uy) {
     T dr, jx, jy;
     pops_moments(p, dr, jx, jy);
     const T inv = T(1) / add_rn(rho0, dr);
-    const T ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
+    ux = mul_rn(jx, inv);
+    uy = mul_rn(jy, inv);
     z[0] = mul_rn(jx, ux);
     z[1] = mul_rn(jx, uy);
     z[2] = mul_rn(jy, uy);
 }
 template <typename T>
 __device__ __forceinline__ void z_of(const T (&f)[9], T rho0, T (&z)[3]) {
-    z_of(pops_of(f), rho0, z);
+    T ux, uy;
+    z_of(pops_of(f), rho0, z, ux, uy);
 }
 
 // The sums of one row (eq. ulbe), off-diagonal entries in row order, then the
@@ -187,10 +189,10 @@ __device__ __forceinline__ void fv_sums_entry(FvSums<T>& s, T gx, T gy, T c, con
 // m = sum_i c_i n_i are removed by subtracting w_i (m0 + 3 c_i.m), which
 // leaves exact values unchanged and stops the residues from acting, sub-step
 // after sub-step, as spurious sources of mass and momentum.
+// n receives the collision sums (residues removed).
 template <typename T>
-__device__ __forceinline__ Pops<T> fv_sums_finish(const Dev<T>& d, FvSums<T>& s, T cP, const RecP<T>& P) {
+__device__ __forceinline__ Pops<T> fv_sums_finish(const Dev<T>& d, FvSums<T>& s, T cP, const RecP<T>& P, Pops<T>& n) {
     const Pr<T> cc = pk(cP, cP);
-    Pops<T> n;
     n.A = pfma(cc, P.A, s.A);
     n.B = pfma(cc, P.B, s.B);
     n.C = pfma(cc, P.C, s.C);
@@ -225,12 +227,16 @@ __device__ __forceinline__ Pops<T> fv_sums_finish(const Dev<T>& d, FvSums<T>& s,
 // wall nodes: impose the lamina velocity, keep the non-equilibrium part:
 // f_i += w_i rho (3 c_i.(U - u) + 4.5 ((c_i.U)^2 - (c_i.u)^2) - 1.5 (U^2 - u^2)),
 // the squares as products of sums and differences
+// (the update's moments rho, u go to mo)
 template <typename T>
-__device__ __forceinline__ void fv_wall(const Dev<T>& d, T U, T V, Pops<T>& p) {
+__device__ __forceinline__ void fv_wall(const Dev<T>& d, T U, T V, Pops<T>& p, T (&mo)[3]) {
     T dr, jx, jy;
     pops_moments(p, dr, jx, jy);
     const T rho = add_rn(d.rho0, dr), inv = T(1) / rho;
     const T ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
+    mo[0] = rho;
+    mo[1] = ux;
+    mo[2] = uy;
     const T dx = sub_rn(U, ux), dy = sub_rn(V, uy), sx = add_rn(U, ux), sy = add_rn(V, uy);
     const T b = mul_rn(T(-1.5), fma_rn(dx, sx, mul_rn(dy, sy)));
     const Pr<T> bb = pk(b, b), h = pk(T(4.5), T(4.5)), three = pk(T(3), T(3));
@@ -308,13 +314,15 @@ __device__ __forceinline__ void fv_acc_finish(const Dev<T>& d, FvAcc<T>& a, T cP
     RecP<T> P;
     P.A = pk(fP[1], fP[2]), P.B = pk(fP[3], fP[4]), P.C = pk(fP[5], fP[6]), P.D = pk(fP[7], fP[8]);
     P.E = pk(fP[0], zP[0]), P.F = pk(zP[1], zP[2]);
-    pops_to(fv_sums_finish(d, s, cP, P), fn);
+    Pops<T> n;
+    pops_to(fv_sums_finish(d, s, cP, P, n), fn);
 }
 
 template <typename T>
 __device__ __forceinline__ void fv_wall(const Dev<T>& d, T U, T V, T (&fn)[9]) {
     Pops<T> p = pops_of(fn);
-    fv_wall(d, U, V, p);
+    T mo[3];
+    fv_wall(d, U, V, p, mo);
     pops_to(p, fn);
 }
 

@@ -1914,6 +1914,9 @@ struct AdjCkpt {
     int pbx0 = 0, pby0 = 0, ci = 0, si = 0, ui = 0, fi = 0;
 };
 
+// Most bytes of FV records the adjoint keeps for a segment of steps.
+constexpr size_t kAdjKeep = (size_t)8 << 30;
+
 // What the reverse of one step needs from its forward pass.
 template <typename T>
 struct AdjRec {
@@ -1929,6 +1932,7 @@ struct AdjRec {
     int32_t* rt = nullptr;
     int32_t* rd = nullptr;
     T* snap = nullptr;
+    T* rec = nullptr;  // FV sub-steps recorded by the forward step (null: recorded again by the reverse)
 };
 
 template <typename T>
@@ -2012,7 +2016,9 @@ int adj_forward_step(hlbm* h, AdjRec<T>& R) {
     cp(R.rt, d.rtype, (size_t)d.n * sizeof(int32_t));
     cp(R.rd, d.rdonor, (size_t)d.n * sizeof(int32_t));
     cp(R.snap, d.snap, (size_t)24 * std::max(d.n_outer, 1) * sizeof(T));
+    d.fv_rec = R.rec;
     rc = step_fv<T>(h, s, ps);
+    d.fv_rec = nullptr;
     if (rc == HLBM_OK) rc = step_finish<T>(h, s, ps);
     cp(R.Pnext, h->fu[h->ui], fu);
     return rc;
@@ -2021,29 +2027,42 @@ int adj_forward_step(hlbm* h, AdjRec<T>& R) {
 // adjoint buffers: adjoints in the population type, parameter sums in FP64
 template <typename T>
 struct AdjBufs {
-    T *lfA, *lfB, *lSo, *lSn, *lPn, *lPm, *lP0, *psi, *x0, *x1, *lsnap;
+    T *lfA, *lfB, *lSo, *lSn, *lPn, *lPm, *lP0, *x0, *x1, *lsnap;
     double *par, *lY, *lV;
-    int32_t* tpos;
+    Coef<T>* tco;      // transposed FV rows
+    int max_row;       // most entries of a row
+    unsigned char* px; // packets of the reverse pass, tag of its next
+    unsigned tag;
+    int32_t* order;    // patch nodes by kind
+    T *rec, *b0, *b1;  // records and patch states of one step, for steps not recorded forward
 };
 
 // reverse of step R.a.t; B.lPn holds the adjoint of the patch at t+1 on entry
 // and of the patch at t on exit, B.lfB / lfA and lSn / lSo likewise
 template <typename T>
-int adj_reverse_step(hlbm* h, const AdjRec<T>& R, AdjBufs<T>& B, T* sub, double lamF) {
+int adj_reverse_step(hlbm* h, const AdjRec<T>& R, AdjBufs<T>& B, double lamF) {
     cudaStream_t s = h->stream;
     Dev<T> dd = dev_of<T>(h);
-    const int n = dd.n, ns = dd.n_sub;
-    const size_t rec = (size_t)kRec * n;
-    // the FV sub-steps again (every state kept) and their reverse, one launch;
-    // the force at t+1 first, from the state after the last sub-step
+    const int n = dd.n;
+    // the reverse of the FV sub-steps, one launch (their records are made again
+    // first where the forward step kept none); the force at t+1 before it, from
+    // the state after the last sub-step
     dd.snap = R.snap;
-    cudaMemcpyAsync(sub, R.Pm, rec * sizeof(T), cudaMemcpyDeviceToDevice, s);
     cudaMemsetAsync(B.lsnap, 0, (size_t)24 * std::max(dd.n_outer, 1) * sizeof(T), s);
     if (lamF != 0.0) {  // the force at t+1, from the patch after the sub-steps
         dd.fu_in = R.Pnext;
         launch_adj_force<T>(dd, lamF, B.lPn, s);
     }
-    cudaError_t fe = launch_adj_fv<T>(dd, R.a, sub, B.lPn, B.x0, B.x1, B.psi, B.tpos, B.lsnap, B.par, B.lV, B.lPm, s);
+    cudaError_t fe = cudaSuccess;
+    if (!R.rec) {
+        dd.fv_rec = B.rec;
+        fe = launch_adj_fv_record<T>(dd, R.a, R.Pm, B.b0, B.b1, s);
+        dd.fv_rec = nullptr;
+    }
+    if (fe == cudaSuccess)
+        fe = launch_adj_fv<T>(dd, R.a, R.rec ? R.rec : B.rec, R.Pm, B.lPn, B.x0, B.x1, B.tco, B.lsnap, B.par, B.lV,
+                              B.lPm, B.max_row, B.px, B.tag, B.order, s);
+    B.tag += (unsigned)dd.n_sub;
     if (fe != cudaSuccess) return cuda_check(h, fe, "adjoint FV launch");
     // feed, stream-collide, eq. 178 fill, refill
     dd.sbox_old = R.sbo;
@@ -2131,6 +2150,7 @@ int adjoint_impl(hlbm* h, int64_t nsteps, double discard, double fit, double w_r
             rc = fail(h, HLBM_ENOMEM, "adjoint step records");
     }
     AdjBufs<T> B{};
+    for (int k = 0; k < n; ++k) B.max_row = std::max(B.max_row, h->row_ptr[k + 1] - h->row_ptr[k]);
     const size_t z = sizeof(T);
     B.lfA = (T*)alloc(9 * (size_t)d.plane * z);
     B.lfB = (T*)alloc(9 * (size_t)d.plane * z);
@@ -2139,23 +2159,44 @@ int adjoint_impl(hlbm* h, int64_t nsteps, double discard, double fit, double w_r
     B.lPn = (T*)alloc(9 * (size_t)n * z);
     B.lPm = (T*)alloc(9 * (size_t)n * z);
     B.lP0 = (T*)alloc(9 * (size_t)n * z);
-    B.psi = (T*)alloc(9 * (size_t)n * z);
-    B.x0 = (T*)alloc(9 * (size_t)n * z);
-    B.x1 = (T*)alloc(9 * (size_t)n * z);
+    B.x0 = (T*)alloc(kAdjPsi * (size_t)n * z);
+    B.x1 = (T*)alloc(kAdjPsi * (size_t)n * z);
     B.lsnap = (T*)alloc(24 * (size_t)std::max(d.n_outer, 1) * z);
     B.par = (double*)alloc(8 * 8);
     B.lY = (double*)alloc((size_t)(nsteps + 2) * 8);
     B.lV = (double*)alloc((size_t)(nsteps + 1) * ns * 8);
-    B.tpos = (int32_t*)alloc((size_t)std::max(h->nnz, 1) * 4);
-    T* sub = (T*)alloc((size_t)(ns + 1) * fu);
-    if (!B.lfA || !B.lfB || !B.lSo || !B.lSn || !B.lPn || !B.lPm || !B.lP0 || !B.psi || !B.x0 || !B.x1 ||
-        !B.lsnap || !B.par || !B.lY || !B.lV || !B.tpos || !sub)
+    B.tco = (Coef<T>*)alloc((size_t)std::max(h->nnz, 1) * sizeof(Coef<T>));
+    B.px = (unsigned char*)alloc(adj_packet_bytes(n));
+    B.tag = 1;
+    B.order = (int32_t*)alloc((size_t)n * 4);
+    std::vector<int32_t> order(n);
+    for (int k = 0; k < n; ++k) order[k] = k;
+    std::stable_sort(order.begin(), order.end(), [&](int32_t p, int32_t q) { return h->kind[p] < h->kind[q]; });
+    int32_t* d_tpos = (int32_t*)alloc((size_t)std::max(h->nnz, 1) * 4);
+    // records of the FV sub-steps: kept by the forward steps of a segment when
+    // the deep-tile kernel runs them and they take no more than kAdjKeep, else
+    // made again step by step
+    const size_t recb = adj_record_values(n, ns) * z;
+    bool keep = h->fv_kind == HLBM_FV_DEEP && recb * (size_t)every <= kAdjKeep;
+    T* kept = keep ? (T*)alloc(recb * (size_t)every) : nullptr;
+    keep = kept != nullptr;
+    for (int k = 0; k < every && keep; ++k) recs[k].rec = kept + (recb / z) * (size_t)k;
+    if (!keep) {
+        B.rec = (T*)alloc(recb);
+        B.b0 = (T*)alloc(fu);
+        B.b1 = (T*)alloc(fu);
+    }
+    if (!B.lfA || !B.lfB || !B.lSo || !B.lSn || !B.lPn || !B.lPm || !B.lP0 || !B.x0 || !B.x1 ||
+        !B.lsnap || !B.par || !B.lY || !B.lV || !B.tco || !B.px || !B.order || !d_tpos || (!keep && (!B.rec || !B.b0 || !B.b1)))
         rc = fail(h, HLBM_ENOMEM, "adjoint buffers");
     if (rc != HLBM_OK) {
         release();
         return rc;
     }
-    cudaMemcpyAsync(B.tpos, tpos.data(), tpos.size() * 4, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(d_tpos, tpos.data(), tpos.size() * 4, cudaMemcpyHostToDevice, s);
+    launch_adj_rows<T>(d, d_tpos, B.tco, s);
+    cudaMemsetAsync(B.px, 0, adj_packet_bytes(n), s);
+    cudaMemcpyAsync(B.order, order.data(), order.size() * 4, cudaMemcpyHostToDevice, s);
     cudaEvent_t e0, e1, e2;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -2232,7 +2273,7 @@ int adjoint_impl(hlbm* h, int64_t nsteps, double discard, double fit, double w_r
         const int64_t ta = g * every, tb = std::min<int64_t>(nsteps, ta + every);
         for (int64_t t = ta; t < tb && rc == HLBM_OK; ++t) rc = adj_forward_step<T>(h, recs[t - ta]);
         for (int64_t t = tb - 1; t >= ta && rc == HLBM_OK; --t)
-            rc = adj_reverse_step<T>(h, recs[t - ta], B, sub, lamF[t + 1]);
+            rc = adj_reverse_step<T>(h, recs[t - ta], B, lamF[t + 1]);
     }
     cudaEvent_t e3;
     cudaEventCreate(&e3);
@@ -2245,6 +2286,9 @@ int adjoint_impl(hlbm* h, int64_t nsteps, double discard, double fit, double w_r
         if (e == cudaSuccess) e = cudaMemcpyAsync(lV.data(), B.lV, lV.size() * 8, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) rc = cuda_check(h, e, "adjoint read-back");
+        unsigned st = 0;  // a wait of the reverse pass that ran out
+        if (rc == HLBM_OK) rc = sync_status(h, &st);
+        if (rc == HLBM_OK) rc = status_error(h, st);
         if (rc == HLBM_OK) {
             const double om = mo.omega, A = mo.A, ts = h->tau_s;
             for (int64_t t = 0; t <= nsteps; ++t) {

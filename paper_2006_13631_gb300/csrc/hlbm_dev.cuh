@@ -257,6 +257,7 @@ struct Dev {
     const T* fu_in;
     T* fu_out;
     T* snap;               // outer-node feed [2][12][n_outer]
+    T* fv_rec;             // reverse mode: what it needs of every FV sub-step (null: not recorded)
     int32_t* rtype;
     int32_t* rdonor;
     double* force;         // [cap][2]
@@ -644,9 +645,18 @@ void launch_gamma_sums(const double* force, int64_t t0, int64_t t1, double omega
 // adjoint of one lattice step (decisions held fixed); adjoints in the
 // population type T, parameter sums (par, lY, lV) in FP64
 template <typename T> void launch_adj_force(const Dev<T>& d, double lamF, T* lP, cudaStream_t s);
-template <typename T> cudaError_t launch_adj_fv(const Dev<T>& d, const StepArgs& a, T* sub, const T* lPn, T* x0,
-                                                T* x1, T* psi, const int32_t* tpos, T* lsnap, double* par,
-                                                double* lV, T* lPm, cudaStream_t s);
+size_t adj_record_values(int n, int n_sub);  // values of the FV records of one step (Dev::fv_rec)
+size_t adj_packet_bytes(int n);              // packets of the reverse pass (zeroed once)
+constexpr int kAdjPsi = 12;                  // values per node of the FV adjoint buffers
+// row k's entries of the transposed FV matrices (pivot first: minus the sum of the row's own g)
+template <typename T> void launch_adj_rows(const Dev<T>& d, const int32_t* tpos, Coef<T>* tco, cudaStream_t s);
+// the FV sub-steps from patch state P0 in global memory, recorded into d.fv_rec (b0, b1: patch-sized scratch)
+template <typename T> cudaError_t launch_adj_fv_record(const Dev<T>& d, const StepArgs& a, const T* P0, T* b0, T* b1,
+                                                       cudaStream_t s);
+template <typename T> cudaError_t launch_adj_fv(const Dev<T>& d, const StepArgs& a, const T* rec, const T* P0,
+                                                const T* lPn, T* x0, T* x1, const Coef<T>* tco, T* lsnap, double* par,
+                                                double* lV, T* lPm, int max_row, unsigned char* px, unsigned tag0,
+                                                const int32_t* order, cudaStream_t s);
 template <typename T> void launch_adj_feed(const Dev<T>& d, const StepArgs& a, const T* lsnap, T* lSo, T* lSn,
                                            double* lY, cudaStream_t s);
 template <typename T> void launch_adj_stream(const Dev<T>& d, const StepArgs& a, const T* lfB, const T* lSn, T* lfA,

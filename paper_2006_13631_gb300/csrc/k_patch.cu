@@ -1444,16 +1444,42 @@ __device__ __forceinline__ void deep_entry(const uint32_t (&v)[N], int w, T& gx,
     col = (int)v[w + 6];
 }
 
+// Record of one node's sub-step for the reverse mode (StepArgs-wide buffer
+// Dev::fv_rec, [n_sub][n][kAdjRec]): the collision sums n_1 .. n_8, n_0, the
+// velocity of the state before the sub-step, and at wall nodes rho and u of
+// the update before the wall rule.
+constexpr int kAdjRec = 16;
+enum { kAdjN0 = 8, kAdjU = 9, kAdjWall = 11 };
+
+template <typename T>
+__device__ __forceinline__ void adj_record(const Dev<T>& d, int m, int g, bool row, const Pops<T>& n, bool wall,
+                                           const T (&mo)[3], T ux, T uy) {
+    T* r = d.fv_rec + ((int64_t)m * d.n + g) * kAdjRec;
+    if (row) {
+        const T v[9] = {px(n.A), py(n.A), px(n.B), py(n.B), px(n.C), py(n.C), px(n.D), py(n.D), n.f0};
+#pragma unroll
+        for (int i = 0; i < 9; ++i) r[i] = v[i];
+        if (wall) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) r[kAdjWall + j] = mo[j];
+        }
+    }
+    if (m + 1 < d.n_sub) {  // the velocity of the next sub-step's state
+        r[(int64_t)d.n * kAdjRec + kAdjU] = ux;
+        r[(int64_t)d.n * kAdjRec + kAdjU + 1] = uy;
+    }
+}
+
 // The update of slot x (warp-uniform call: lanes with valid = false take
 // part in the TMEM loads only), written into the next record buffer and,
 // when pkt is set, sent to the tiles that hold the node as a ghost.  The row
 // image is loaded by every lane of the warp at points where the warp is
 // converged (tcgen05.ld is .sync.aligned); only the arithmetic between the
 // loads is predicated.
-template <typename T>
+template <typename T, bool kRecord>
 __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* sm, const DeepSmem& L, const T* cur,
                                           T* nxt, uint32_t tslot, bool valid, int x, int m, unsigned char* pkt,
-                                          unsigned tag) {
+                                          unsigned tag, bool own_slot) {
     constexpr int EW = kDeepEntryWords<T>;
     const int8_t kind = valid ? reinterpret_cast<const int8_t*>(sm + L.kind)[x] : (int8_t)HLBM_NODE_OUTER;
     Pops<T> P{};
@@ -1514,19 +1540,25 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
         }
     }
     if (!valid) return;
-    Pops<T> fn;
+    Pops<T> fn, nq{};
+    T mo[3] = {};
     if (kind == HLBM_NODE_OUTER) {
         const int q = reinterpret_cast<const int16_t*>(sm + L.omap)[x];
         fn = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m);
     } else {
-        fn = fv_sums_finish(d, acc, cP, ld_rec(cur + (size_t)kSR * x));
+        fn = fv_sums_finish(d, acc, cP, ld_rec(cur + (size_t)kSR * x), nq);
         if (kind == HLBM_NODE_WALL) {
             const T* uv = reinterpret_cast<const T*>(sm + L.uv);
-            fv_wall(d, uv[m], uv[d.n_sub + m], fn);
+            fv_wall(d, uv[m], uv[d.n_sub + m], fn, mo);
         }
     }
-    T z[3];
-    z_of(fn, d.rho0, z);
+    T z[3], ux, uy;
+    z_of(fn, d.rho0, z, ux, uy);
+    if constexpr (kRecord) {
+        if (own_slot)
+            adj_record(d, m, reinterpret_cast<const int32_t*>(sm + L.gid)[x], kind != HLBM_NODE_OUTER, nq,
+                       kind == HLBM_NODE_WALL, mo, ux, uy);
+    }
     const RecP<T> r = rec_of(fn, z);
     st_rec(nxt + (size_t)kSR * x, r);
     if (pkt) send_record(pkt, r, tag);
@@ -1567,9 +1599,15 @@ __device__ __forceinline__ double quad_dot(const Quad& Q, double x, double y) {
 }
 
 // the update of the quad's slot x (every lane of the warp takes part)
+template <bool kRecord>
 __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned char* sm, const DeepSmem& L,
                                           const double* cur, double* nxt, const Quad& Q, bool valid, int x, int m,
-                                          unsigned char* pkt, unsigned tag) {
+                                          unsigned char* pkt, unsigned tag, bool own_slot) {
+    double* rec = nullptr;  // this sub-step's record of the node
+    if constexpr (kRecord) {
+        if (valid && own_slot)
+            rec = d.fv_rec + ((int64_t)m * d.n + reinterpret_cast<const int32_t*>(sm + L.gid)[x]) * kAdjRec;
+    }
     const int q = Q.q, ia = q < 2 ? q : q + 2, ib = ia + 2, ie = 8 + q;
     const int8_t kind = valid ? reinterpret_cast<const int8_t*>(sm + L.kind)[x] : (int8_t)HLBM_NODE_OUTER;
     const bool row = kind != HLBM_NODE_OUTER;
@@ -1615,6 +1653,13 @@ __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned c
         b = __fma_rn(-dt, __fma_rn(iv, Cb, Sb), Pb);
         e = __fma_rn(d.dt_u, __dmul_rn(-d.inv_tau_u, Ce), Pe);
         const bool wall = kind == HLBM_NODE_WALL;
+        if constexpr (kRecord) {
+            if (rec && row) {
+                rec[ia] = Ca;
+                rec[ib] = Cb;
+                if (q == 0) rec[kAdjN0] = Ce;
+            }
+        }
         if (__any_sync(0xffffffffu, wall)) {
             const double* uv = reinterpret_cast<const double*>(sm + L.uv);
             const double U = uv[m], V = uv[d.n_sub + m];
@@ -1626,6 +1671,9 @@ __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned c
             const double cd = quad_dot(Q, dx, dy);
             const double Gw = __fma_rn(__dmul_rn(4.5, cd), quad_dot(Q, sx, sy), bb), Hw = __dmul_rn(3.0, cd);
             const double wr = __dmul_rn(Q.w, rho);
+            if constexpr (kRecord) {
+                if (rec && wall && q < 3) rec[kAdjWall + q] = q == 0 ? rho : q == 1 ? ux : uy;
+            }
             if (wall) {
                 a = __fma_rn(wr, __dadd_rn(Gw, Hw), a);
                 b = __fma_rn(wr, __dsub_rn(Gw, Hw), b);
@@ -1650,6 +1698,9 @@ __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned c
     quad_moments(Q, a, b, e, dr, jx, jy);
     const double inv = 1.0 / __dadd_rn(d.rho0, dr), ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
     if (q != 0) e = __dmul_rn(q == 3 ? jy : jx, q == 1 ? ux : uy);
+    if constexpr (kRecord) {
+        if (rec && m + 1 < d.n_sub && q < 2) rec[(int64_t)d.n * kAdjRec + kAdjU + q] = q == 0 ? ux : uy;
+    }
     if (!valid) return;
     double* o = nxt + (size_t)kSR * x;
     o[ia] = a;
@@ -1766,7 +1817,8 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
     return ok;
 }
 
-template <typename T>
+// kRecord: also writes what the reverse mode needs of every sub-step (Dev::fv_rec)
+template <typename T, bool kRecord>
 __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int abort_sh;
@@ -1898,7 +1950,7 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                         const int x = j * NT + tid;
                         const bool v = x < n_early;
                         if (__any_sync(0xffffffffu, v))
-                            deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u);
+                            deep_node<T, kRecord>(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u, true);
                     }
                     bool ok = deep_receive<T, NT>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
                                                   a.xtag + (unsigned)b, NT - 1 - tid);
@@ -1939,8 +1991,10 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                     for (int x0 = 8 * warp; x0 < cs && quads; x0 += NT / 4) {
                         const int x = x0 + ((tid & 31) >> 2);
                         const bool v = x < cs;
-                        quad_node(d, sm, L, cur, nxt, Q, v, x, m,
-                                  send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out);
+                        quad_node<kRecord>(
+                            d, sm, L, cur, nxt, Q, v, x, m,
+                            send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out,
+                            x < n_own);
                     }
                 }
 #pragma unroll
@@ -1948,8 +2002,10 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                     const int x = j * NT + tid;
                     const bool v = x >= lo && x < cs;
                     if (__any_sync(0xffffffffu, v))
-                        deep_node(d, sm, L, cur, nxt, tslot_of(j), v, x, m,
-                                  send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out);
+                        deep_node<T, kRecord>(
+                            d, sm, L, cur, nxt, tslot_of(j), v, x, m,
+                            send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out,
+                            x < n_own);
                 }
                 fv_bar<NT>();
             }
@@ -1991,21 +2047,23 @@ int fv_deep_tile_capacity(size_t smem) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, (const void*)k_fv_deep<T>) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    const int limit = maxsm - (int)fa.sharedSizeBytes;
-    if (smem > (size_t)limit) return 0;
-    if (cudaFuncSetAttribute((const void*)k_fv_deep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
     // each block allocates all 512 TMEM columns: only one block per SM
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, (const void*)k_fv_deep<T>, kDeepThreads<T>, smem);
-    return per == 1 ? sms : 0;
+    for (const void* fn : {(const void*)k_fv_deep<T, false>, (const void*)k_fv_deep<T, true>}) {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        const int limit = maxsm - (int)fa.sharedSizeBytes;
+        if (smem > (size_t)limit) return 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kDeepThreads<T>, smem);
+        if (per != 1) return 0;
+    }
+    return sms;
 }
 
 template <typename T>
@@ -2018,8 +2076,8 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
     if (far && sizeof(T) == 4) fa = *far;
     void* args[] = {&dd, &aa, &b0, &b1, &fa};
     const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads);
-    return cudaLaunchCooperativeKernel((const void*)k_fv_deep<T>, dim3(d.n_tiles), dim3(kDeepThreads<T>), args, smem,
-                                       s);
+    const void* fn = d.fv_rec ? (const void*)k_fv_deep<T, true> : (const void*)k_fv_deep<T, false>;
+    return cudaLaunchCooperativeKernel(fn, dim3(d.n_tiles), dim3(kDeepThreads<T>), args, smem, s);
 }
 
 // Row image of computed slot i: header (C_PP, entry count), then the
@@ -2288,76 +2346,102 @@ void launch_gamma_resid(const double* force, int64_t t0, int64_t t1, double omeg
 // so that d feq_i / d f_j = A_i + B_i . (c_j - u) / rho, and the transpose
 // product is (J^T l)_j = a + b . (c_j - u) / rho with a = sum_i l_i A_i,
 // b = sum_i l_i B_i.
+// The sums run over pairs of opposite directions (c_opp = -c_i: the even terms
+// take l_i + l_opp, the odd ones l_i - l_opp) and use 1 / rho once: an FP64
+// division is some ten FP64 instructions, which issue at 1/64 of the FP32 rate.
 template <typename R>
-__device__ __forceinline__ void feq_ab(int i, R rho, R ux, R uy, R& A, R& Bx, R& By) {
-    const R w = w_of<R>(i), cx = R(cx_of(i)), cy = R(cy_of(i));
-    const R cu = cx * ux + cy * uy, usq = ux * ux + uy * uy;
-    A = w * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * usq);
-    Bx = w * rho * (R(3) * cx + R(9) * cu * cx - R(3) * ux);
-    By = w * rho * (R(3) * cy + R(9) * cu * cy - R(3) * uy);
+__device__ __forceinline__ void mom_d(const R (&f)[9], R rho0, R& dr, R& rho, R& ux, R& uy, R& inv) {
+    R m0, mx, my;
+    pops_moments(pops_of(f), m0, mx, my);
+    dr = m0;
+    rho = rho0 + m0;
+    inv = R(1) / rho;
+    ux = mx * inv;
+    uy = my * inv;
 }
-
 template <typename R>
 __device__ __forceinline__ void mom_d(const R (&f)[9], R rho0, R& dr, R& rho, R& ux, R& uy) {
-    R r = 0, jx = 0, jy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        r += f[i];
-        jx += R(cx_of(i)) * f[i];
-        jy += R(cy_of(i)) * f[i];
-    }
-    dr = r;
-    rho = rho0 + r;
-    ux = jx / rho;
-    uy = jy / rho;
+    R inv;
+    mom_d(f, rho0, dr, rho, ux, uy, inv);
 }
 
+// f_i^eq - w_i rho0 for all i
 template <typename R>
-__device__ __forceinline__ R feq_d(int i, R dr, R rho, R ux, R uy) {
-    const R cu = R(cx_of(i)) * ux + R(cy_of(i)) * uy, usq = ux * ux + uy * uy;
-    return w_of<R>(i) * (dr + rho * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * usq));
+__device__ __forceinline__ void feq_all(R dr, R rho, R ux, R uy, R (&e)[9]) {
+    const R q = R(-1.5) * (ux * ux + uy * uy);
+    e[0] = w_of<R>(0) * (dr + rho * q);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        if (opp_of(i) < i) continue;
+        const R cu = cdot(i, ux, uy), G = dr + rho * (R(4.5) * cu * cu + q), H = rho * (R(3) * cu);
+        e[i] = w_of<R>(i) * (G + H);
+        e[opp_of(i)] = w_of<R>(i) * (G - H);
+    }
 }
 
-// out += scale * J_feq(f)^T lam, J at the moments (dr, rho, u) of f
+// a = sum_i l_i A_i, b = sum_i l_i B_i / rho at velocity u
 template <typename R>
-__device__ __forceinline__ void jfeqT_add(R rho, R ux, R uy, const R (&lam)[9], R scale, R (&out)[9]) {
-    R a = 0, bx = 0, by = 0;
+__device__ __forceinline__ void feq_ab(R ux, R uy, const R (&l)[9], R& a, R& bx, R& by) {
+    const R z = R(1) - R(1.5) * (ux * ux + uy * uy);
+    R ws = w_of<R>(0) * l[0];
+    a = z * ws;
+    R tx = R(0), ty = R(0);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        R A, Bx, By;
-        feq_ab(i, rho, ux, uy, A, Bx, By);
-        a += lam[i] * A;
-        bx += lam[i] * Bx;
-        by += lam[i] * By;
+    for (int i = 1; i < 9; ++i) {
+        if (opp_of(i) < i) continue;
+        const R s = l[i] + l[opp_of(i)], d = l[i] - l[opp_of(i)], cu = cdot(i, ux, uy), w = w_of<R>(i);
+        a += w * ((z + R(4.5) * cu * cu) * s + R(3) * cu * d);
+        const R t = w * (R(3) * d + R(9) * cu * s);
+        ws += w * s;
+        tx = add_cx(i, tx, t);
+        ty = add_cy(i, ty, t);
     }
+    bx = tx - R(3) * ux * ws;
+    by = ty - R(3) * uy * ws;
+}
+
+// out += scale * (g + b . c_j)
+template <typename R>
+__device__ __forceinline__ void lin_add(R g, R bx, R by, R scale, R (&out)[9]) {
+    out[0] += scale * g;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) out[j] += scale * (a + (bx * (R(cx_of(j)) - ux) + by * (R(cy_of(j)) - uy)) / rho);
+    for (int j = 1; j < 9; ++j) out[j] += scale * (g + cdot(j, bx, by));
+}
+
+// out += scale * J_feq(f)^T lam, J at the velocity u of f
+template <typename R>
+__device__ __forceinline__ void jfeqT_add(R ux, R uy, const R (&lam)[9], R scale, R (&out)[9]) {
+    R a, bx, by;
+    feq_ab(ux, uy, lam, a, bx, by);
+    lin_add(a - bx * ux - by * uy, bx, by, scale, out);
 }
 
 // the interpolated state s(f) = (dr, ux, uy, f^neq[9]) of a deviation set
 template <typename R>
 __device__ __forceinline__ void state_d(const R (&f)[9], R rho0, R (&st)[12]) {
-    R dr, rho, ux, uy;
+    R dr, rho, ux, uy, e[9];
     mom_d(f, rho0, dr, rho, ux, uy);
     st[0] = dr;
     st[1] = ux;
     st[2] = uy;
+    feq_all(dr, rho, ux, uy, e);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) st[3 + i] = f[i] - feq_d(i, dr, rho, ux, uy);
+    for (int i = 0; i < 9; ++i) st[3 + i] = f[i] - e[i];
 }
 
-// out += scale * (d s / d f)^T ls
+// out += scale * (d s / d f)^T ls, st the state of the set
 template <typename R>
-__device__ __forceinline__ void stateT_add(const R (&f)[9], R rho0, const R (&ls)[12], R scale, R (&out)[9]) {
-    R dr, rho, ux, uy;
-    mom_d(f, rho0, dr, rho, ux, uy);
-    R ln[9];
+__device__ __forceinline__ void stateT_add(const R (&st)[12], R rho0, const R (&ls)[12], R scale, R (&out)[9]) {
+    const R inv = R(1) / (rho0 + st[0]), ux = st[1], uy = st[2];
+    R ln[9], a, bx, by;
 #pragma unroll
     for (int j = 0; j < 9; ++j) {
         ln[j] = ls[3 + j];
-        out[j] += scale * (ls[0] + (ls[1] * (R(cx_of(j)) - ux) + ls[2] * (R(cy_of(j)) - uy)) / rho + ls[3 + j]);
+        out[j] += scale * ls[3 + j];
     }
-    jfeqT_add(rho, ux, uy, ln, -scale, out);
+    feq_ab(ux, uy, ln, a, bx, by);
+    const R gx = ls[1] * inv - bx, gy = ls[2] * inv - by;
+    lin_add(ls[0] - a - gx * ux - gy * uy, gx, gy, scale, out);
 }
 
 // f = f^eq(st) + k f^neq(st) (eq. continuity_stresses with k = 1 - 1/(2 tau_s),
@@ -2366,20 +2450,18 @@ __device__ __forceinline__ void stateT_add(const R (&f)[9], R rho0, const R (&ls
 template <typename R>
 __device__ __forceinline__ void ffsT(const R (&st)[12], R rho0, R k, const R (&lf)[9], R (&ls)[12], double& lk) {
     const R rho = rho0 + st[0];
-    R a = 0, bx = 0, by = 0;
+    R a, bx, by;
+    feq_ab(st[1], st[2], lf, a, bx, by);
+    R dot = R(0);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        R A, Bx, By;
-        feq_ab(i, rho, st[1], st[2], A, Bx, By);
-        a += lf[i] * A;
-        bx += lf[i] * Bx;
-        by += lf[i] * By;
         ls[3 + i] = k * lf[i];
-        lk += lf[i] * st[3 + i];
+        dot += lf[i] * st[3 + i];
     }
+    lk += double(dot);
     ls[0] = a;
-    ls[1] = bx;
-    ls[2] = by;
+    ls[1] = rho * bx;
+    ls[2] = rho * by;
 }
 
 template <typename T>
@@ -2449,219 +2531,489 @@ __global__ void k_adj_force(Dev<T> d, double lamF, T* lP) {
             ln[i] = -(lxy * cx_of(i) * cy_of(i) + lyy * cy_of(i) * cy_of(i));
             out[i] = -lyy / 3.0 + ln[i];
         }
-        jfeqT_add(rho, ux, uy, ln, T(-1), out);
+        jfeqT_add(ux, uy, ln, T(-1), out);
         atomic_add9(lP + 9 * (int64_t)P, out);
     }
 }
 
-// The FV update of a regular node P from state `in`: the updated
-// populations fv and the collision sums Cf_i - ceq_i (eq. ulbe).
+// ---- reverse of the FV sub-steps.  With psi_P the adjoint of node P's update
+// (through the wall rule at wall nodes, zero at outer nodes), the adjoint of
+// state k before the sub-step is
+//   psi_k + sum_P [ dt (c_j . g_Pk) psi_P,j - dt / tau_u C_Pk psi_P,j ]
+//         + dt / tau_u (J_feq(k)^T sum_P C_Pk psi_P)_j
+// over the rows P that read k.  psi of the sub-step before it is formed from
+// that at the node itself, so a sub-step is one pass and one grid barrier.
+// It needs only what the forward sub-step recorded (adj_record): its collision
+// sums, velocities and the wall moments; J_feq needs u alone, since its B
+// terms carry the rho they are divided by.  Four lanes share a node as in the
+// FP64 quads of the forward kernel: lane q holds the pair of opposite
+// directions q, f0 rides on lane 0.  Bound by the FP64 issue rate of a warp
+// (64 cycles an instruction) in FP64, by the exchange between SMs in FP32.
+// Reverse sweep of 48 steps on the 3008-node FP64 patch (n = 50): 404 ms with
+// a node per thread on 24 SMs, three grid barriers per sub-step and the sums
+// formed again, 62 ms so; 160 steps of the 2588-node FP32 patch (n = 96):
+// 664 ms and 115 ms.
 template <typename T>
-__device__ __forceinline__ void fv_update_d(const Dev<T>& d, const T* in, int P, T (&fv)[9], T (&cneq)[9]) {
-    const T rho0 = T(d.rho0);
-    T S[9], Cf[9], Z[3] = {0, 0, 0}, gpx = 0, gpy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) S[i] = Cf[i] = 0.0;
-    const int r0 = d.row_ptr[P], r1 = d.row_ptr[P + 1];
-    for (int e = r0 + 1; e < r1; ++e) {
-        const Coef<T> c = d.coef[e];
-        T f[9], zz[3];
-        load_d(in + (int64_t)kRec * c.col, f);
-        T dr, rho, ux, uy;
-        mom_d(f, rho0, dr, rho, ux, uy);
-        zz[0] = ux * ux * rho;
-        zz[1] = ux * uy * rho;
-        zz[2] = uy * uy * rho;
-        const T gx = T(c.gx), gy = T(c.gy), cc = T(c.c);
-        gpx -= gx;
-        gpy -= gy;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            S[i] += (cx_of(i) * gx + cy_of(i) * gy) * f[i];
-            Cf[i] += cc * f[i];
-        }
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Z[j] += cc * zz[j];
-    }
-    T fP[9];
-    load_d(in + (int64_t)kRec * P, fP);
-    {
-        T dr, rho, ux, uy;
-        mom_d(fP, rho0, dr, rho, ux, uy);
-        const T cc = T(d.coef[r0].c);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            S[i] += (cx_of(i) * gpx + cy_of(i) * gpy) * fP[i];
-            Cf[i] += cc * fP[i];
-        }
-        Z[0] += cc * ux * ux * rho;
-        Z[1] += cc * ux * uy * rho;
-        Z[2] += cc * uy * uy * rho;
-    }
-    // sum_k C (f^eq_k) from the linear parts Cf and the quadratic ones Z
-    T dr = 0, jx = 0, jy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        dr += Cf[i];
-        jx += cx_of(i) * Cf[i];
-        jy += cy_of(i) * Cf[i];
-    }
-    const T q0 = dr - 1.5 * (Z[0] + Z[2]);
-    const T inv = T(d.inv_tau_u), dt = T(d.dt_u);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const T cx = cx_of(i), cy = cy_of(i);
-        const T ceq = w_of<T>(i) * (q0 + 3.0 * (cx * jx + cy * jy) +
-                                              4.5 * (cx * cx * Z[0] + 2.0 * cx * cy * Z[1] + cy * cy * Z[2]));
-        cneq[i] = Cf[i] - ceq;
-        fv[i] = fP[i] + dt * (S[i] - inv * cneq[i]);
-    }
+struct AQuad {
+    int q, ia, ib;
+    T w;    // weight of the lane's directions
+    T sgn;  // +1 where the first direction's c . g is +g (lanes 0 .. 2), -1 on lane 3
+};
+template <typename T>
+__device__ __forceinline__ AQuad<T> aquad() {
+    AQuad<T> Q;
+    Q.q = threadIdx.x & 3;
+    Q.ia = Q.q < 2 ? Q.q : Q.q + 2;
+    Q.ib = Q.ia + 2;
+    Q.w = w_of<T>(Q.q < 2 ? 1 : 5);
+    Q.sgn = Q.q == 3 ? T(-1) : T(1);
+    return Q;
+}
+template <typename T>
+__device__ __forceinline__ T aq_shfl(T v, int src) {
+    return __shfl_sync(0xffffffffu, v, src, 4);
+}
+template <typename T>
+__device__ __forceinline__ T aq_sum(T v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+}
+template <typename T>
+__device__ __forceinline__ T aq_dot(const AQuad<T>& Q, T x, T y) {
+    return Q.q == 0 ? x : Q.q == 1 ? y : Q.sgn * x + y;
+}
+// a = sum_i l_i A_i and b = sum_i l_i B_i / rho at velocity u of the set l
+// (pair la, lb on each lane, l0 on lane 0): see feq_ab
+template <typename T>
+__device__ __forceinline__ void aq_feq(const AQuad<T>& Q, T ux, T uy, T la, T lb, T l0, T& a, T& bx, T& by) {
+    const T s = la + lb, dd = la - lb, cu = aq_dot(Q, ux, uy), us = T(1) - T(1.5) * (ux * ux + uy * uy);
+    const T z = Q.q == 0 ? w_of<T>(0) * l0 : T(0);
+    const T ws = aq_sum(Q.w * s + z);
+    a = aq_sum(Q.w * ((us + T(4.5) * cu * cu) * s + T(3) * cu * dd) + us * z);
+    const T t = Q.w * (T(3) * dd + T(9) * cu * s);
+    const T t2 = aq_shfl(t, 2), t3 = aq_shfl(t, 3);
+    bx = aq_shfl(t, 0) + (t2 - t3) - T(3) * ux * ws;
+    by = aq_shfl(t, 1) + (t2 + t3) - T(3) * uy * ws;
 }
 
-// Reverse of sub-step m, first pass at node P: psi_P, the adjoint of its
-// FV update (through the wall rule at wall nodes), the outer nodes' feed
-// adjoint, and the parameter terms (1/tau_u, kneq, wall velocity) added to
-// the caller's sums.
+// What a quad holds of its node: at outer nodes the lattice state at t and
+// t + 1 (drho, ux, uy, f^neq of the lane's pair and f^neq_0) and the sums of
+// its adjoint (the lane's share: its pair, and f^neq_0 with drho, ux or uy)
 template <typename T>
-__device__ __forceinline__ void adj_psi_node(const Dev<T>& d, const StepArgs& a, const T* in, int m, const T* lnext,
-                                             T* psi, T* lsnap, int P, T& l_inv, double& l_kneq, T& l_v) {
-    const int8_t kind = d.kind[P];
-    T lam[9], ps[9];
+struct ANode {
+    int k;
+    int8_t kind;
+    bool valid;
+    T s0[6], s1[6];
+    T g0[4], g1[4];
+};
+// what sub-step m's record gives the lane: its collision sums and the wall moments
+template <typename T>
+struct ARec {
+    T na, nb, n0, rho, wx, wy;
+};
+
+template <typename T>
+__device__ __forceinline__ ANode<T> adj_node(const Dev<T>& d, const AQuad<T>& Q, int k, bool valid) {
+    ANode<T> N;
+    N.valid = valid;
+    N.k = valid ? k : 0;
+    N.kind = valid ? d.kind[N.k] : (int8_t)HLBM_NODE_INTERIOR;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) lam[i] = lnext[9 * (int64_t)P + i];
-    if (kind == HLBM_NODE_OUTER) {
+    for (int j = 0; j < 6; ++j) N.s0[j] = N.s1[j] = T(0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) N.g0[j] = N.g1[j] = T(0);
+    if (N.kind == HLBM_NODE_OUTER) {
         const int64_t no = d.n_outer;
-        const int o = d.outer_of[P];
-        const T th = T(m + 1) / T(d.n_sub);
-        T st[12], ls[12];
+        const T* p = d.snap + d.outer_of[N.k];
+        const int at[6] = {0, 1, 2, 4 + Q.ia, 4 + Q.ib, 3};
 #pragma unroll
-        for (int j = 0; j < 12; ++j) st[j] = (T(1) - th) * T(d.snap[j * no + o]) + th * T(d.snap[(12 + j) * no + o]);
-        ffsT(st, T(d.rho0), T(d.kneq), lam, ls, l_kneq);
-#pragma unroll
-        for (int j = 0; j < 12; ++j) {
-            lsnap[j * no + o] += (T(1) - th) * ls[j];
-            lsnap[(12 + j) * no + o] += th * ls[j];
+        for (int j = 0; j < 6; ++j) {
+            N.s0[j] = p[at[j] * no];
+            N.s1[j] = p[(12 + at[j]) * no];
         }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) ps[i] = T(0);
-    } else {
-        T fv[9], cneq[9];
-        fv_update_d(d, in, P, fv, cneq);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) ps[i] = lam[i];
-        if (kind == HLBM_NODE_WALL) {
-            // g(f) = f + f^eq(rho, U) - f^eq(rho, u(f))
-            T U, V;
-            wall_velocity(d, a, m, U, V);
-            T dr, rho, ux, uy;
-            mom_d(fv, T(d.rho0), dr, rho, ux, uy);
-            T aU = T(0);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                T A, Bx, By;
-                feq_ab(i, rho, U, V, A, Bx, By);
-                aU += lam[i] * A;
-                l_v += lam[i] * By;
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) ps[i] += aU;
-            jfeqT_add(rho, ux, uy, lam, T(-1), ps);
-        }
-        const T dt = T(d.dt_u);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) l_inv -= dt * ps[i] * cneq[i];
     }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) psi[9 * (int64_t)P + i] = ps[i];
+    return N;
+}
+// the outer node's sums into the feed adjoint
+template <typename T>
+__device__ __forceinline__ void adj_node_out(const Dev<T>& d, const AQuad<T>& Q, const ANode<T>& N, T* lsnap) {
+    if (N.kind != HLBM_NODE_OUTER) return;
+    const int64_t no = d.n_outer;
+    T* p = lsnap + d.outer_of[N.k];
+    auto put = [&](int j, T v0, T v1) {
+        p[j * no] += v0;
+        p[(12 + j) * no] += v1;
+    };
+    put(4 + Q.ia, N.g0[0], N.g1[0]);
+    put(4 + Q.ib, N.g0[1], N.g1[1]);
+    if (Q.q == 0) put(3, N.g0[2], N.g1[2]);
+    if (Q.q < 3) put(Q.q, N.g0[3], N.g1[3]);
+}
+template <typename T>
+__device__ __forceinline__ ARec<T> adj_rec(const Dev<T>& d, const AQuad<T>& Q, const ANode<T>& N, const T* rec, int m) {
+    const T* r = rec + ((int64_t)m * d.n + N.k) * kAdjRec;
+    ARec<T> v;
+    const bool row = N.kind != HLBM_NODE_OUTER, wall = N.kind == HLBM_NODE_WALL;
+    v.na = row ? r[Q.ia] : T(0);
+    v.nb = row ? r[Q.ib] : T(0);
+    v.n0 = row && Q.q == 0 ? r[kAdjN0] : T(0);
+    v.rho = wall ? r[kAdjWall] : T(1);
+    v.wx = wall ? r[kAdjWall + 1] : T(0);
+    v.wy = wall ? r[kAdjWall + 2] : T(0);
+    return v;
 }
 
-// Reverse of sub-step m, second pass at node k: the adjoint of its state
-// before the sub-step, gathered from the rows that read it (k itself and its
-// neighbours; tpos gives row P's entry of column k).
+// psi at the quad's node for a sub-step (time fraction th, wall velocity U, V,
+// record r) from the adjoint (la, lb, l0) of the state after it, the outer
+// nodes' feed adjoint, and the parameter terms (1/tau_u, kneq, wall velocity)
 template <typename T>
-__device__ __forceinline__ void adj_gather_node(const Dev<T>& d, const T* in, const T* psi, const int32_t* tpos,
-                                                T* lcur, int k) {
-    const T dt = T(d.dt_u), inv = T(d.inv_tau_u);
-    T out[9], Lc[9];
-    const bool regular = d.kind[k] != HLBM_NODE_OUTER;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        out[i] = regular ? psi[9 * (int64_t)k + i] : T(0);
-        Lc[i] = T(0);
+__device__ __forceinline__ void adj_psi(const Dev<T>& d, const AQuad<T>& Q, ANode<T>& N, const ARec<T>& r, T th, T U, T V,
+                                        T la, T lb, T l0, T& pa, T& pb, T& p0, T& l_inv, double& l_kneq, T& l_v) {
+    pa = la, pb = lb, p0 = l0;
+    const bool wall = N.kind == HLBM_NODE_WALL, outer = N.kind == HLBM_NODE_OUTER;
+    if (__any_sync(0xffffffffu, wall)) {
+        // g(f) = f + f^eq(rho, U) - f^eq(rho, u(f))
+        T a1, bx1, by1, a2, bx2, by2;
+        aq_feq(Q, U, V, la, lb, l0, a1, bx1, by1);
+        aq_feq(Q, r.wx, r.wy, la, lb, l0, a2, bx2, by2);
+        if (wall) {
+            const T g = a1 - a2 + bx2 * r.wx + by2 * r.wy, c = aq_dot(Q, bx2, by2);
+            pa += g - c;
+            pb += g + c;
+            p0 += g;
+            if (Q.q == 0) l_v += r.rho * by1;
+        }
     }
-    const int r0 = d.row_ptr[k], r1 = d.row_ptr[k + 1];
-    for (int e = r0; e < r1; ++e) {
-        const int P = e == r0 ? k : d.coef[e].col;
-        if (d.kind[P] == HLBM_NODE_OUTER) continue;
-        T gx, gy, cc;
-        if (P == k) {
-            gx = gy = T(0);
-            for (int q = r0 + 1; q < r1; ++q) {
-                gx -= d.coef[q].gx;
-                gy -= d.coef[q].gy;
+    if (__any_sync(0xffffffffu, outer)) {
+        const T t0 = T(1) - th;
+        T st[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) st[j] = t0 * N.s0[j] + th * N.s1[j];
+        T a, bx, by;
+        aq_feq(Q, st[1], st[2], la, lb, l0, a, bx, by);
+        if (outer) {
+            const T rho = d.rho0 + st[0];
+            const T v[4] = {d.kneq * la, d.kneq * lb, d.kneq * l0, Q.q == 0 ? a : rho * (Q.q == 1 ? bx : by)};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                N.g0[j] += t0 * v[j];
+                N.g1[j] += th * v[j];
             }
-            cc = d.coef[r0].c;
-        } else {
-            const Coef<T> c = d.coef[tpos[e]];
-            gx = c.gx;
-            gy = c.gy;
-            cc = c.c;
-        }
-        const T* pp = psi + 9 * (int64_t)P;
-#pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            out[j] += dt * ((T(cx_of(j)) * gx + T(cy_of(j)) * gy) - inv * cc) * pp[j];
-            Lc[j] += cc * pp[j];
+            l_kneq += double(la * st[3] + lb * st[4] + (Q.q == 0 ? l0 * st[5] : T(0)));
+            pa = pb = p0 = T(0);
         }
     }
-    T f[9], dr, rho, ux, uy;
-    load_d(in + (int64_t)kRec * k, f);
-    mom_d(f, T(d.rho0), dr, rho, ux, uy);
-    jfeqT_add(rho, ux, uy, Lc, dt * inv, out);
-#pragma unroll
-    for (int j = 0; j < 9; ++j) lcur[9 * (int64_t)k + j] = out[j];
+    if (!N.valid) return;
+    l_inv -= d.dt_u * (pa * r.na + pb * r.nb + (Q.q == 0 ? p0 * r.n0 : T(0)));
+}
+template <typename T>
+__device__ __forceinline__ void adj_put(const AQuad<T>& Q, const ANode<T>& N, T* psi, T pa, T pb, T p0) {
+    if (!N.valid) return;
+    T* o = psi + kAdjPsi * (int64_t)N.k;
+    o[Q.ia] = pa;
+    o[Q.ib] = pb;
+    if (Q.q == 0) o[kAdjN0] = p0;
 }
 
-// The FV part of one step's reverse in one cooperative launch: the n
-// sub-steps forward again from sub[0] (every state kept in sub), then their
-// reverse from lPn (the adjoint of the patch after them) to lPm (before
-// them), with grid-wide barriers between the passes.  Every thread runs the
-// same number of node iterations, so the warp sums stay convergent.
+// psi as packets (see k_fv_deep): one per lane of the quad in FP32 (its pair,
+// f0 and the tag), three in FP64 (a value each; the third on lane 0 only)
 template <typename T>
-__global__ void __launch_bounds__(128) k_adj_fv_all(Dev<T> d, StepArgs a, T* sub, const T* lPn, T* x0, T* x1,
-                                                    T* psi, const int32_t* tpos, T* lsnap, double* par, double* lV,
-                                                    T* lPm) {
+constexpr int kAdjPkts = sizeof(T) == 4 ? 1 : 3;
+__device__ __forceinline__ void adj_send(unsigned char* p, int, float a, float b, float c, unsigned tag) {
+    auto w = [](float v) { return (unsigned long long)__float_as_uint(v); };
+    st_packet(p, w(a) | (w(b) << 32), w(c) | ((unsigned long long)tag << 32));
+}
+__device__ __forceinline__ void adj_send(unsigned char* p, int q, double a, double b, double c, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    st_packet(p, (unsigned long long)__double_as_longlong(a), t);
+    st_packet(p + 16, (unsigned long long)__double_as_longlong(b), t);
+    if (q == 0) st_packet(p + 32, (unsigned long long)__double_as_longlong(c), t);
+}
+__device__ __forceinline__ bool adj_recv(const unsigned char* p, int, float& a, float& b, float& c, unsigned tag) {
+    const Packet k = ld_packet(p);
+    a = __uint_as_float((unsigned)k.lo);
+    b = __uint_as_float((unsigned)(k.lo >> 32));
+    c = __uint_as_float((unsigned)k.hi);
+    return packet_tag(k) == tag;
+}
+__device__ __forceinline__ bool adj_recv(const unsigned char* p, int q, double& a, double& b, double& c, unsigned tag) {
+    const Packet k = ld_packet(p), l = ld_packet(p + 16);
+    a = __longlong_as_double((long long)k.lo);
+    b = __longlong_as_double((long long)l.lo);
+    bool ok = packet_tag(k) == tag && packet_tag(l) == tag;
+    c = 0.0;
+    if (q == 0) {
+        const Packet e = ld_packet(p + 32);
+        c = __longlong_as_double((long long)e.lo);
+        ok = ok && packet_tag(e) == tag;
+    }
+    return ok;
+}
+
+// kEntries > 0: every quad has at most one node, of at most that many row
+// entries, and keeps them, its outer state and its sums in registers over the
+// sub-steps; psi travels as tagged packets from node to node, without a
+// barrier.  A node overwrites its packets of sub-step m at sub-step m - 2,
+// after receiving psi of sub-step m - 1 from every node that reads its own (the
+// rows are symmetric), each of which read the packets of sub-step m before
+// sending it.  Quads take the nodes in `order` (by kind), so that a warp runs
+// the wall rule or the outer rule only where its nodes need it.  Tags (tag0 + the sub-step's distance from the last) grow over
+// the solver's life.  0: any patch, with grid barriers.
+template <typename T, int kEntries>
+__global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const T* rec, const T* P0, const T* lPn, T* x0,
+                                                    T* x1, const Coef<T>* tco, T* lsnap, double* par, double* lV,
+                                                    T* lPm, int use_tab, unsigned char* px, unsigned tag0,
+                                                    const int32_t* order) {
     namespace cg = cooperative_groups;
     cg::grid_group grid = cg::this_grid();
     const int n = d.n, ns = d.n_sub;
-    const int nth = gridDim.x * blockDim.x, gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t rec = (int64_t)kRec * n;
-    for (int m = 0; m < ns; ++m) {
-        T U, V;
-        wall_velocity(d, a, m, U, V);
-        for (int P = gtid; P < n; P += nth) fv_node(d, sub + m * rec, sub + (m + 1) * rec, P, m, U, V);
-        grid.sync();
+    const AQuad<T> Q = aquad<T>();
+    const int nq = gridDim.x * blockDim.x / 4, gq = (blockIdx.x * blockDim.x + threadIdx.x) / 4;
+    // time fraction and wall velocity of every sub-step (an FP64 cosine and
+    // divisions each), when they fit
+    extern __shared__ __align__(16) unsigned char sm[];
+    T* tab = reinterpret_cast<T*>(sm);
+    for (int m = threadIdx.x; m < ns && use_tab; m += blockDim.x) {
+        tab[3 * m] = T(m + 1) / T(ns);
+        wall_velocity(d, a, m, tab[3 * m + 1], tab[3 * m + 2]);
     }
-    T l_inv = T(0);
-    double l_kneq = 0.0;
-    const T* lnext = lPn;
-    for (int m = ns - 1; m >= 0; --m) {
-        const T* in = sub + m * rec;
-        T l_v = T(0);
-        for (int base = 0; base < n; base += nth) {
-            const int P = base + gtid;
-            if (P < n) adj_psi_node(d, a, in, m, lnext, psi, lsnap, P, l_inv, l_kneq, l_v);
+    __syncthreads();
+    auto at_substep = [&](int m, T& th, T& U, T& V) {
+        if (use_tab) {
+            th = tab[3 * m], U = tab[3 * m + 1], V = tab[3 * m + 2];
+        } else {
+            th = T(m + 1) / T(ns);
+            wall_velocity(d, a, m, U, V);
         }
-        warp_atomic_add(lV + (int64_t)a.t * ns + m, double(l_v));
-        grid.sync();
-        T* lcur = (m & 1) ? x1 : x0;
-        for (int k = gtid; k < n; k += nth) adj_gather_node(d, in, psi, tpos, lcur, k);
-        grid.sync();
-        lnext = lcur;
+    };
+    // velocity of node k's state before sub-step m
+    auto velocity = [&](int k, int m, T& ux, T& uy) {
+        if (m > 0) {
+            const T* r = rec + ((int64_t)m * n + k) * kAdjRec + kAdjU;
+            ux = r[0];
+            uy = r[1];
+        } else {
+            T f[9], dr, rho;
+            load_d(P0 + (int64_t)kRec * k, f);
+            mom_d(f, T(d.rho0), dr, rho, ux, uy);
+        }
+    };
+    // the adjoint of state m at the node from the row sums
+    const T dt = d.dt_u, di = d.dt_u * d.inv_tau_u;
+    auto close = [&](T pa, T pb, T p0, T ux, T uy, T Sa, T Sb, T La, T Lb, T L0, T& la, T& lb, T& l0) {
+        T fa, fx, fy;
+        aq_feq(Q, ux, uy, La, Lb, L0, fa, fx, fy);
+        const T g = fa - fx * ux - fy * uy, c = aq_dot(Q, fx, fy);
+        la = pa + dt * Q.sgn * Sa - di * La + di * (g + c);
+        lb = pb - dt * Q.sgn * Sb - di * Lb + di * (g - c);
+        l0 = Q.q == 0 ? p0 - di * L0 + di * g : T(0);
+    };
+    auto put_out = [&](int k, T la, T lb, T l0) {
+        T* o = lPm + 9 * (int64_t)k;
+        o[1 + Q.ia] = la;
+        o[1 + Q.ib] = lb;
+        if (Q.q == 0) o[0] = l0;
+    };
+    T l_inv = T(0), th, U, V;
+    double l_kneq = 0.0;
+    auto add_v = [&](int m, T l_v) {
+        if (__any_sync(0xffffffffu, l_v != T(0))) warp_atomic_add(lV + (int64_t)a.t * ns + m, double(l_v));
+    };
+    if constexpr (kEntries > 0) {
+        constexpr int E = kEntries;
+        ANode<T> N = adj_node(d, Q, gq < n ? order[gq] : 0, gq < n);
+        T eg[E], ec[E];
+        int ecol[E];
+        const int r0 = d.row_ptr[N.k], r1 = d.row_ptr[N.k + 1];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const bool have = r0 + e < r1;
+            const Coef<T> c = tco[have ? r0 + e : r0];
+            eg[e] = have ? aq_dot(Q, Q.sgn * c.gx, Q.sgn * c.gy) : T(0);  // lane 3: gx - gy
+            ec[e] = have ? c.c : T(0);
+            ecol[e] = have ? c.col : N.k;
+        }
+        // the packets of node g for the sub-step i steps from the last
+        auto at = [&](int g, int i) {
+            return px + (((int64_t)(i & 1) * n + g) * 4 + Q.q) * (kAdjPkts<T> * 16);
+        };
+        ARec<T> r = adj_rec(d, Q, N, rec, ns - 1);
+        T pa, pb, p0;
+        {
+            T l_v = T(0);
+            at_substep(ns - 1, th, U, V);
+            const T* l = lPn + 9 * (int64_t)N.k;
+            adj_psi(d, Q, N, r, th, U, V, l[1 + Q.ia], l[1 + Q.ib], Q.q == 0 ? l[0] : T(0), pa, pb, p0, l_inv, l_kneq, l_v);
+            if (N.valid) adj_send(at(N.k, 0), Q.q, pa, pb, p0, tag0);
+            add_v(ns - 1, l_v);
+        }
+        bool ok = true;
+        for (int m = ns - 1; m >= 0 && ok; --m) {
+            const int i = ns - 1 - m;
+            T ux, uy, l_v = T(0);
+            velocity(N.k, m, ux, uy);
+            if (m > 0) {
+                r = adj_rec(d, Q, N, rec, m - 1);
+                at_substep(m - 1, th, U, V);
+            }
+            T fa[E], fb[E], f0[E], Sa = T(0), Sb = T(0), La = T(0), Lb = T(0), L0 = T(0), la, lb, l0;
+            for (long spins = 0; ok; ++spins) {
+                bool have = true;
+#pragma unroll
+                for (int e = 0; e < E; ++e) have = adj_recv(at(ecol[e], i), Q.q, fa[e], fb[e], f0[e], tag0 + i) && have;
+                if (__all_sync(0xffffffffu, have || !N.valid)) break;
+                if ((spins & 63) == 63) ok = !*(volatile unsigned*)d.abort_flag;
+                if (spins > d.spin_limit) {
+                    atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
+                    atomicExch(d.abort_flag, 1u);
+                    ok = false;
+                }
+                ok = __all_sync(0xffffffffu, ok);
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                Sa += eg[e] * fa[e];
+                Sb += eg[e] * fb[e];
+                La += ec[e] * fa[e];
+                Lb += ec[e] * fb[e];
+                L0 += ec[e] * f0[e];
+            }
+            close(pa, pb, p0, ux, uy, Sa, Sb, La, Lb, L0, la, lb, l0);
+            if (m > 0) {
+                adj_psi(d, Q, N, r, th, U, V, la, lb, l0, pa, pb, p0, l_inv, l_kneq, l_v);
+                if (N.valid && ok) adj_send(at(N.k, i + 1), Q.q, pa, pb, p0, tag0 + i + 1);
+                add_v(m - 1, l_v);
+            } else if (N.valid) {
+                put_out(N.k, la, lb, l0);
+            }
+        }
+        adj_node_out(d, Q, N, lsnap);
+    } else {
+        T l_v = T(0);
+        at_substep(ns - 1, th, U, V);
+        for (int base = 0; base < n; base += nq) {  // the same number of turns on every thread
+            ANode<T> N = adj_node(d, Q, base + gq, base + gq < n);
+            const T* l = lPn + 9 * (int64_t)N.k;
+            T pa, pb, p0;
+            adj_psi(d, Q, N, adj_rec(d, Q, N, rec, ns - 1), th, U, V, l[1 + Q.ia], l[1 + Q.ib], Q.q == 0 ? l[0] : T(0), pa,
+                    pb, p0, l_inv, l_kneq, l_v);
+            adj_put(Q, N, x0, pa, pb, p0);
+            adj_node_out(d, Q, N, lsnap);
+        }
+        add_v(ns - 1, l_v);
+        for (int m = ns - 1; m >= 0; --m) {
+            const T* psi = ((ns - 1 - m) & 1) ? x1 : x0;
+            T* nxt = ((ns - 1 - m) & 1) ? x0 : x1;
+            l_v = T(0);
+            if (m > 0) at_substep(m - 1, th, U, V);
+            grid.sync();
+            for (int base = 0; base < n; base += nq) {
+                ANode<T> N = adj_node(d, Q, base + gq, base + gq < n);
+                T Sa = T(0), Sb = T(0), La = T(0), Lb = T(0), L0 = T(0), la, lb, l0, ux, uy;
+                const int r0 = d.row_ptr[N.k], r1 = N.valid ? d.row_ptr[N.k + 1] : r0;
+#pragma unroll 2
+                for (int e = r0; e < r1; ++e) {
+                    const Coef<T> c = tco[e];
+                    const T* p = psi + kAdjPsi * (int64_t)c.col;
+                    const T g = aq_dot(Q, Q.sgn * c.gx, Q.sgn * c.gy);
+                    const T pa = p[Q.ia], pb = p[Q.ib];
+                    Sa += g * pa;
+                    Sb += g * pb;
+                    La += c.c * pa;
+                    Lb += c.c * pb;
+                    L0 += c.c * p[kAdjN0];
+                }
+                __syncwarp();
+                velocity(N.k, m, ux, uy);
+                const T* p = psi + kAdjPsi * (int64_t)N.k;
+                close(p[Q.ia], p[Q.ib], p[kAdjN0], ux, uy, Sa, Sb, La, Lb, L0, la, lb, l0);
+                if (m > 0) {
+                    T pa, pb, p0;
+                    adj_psi(d, Q, N, adj_rec(d, Q, N, rec, m - 1), th, U, V, la, lb, l0, pa, pb, p0, l_inv, l_kneq, l_v);
+                    adj_put(Q, N, nxt, pa, pb, p0);
+                    adj_node_out(d, Q, N, lsnap);
+                } else if (N.valid) {
+                    put_out(N.k, la, lb, l0);
+                }
+            }
+            if (m > 0) add_v(m - 1, l_v);
+        }
     }
-    for (int64_t i = gtid; i < 9 * (int64_t)n; i += nth) lPm[i] = lnext[i];
     warp_atomic_add(par + 1, double(l_inv));
     warp_atomic_add(par + 3, l_kneq);
+}
+
+// The transposed rows: entry e of row k (pivot first) holds g and C of row
+// col's entry of column k; the pivot's g is minus the sum of the row's own.
+template <typename T>
+__global__ void k_adj_rows(Dev<T> d, const int32_t* tpos, Coef<T>* tco) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= d.n) return;
+    const int r0 = d.row_ptr[k], r1 = d.row_ptr[k + 1];
+    Coef<T> pv = d.coef[r0];
+    pv.gx = pv.gy = T(0);
+    for (int e = r0 + 1; e < r1; ++e) {
+        pv.gx -= d.coef[e].gx;
+        pv.gy -= d.coef[e].gy;
+        Coef<T> c = d.coef[tpos[e]];
+        c.col = d.coef[e].col;
+        tco[e] = c;
+    }
+    pv.col = k;
+    tco[r0] = pv;
+}
+
+// The FV sub-steps of a step from patch state P0 with their records, in
+// global memory with grid barriers: for the patches and kernels whose forward
+// step does not record.
+template <typename T>
+__global__ void __launch_bounds__(128) k_adj_fv_record(Dev<T> d, StepArgs a, const T* P0, T* b0, T* b1) {
+    namespace cg = cooperative_groups;
+    cg::grid_group grid = cg::this_grid();
+    const int nth = gridDim.x * blockDim.x, gtid = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int m = 0; m < d.n_sub; ++m) {
+        const T* in = m == 0 ? P0 : ((m & 1) ? b1 : b0);
+        T* out = (m & 1) ? b0 : b1;
+        T U, V;
+        wall_velocity(d, a, m, U, V);
+        for (int P = gtid; P < d.n; P += nth) {
+            const int8_t kind = d.kind[P];
+            Pops<T> fn, nq{};
+            T mo[3] = {};
+            if (kind == HLBM_NODE_OUTER) {
+                fn = fv_outer_from(d, d.snap + d.outer_of[P], (int64_t)d.n_outer, m);
+            } else {
+                auto get = [&](int g) {
+                    const T* r = in + (int64_t)kRec * g;
+                    return RecP<T>{pk(r[1], r[2]), pk(r[3], r[4]), pk(r[5], r[6]),
+                                   pk(r[7], r[8]), pk(r[0], r[9]), pk(r[10], r[11])};
+                };
+                const RecP<T> own = get(P);
+                const Pops<T> Q{own.A, own.B, own.C, own.D, px(own.E)};
+                FvSums<T> acc;
+                fv_sums_init(acc);
+                const int r0 = d.row_ptr[P], r1 = d.row_ptr[P + 1];
+                for (int e = r0 + 1; e < r1; ++e) {
+                    const Coef<T> c = d.coef[e];
+                    fv_sums_entry(acc, c.gx, c.gy, c.c, get(c.col), Q);
+                }
+                fn = fv_sums_finish(d, acc, d.coef[r0].c, own, nq);
+                if (kind == HLBM_NODE_WALL) fv_wall(d, U, V, fn, mo);
+            }
+            T z[3], ux, uy;
+            z_of(fn, d.rho0, z, ux, uy);
+            adj_record(d, m, P, kind != HLBM_NODE_OUTER, nq, kind == HLBM_NODE_WALL, mo, ux, uy);
+            T f[9];
+            pops_to(fn, f);
+            T* r = out + (int64_t)kRec * P;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) r[i] = f[i];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) r[9 + j] = z[j];
+        }
+        grid.sync();
+    }
 }
 
 // Reverse of the outer nodes' feed: snap[0] bilinear from the window state
@@ -2692,7 +3044,7 @@ __global__ void k_adj_feed(Dev<T> d, StepArgs a, const T* lsnap, T* lSo, T* lSn,
                     out[i] = 0.0;
                 }
                 state_d(f, T(d.rho0), st);
-                stateT_add(f, T(d.rho0), ls, T(w), out);
+                stateT_add(st, T(d.rho0), ls, T(w), out);
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
                     if (out[i] != 0.0) atomicAdd(lS + i * d.bplane + b, out[i]);
@@ -2758,14 +3110,15 @@ __global__ void k_adj_stream(Dev<T> d, StepArgs a, const T* lfB, const T* lSn, T
         mom_d(f, T(d.rho0), dr, rho, ux, uy);
         const T om = 1.0 / T(d.tau_s);
         const int64_t s = (int64_t)y * d.pitch + x;
-        T lam[9], mu[9];
+        T lam[9], mu[9], eq[9];
+        feq_all(dr, rho, ux, uy, eq);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             lam[i] = lfB[i * d.plane + s];
-            mu[i] = (1.0 - om) * lam[i];
-            l_om -= lam[i] * (f[i] - feq_d(i, dr, rho, ux, uy));
+            mu[i] = (T(1) - om) * lam[i];
+            l_om -= lam[i] * (f[i] - eq[i]);
         }
-        jfeqT_add(rho, ux, uy, lam, om, mu);
+        jfeqT_add(ux, uy, lam, om, mu);
         if (b >= 0) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) mu[i] += lSn[i * d.bplane + b];
@@ -2828,7 +3181,7 @@ __global__ void k_adj_fill(Dev<T> d, StepArgs a, T* lfA, T* lP, double* par, dou
                 T out[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) out[i] = 0.0;
-                stateT_add(fv[q], rho0, ls, T(lam[q]), out);
+                stateT_add(sv[q], rho0, ls, T(lam[q]), out);
                 atomic_add9(lP + 9 * (int64_t)d.tri[3 * k + q], out);
                 T dot = 0.0;
 #pragma unroll
@@ -2901,7 +3254,7 @@ __global__ void k_adj_refill(Dev<T> d, StepArgs a, const T* lPm, T* lP0, T* lSo,
                 T out[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) out[i] = 0.0;
-                stateT_add(fq[q], rho0, ls, T(wq[q]), out);
+                stateT_add(sq[q], rho0, ls, T(wq[q]), out);
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
                     if (out[i] != 0.0) atomicAdd(lSo + i * d.bplane + bq[q], out[i]);
@@ -2921,18 +3274,46 @@ template <typename T>
 void launch_adj_force(const Dev<T>& d, double lamF, T* lP, cudaStream_t s) {
     if (d.nseg > 0) k_adj_force<T><<<(d.nseg + 127) / 128, 128, 0, s>>>(d, lamF, lP);
 }
+size_t adj_packet_bytes(int n) { return (size_t)2 * n * 4 * 3 * 16; }
+size_t adj_record_values(int n, int n_sub) { return (size_t)n_sub * n * kAdjRec; }
 template <typename T>
-cudaError_t launch_adj_fv(const Dev<T>& d, const StepArgs& a, T* sub, const T* lPn, T* x0, T* x1, T* psi,
-                          const int32_t* tpos, T* lsnap, double* par, double* lV, T* lPm, cudaStream_t s) {
+void launch_adj_rows(const Dev<T>& d, const int32_t* tpos, Coef<T>* tco, cudaStream_t s) {
+    k_adj_rows<T><<<(d.n + 127) / 128, 128, 0, s>>>(d, tpos, tco);
+}
+// as many blocks of `block` threads as `threads` needs, all resident
+static int resident_blocks(const void* fn, int64_t threads, size_t smem = 0, int block = 128) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, (const void*)k_adj_fv_all<T>, 128, 0);
-    const int blocks = std::max(1, std::min((d.n + 127) / 128, std::max(per, 1) * sms));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, block, smem);
+    return (int)std::max<int64_t>(1, std::min<int64_t>((threads + block - 1) / block, (int64_t)std::max(per, 1) * sms));
+}
+template <typename T>
+cudaError_t launch_adj_fv_record(const Dev<T>& d, const StepArgs& a, const T* P0, T* b0, T* b1, cudaStream_t s) {
+    const void* fn = (const void*)k_adj_fv_record<T>;
     Dev<T> dd = d;
     StepArgs aa = a;
-    void* args[] = {&dd, &aa, &sub, &lPn, &x0, &x1, &psi, &tpos, &lsnap, &par, &lV, &lPm};
-    return cudaLaunchCooperativeKernel((const void*)k_adj_fv_all<T>, dim3(blocks), dim3(128), args, 0, s);
+    void* args[] = {&dd, &aa, &P0, &b0, &b1};
+    return cudaLaunchCooperativeKernel(fn, dim3(resident_blocks(fn, d.n)), dim3(128), args, 0, s);
+}
+template <typename T>
+cudaError_t launch_adj_fv(const Dev<T>& d, const StepArgs& a, const T* rec, const T* P0, const T* lPn, T* x0, T* x1,
+                          const Coef<T>* tco, T* lsnap, double* par, double* lV, T* lPm, int max_row,
+                          unsigned char* px, unsigned tag0, const int32_t* order,
+                          cudaStream_t s) {
+    // one node per quad over resident blocks (at most 7 off-diagonal entries), else any
+    const void* fn = (const void*)k_adj_fv_rev<T, kTmemMaxEntries + 1>;
+    // FP64: three warps issue at the full rate of a warp on its own, four do not
+    const int block = sizeof(T) == 8 ? 96 : 128;
+    const size_t tab = 3 * (size_t)d.n_sub * sizeof(T), smem = tab <= 48 * 1024 ? tab : 0;
+    if (max_row > kTmemMaxEntries + 1 || (int64_t)resident_blocks(fn, 4 * (int64_t)d.n, smem, block) * (block / 4) < d.n)
+        fn = (const void*)k_adj_fv_rev<T, 0>;
+    int use_tab = smem > 0;
+    Dev<T> dd = d;
+    StepArgs aa = a;
+    void* args[] = {&dd, &aa, &rec, &P0, &lPn, &x0, &x1, &tco, &lsnap, &par, &lV, &lPm, &use_tab, &px, &tag0, &order};
+    return cudaLaunchCooperativeKernel(fn, dim3(resident_blocks(fn, 4 * (int64_t)d.n, smem, block)), dim3(block), args, smem,
+                                       s);
 }
 template <typename T>
 void launch_adj_feed(const Dev<T>& d, const StepArgs& a, const T* lsnap, T* lSo, T* lSn, double* lY,
@@ -2984,8 +3365,11 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template void launch_force<T>(const Dev<T>&, int64_t, cudaStream_t);                                      \
     template void launch_patch_macro<T>(const Dev<T>&, double*, double*, double*, double*, cudaStream_t);    \
     template void launch_adj_force<T>(const Dev<T>&, double, T*, cudaStream_t);                               \
-    template cudaError_t launch_adj_fv<T>(const Dev<T>&, const StepArgs&, T*, const T*, T*, T*, T*,            \
-                                          const int32_t*, T*, double*, double*, T*, cudaStream_t);            \
+    template void launch_adj_rows<T>(const Dev<T>&, const int32_t*, Coef<T>*, cudaStream_t);                  \
+    template cudaError_t launch_adj_fv_record<T>(const Dev<T>&, const StepArgs&, const T*, T*, T*, cudaStream_t); \
+    template cudaError_t launch_adj_fv<T>(const Dev<T>&, const StepArgs&, const T*, const T*, const T*, T*, T*, \
+                                          const Coef<T>*, T*, double*, double*, T*, int, unsigned char*, unsigned,             \
+                                          const int32_t*, cudaStream_t);                                      \
     template void launch_adj_feed<T>(const Dev<T>&, const StepArgs&, const T*, T*, T*, double*, cudaStream_t); \
     template void launch_adj_stream<T>(const Dev<T>&, const StepArgs&, const T*, const T*, T*, double*,        \
                                        cudaStream_t);                                                         \

@@ -1,0 +1,76 @@
+"""Paths of the FV kernels chosen by size, precision and patch, at the sizes
+where they can go wrong, against the oracle or against the general path."""
+import numpy as np
+import pytest
+
+import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2006_13631_gb300.build import build
+
+    build()
+
+
+def _case(dtype, mesh_args, n_sub=24, L=20.0, n=128):
+    A, om, tau = inputs.harmonic_params(L, 0.5, 100.0)
+    w = inputs.Workload("paths", n, n - 12, L, L / 50.0, 0.5 * n + 0.3, 0.5 * n - 5.8, tau, n_sub,
+                        inputs.MOTION_HARMONIC, A=A, omega=om, dtype=dtype, noise_amp=1e-6, seed=3, mesh_args=mesh_args)
+    w.n_sub = inputs.stable_substeps(w.mesh(), tau - 0.5, minimum=n_sub)
+    return w
+
+
+SMALL = dict(n_L=17, n_T=2, n_layers=9, h1=0.3, d_out=4.0)
+MEDIUM = dict(n_L=110, n_T=2, n_layers=20, h1=0.15, d_out=4.0)
+LARGE = dict(n_L=200, n_T=4, n_layers=45, h1=0.08, d_out=4.0)
+
+
+@pytest.mark.parametrize("dtype,tol", [("f64", 1e-9), ("f32", 2e-3)])
+@pytest.mark.parametrize("mesh_args", [SMALL, MEDIUM], ids=["small", "medium"])
+def test_adjoint_from_recorded_and_rerecorded_substeps(mesh_args, dtype, tol):
+    """The adjoint whose forward steps record the FV sub-steps (deep tiles) and the
+    one that records them again in global memory (global-memory kernel): the same
+    gradient up to the order of the atomic sums (FP64: 1e-16 per term over 1e6
+    terms, cancelling; FP32: 1e-7 likewise)."""
+    from paper_2006_13631_gb300 import hlbm as H
+
+    H.use_torch_allocator()
+    w = _case(dtype, mesh_args)
+    got = []
+    for kern in (0, 1):
+        w.fv_kernel = kern
+        grid, patch, motion = H.workload_inputs(w)
+        got.append(H.hlbm_theta_adjoint(grid, patch, w.tau_s, motion, 9, 0.0, 8.5 / w.period, 1.0, 0.5, 4))
+    (t0, g0, _, _), (t1, g1, _, _) = got
+    assert t0 == t1
+    assert np.abs(g0 - g1).max() <= tol * np.abs(g1).max()
+
+
+def test_adjoint_of_a_patch_of_more_nodes_than_resident_quads():
+    """The reverse pass that strides over the nodes with grid barriers, against
+    central differences of the CUDA path in tau_s (no node moves; FP64, the
+    quotient's error is the square of the 1e-5 step and 1e-13 / 1e-5)."""
+    from paper_2006_13631_gb300 import hlbm as H
+
+    H.use_torch_allocator()
+    w = _case("f64", LARGE)
+    assert w.mesh().n_nodes > 152 * 4 * 24
+    mesh, rho = w.mesh(), w.rho_init()
+    steps, fit = 6, 5.5 / w.period
+    grid, patch, motion = H.workload_inputs(w, mesh, rho)
+    _, g, _, _ = H.hlbm_theta_adjoint(grid, patch, w.tau_s, motion, steps, 0.0, fit, 1.0, 0.5, 3)
+    L = []
+    for sign in (-1.0, 1.0):
+        h = H.hlbm_create(grid, patch, w.tau_s * (1.0 + sign * 1e-5), motion, 0)
+        H.hlbm_step(h, steps)
+        re, im, _ = H.hlbm_gamma_window(h, w.omega, 0.0, fit)
+        L.append(re + 0.5 * im)
+        H.hlbm_destroy(h)
+    quotient = (L[1] - L[0]) / (2e-5 * w.tau_s)
+    assert abs(g[2] - quotient) <= 1e-5 * abs(quotient)
