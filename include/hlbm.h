@@ -152,8 +152,9 @@ typedef struct {
  * truncated control volume, with the starred values of the paper
  * (interpolated at interpolation nodes, the patch state elsewhere).
  * fv_kernel picks the kernel of the FV sub-steps, HLBM_FV_*: AUTO takes the
- * first that applies of DEEP and TMEM (rows of at most 7 off-diagonal
- * entries, outer_fv = 0), SMEM and GLOBAL; the others are for testing and
+ * first that applies of DEEP (rows of at most 7 off-diagonal entries), TMEM
+ * (such rows, outer_fv = 0), SMEM and GLOBAL; the others are for testing
+ * (DEEP and TMEM with outer_fv = 0) and
  * hlbm_create fails with HLBM_EINVAL when the one asked for cannot run the
  * patch.  All give the same results bit for bit. */
 typedef struct {

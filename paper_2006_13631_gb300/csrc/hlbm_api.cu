@@ -541,7 +541,7 @@ int step_fv(hlbm* h, cudaStream_t s, PendingStep& ps, cudaEvent_t ev0 = nullptr,
 template <typename T>
 void step_fv_packed_done(hlbm* h) {
     Dev<T>& d = dev_of<T>(h);
-    if (d.n_sub & 1) h->ui = 1 - h->ui;
+    if (h->fv_kind == HLBM_FV_DEEP || (d.n_sub & 1)) h->ui = 1 - h->ui;
     bind(h, d);
 }
 
@@ -616,7 +616,9 @@ int step_impl(hlbm* h, int64_t nsteps) {
 // with K layers of ghost nodes.  Layer 0 is the tile's own nodes; layer j
 // the nodes the updates of layer j-1 read (row columns; outer nodes read
 // nothing) that are in no earlier layer.  Slots: own nodes whose updates read
-// only own nodes (n_a), the other own nodes, then layers 1 .. K, each group
+// only own nodes (n_a of them; none when there are fewer than `early`, which
+// the kernel does not update ahead of the others), the other own nodes, then
+// layers 1 .. K, each group
 // in the caller's node order (on meshes built layer by layer consecutive
 // slots then run along a layer, which spreads a warp's gathers over the
 // shared-memory banks).  Sub-step s of a block computes the own nodes and
@@ -633,7 +635,7 @@ struct DeepTables {
 };
 
 bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, const std::vector<int32_t>& owner,
-                       int K, int comp_cap, DeepTables& D) {
+                       int K, int comp_cap, int early, DeepTables& D) {
     const int n = h->patch.n_nodes, n_tiles = (int)tile_start.size() - 1;
     D = DeepTables{};
     D.K = K;
@@ -642,11 +644,12 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
     D.rptr.assign(n_tiles + 1, 0);
     D.cnt.assign((size_t)kDeepCnt * n_tiles, 0);
     std::vector<int32_t> loc(n, -1);
+    const bool ofv = h->patch.outer_fv != 0;  // outer nodes' rows are summed too
     std::vector<int8_t> held(n, 0);  // a node some other tile holds as a ghost
     std::vector<std::vector<int32_t>> nbs(n_tiles);
     auto by_caller = [&](int32_t a, int32_t b) { return h->perm[a] < h->perm[b]; };
     auto reads = [&](int q, auto&& fn) {
-        if (h->kind[q] == HLBM_NODE_OUTER) return;
+        if (h->kind[q] == HLBM_NODE_OUTER && !ofv) return;
         for (int e = h->row_ptr[q] + 1; e < h->row_ptr[q + 1]; ++e) fn(h->col[e]);
     };
     for (int k = 0; k < n_tiles; ++k) {
@@ -656,6 +659,10 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
             bool inside = true;
             reads(q, [&](int c) { inside = inside && c >= p0 && c < p1; });
             (inside ? A : B).push_back(q);
+        }
+        if ((int)A.size() < early) {  // none are updated early: one run over the own nodes
+            B.insert(B.end(), A.begin(), A.end());
+            A.clear();
         }
         std::sort(A.begin(), A.end(), by_caller);
         std::sort(B.begin(), B.end(), by_caller);
@@ -697,18 +704,21 @@ bool build_deep_tables(const hlbm* h, const std::vector<int32_t>& tile_start, co
         if (n_comp > comp_cap) return false;
         D.comp_cap = std::max(D.comp_cap, n_comp);
         // computed slots: row images (columns as local slots; outer nodes
-        // read none of theirs), outer slots for the staged feed
+        // read none of theirs without outer_fv)
         for (int x = 0; x < n_comp; ++x) {
             const int q = order[x];
             D.row_gid.push_back(q);
             for (int j = 0; j < kTmemMaxEntries; ++j) {
                 const int e = h->row_ptr[q] + 1 + j;
                 int lc = x;
-                if (e < h->row_ptr[q + 1] && h->kind[q] != HLBM_NODE_OUTER) lc = loc[h->col[e]];
+                if (e < h->row_ptr[q + 1] && (ofv || h->kind[q] != HLBM_NODE_OUTER)) lc = loc[h->col[e]];
                 D.lcol.push_back(lc);
             }
-            if (h->kind[q] == HLBM_NODE_OUTER) D.oslot.push_back((uint16_t)x);
         }
+        // outer slots: those computed, and with outer_fv every one (their rows
+        // read the interpolated values of ghosts too)
+        for (int x = 0; x < (ofv ? n_slot : n_comp); ++x)
+            if (h->kind[order[x]] == HLBM_NODE_OUTER) D.oslot.push_back((uint16_t)x);
         D.gid.insert(D.gid.end(), order.begin(), order.end());
         D.ptr[k + 1] = (int32_t)D.gid.size();
         D.rptr[k + 1] = (int32_t)D.row_gid.size();
@@ -769,7 +779,7 @@ constexpr int kDeepQuadMax = 160;
 // tile-local columns, node orders and send flags; previous tables are
 // released.  Needs the FV matrices (d.coef).
 template <typename T>
-int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
+int build_tiles(hlbm* h, int n_tiles_req, int kind = HLBM_FV_AUTO) {
     Dev<T>& d = dev_of<T>(h);
     cudaStream_t s = h->stream;
     const int n = h->patch.n_nodes;
@@ -827,21 +837,24 @@ int build_tiles(hlbm* h, int n_tiles_req, bool tmem_only = false) {
         return cap;
     };
     const int ocap0 = outer_cap();
-    // HLBM_FV_* (0: the fastest that applies); a sweep pack needs the tensor-memory kernel
-    const int want = tmem_only ? HLBM_FV_TMEM : h->patch.fv_kernel;
+    // HLBM_FV_* (0: the fastest that applies); a sweep pack asks for one kernel
+    const int want = kind != HLBM_FV_AUTO ? kind : h->patch.fv_kernel;
     const bool tiles_ok = tile_cap <= fv_tile_max<T>() && tile_cap + halo_cap < 65536;
     // deep tiles: the deepest exchange interval up to fv_depth that fits
     DeepTables deep;
     bool deep_ok = false;
     int deep_quads = 0;
-    if ((want == HLBM_FV_AUTO || want == HLBM_FV_DEEP) && max_row - 1 <= 7 && h->patch.outer_fv == 0) {
-        for (int K = std::min(h->fv_depth, kDeepMaxK); K >= 1 && !deep_ok; --K) {
-            if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), deep)) continue;
+    if ((want == HLBM_FV_AUTO || (want == HLBM_FV_DEEP && h->patch.outer_fv == 0)) && max_row - 1 <= 7) {
+        // a pack of FP64 solvers fills the SMs' FP64 pipes, and recomputed ghosts cost more than exchanges
+        const int depth = kind != HLBM_FV_AUTO && sizeof(T) == 8 ? 1 : std::min(h->fv_depth, kDeepMaxK);
+        for (int K = depth; K >= 1 && !deep_ok; --K) {
+            if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), fv_deep_early<T>(), deep)) continue;
             // FP64, few computed slots: four lanes per node
-            deep_quads = sizeof(T) == 8 && deep.comp_cap <= kDeepQuadMax ? deep.comp_cap : 0;
+            const int ocap1 = std::max(deep.ocap, 1);
+            deep_quads = sizeof(T) == 8 && h->patch.outer_fv == 0 && deep.comp_cap <= kDeepQuadMax ? deep.comp_cap : 0;
             deep_ok = deep.slot_cap < 65536 &&
-                      fv_deep_tile_capacity<T>(fv_deep_smem_bytes<T>(deep.slot_cap, h->patch.n_sub,
-                                                                       std::max(deep.ocap, 1), deep_quads)) >= n_tiles;
+                      fv_deep_tile_capacity<T>(fv_deep_smem_bytes<T>(deep.slot_cap, h->patch.n_sub, ocap1, deep_quads,
+                                                                   h->patch.outer_fv ? ocap1 : 0)) >= n_tiles;
         }
     }
     const size_t smem = fv_smem_bytes<T>(tile_cap, std::max(halo_cap, 1), std::max(max_row - 1, 0),
@@ -1805,8 +1818,8 @@ int inst_fv(hlbm* h, cudaStream_t s, PendingStep& ps, cudaEvent_t e0, cudaEvent_
 int inst_finish(hlbm* h, cudaStream_t s, const PendingStep& ps) {
     return h->dtype != HLBM_F64 ? step_finish<float>(h, s, ps) : step_finish<double>(h, s, ps);
 }
-int inst_retile(hlbm* h, int tiles, bool tmem_only = false) {
-    return h->dtype != HLBM_F64 ? build_tiles<float>(h, tiles, tmem_only) : build_tiles<double>(h, tiles, tmem_only);
+int inst_retile(hlbm* h, int tiles, int kind = HLBM_FV_AUTO) {
+    return h->dtype != HLBM_F64 ? build_tiles<float>(h, tiles, kind) : build_tiles<double>(h, tiles, kind);
 }
 
 // the tile count of solver i for the tuner's pick (0, the default, before tuning)
@@ -1815,13 +1828,14 @@ int tuned_tiles(const hlbm_sweep* w, int i) {
     return c > 0 ? (w->inst[i]->patch.n_nodes + c - 1) / c : 0;
 }
 
-// The FV sub-steps of pack p's instances in one cooperative launch of the
-// tensor-memory kernel on the sweep's FV stream.
+// The FV sub-steps of pack p's instances in one cooperative launch on the
+// sweep's FV stream (the kernel that sweep_pack chose for all of them).
 template <typename T>
 int pack_fv(hlbm_sweep* w, size_t p, const std::vector<PendingStep>& ps) {
     const std::vector<int>& mem = w->packs[p];
     FvPack<T> pk{};
     pk.n = (int)mem.size();
+    const bool deep = w->inst[mem[0]]->fv_kind == HLBM_FV_DEEP;
     int blocks = 0;
     size_t smem = 0;
     for (int k = 0; k < pk.n; ++k) {
@@ -1833,9 +1847,15 @@ int pack_fv(hlbm_sweep* w, size_t p, const std::vector<PendingStep>& ps) {
         pk.g0[k] = (T*)d.fu_in;
         pk.g1[k] = d.fu_out;
         blocks += d.n_tiles;
-        smem = std::max(smem, fv_tmem_smem_bytes<T>(d.tile_cap, d.halo_cap, d.n_sub, d.tile_ocap));
+        if (deep) {
+            pk.a[k].xtag = h->xtag;
+            h->xtag += (unsigned)((d.n_sub + d.deep_k - 1) / d.deep_k);
+            smem = std::max(smem, fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads, 0));
+        } else {
+            smem = std::max(smem, fv_tmem_smem_bytes<T>(d.tile_cap, d.halo_cap, d.n_sub, d.tile_ocap));
+        }
     }
-    cudaError_t e = launch_fv_tmem_pack<T>(pk, blocks, smem, w->fv);
+    cudaError_t e = deep ? launch_fv_deep_pack<T>(pk, blocks, smem, w->fv) : launch_fv_tmem_pack<T>(pk, blocks, smem, w->fv);
     if (e != cudaSuccess) {
         w->err = std::string("packed FV launch: ") + cudaGetErrorString(e);
         return HLBM_ECUDA;
@@ -3142,26 +3162,34 @@ int hlbm_sweep_pack(hlbm_sweep_t* w, int32_t enable, int32_t* n_packs) {
                 --tiles[big];
                 --tsum;
             }
-            bool ok = tsum <= sms;
-            for (size_t q = 0; q < g.size() && ok && rc == HLBM_OK; ++q) {
-                hlbm* h = w->inst[g[q]];
-                // tiles the tensor-memory kernel cannot hold (its shared
-                // memory grows with the tile and its halo) are made smaller,
-                // a quarter more tiles at a time, while the SMs last
-                for (;;) {
-                    rc = inst_retile(h, tiles[q], true);
-                    if (rc != HLBM_EINVAL) break;
-                    const int more = std::max(1, tiles[q] / 4);
-                    if (tsum + more > sms || tiles[q] + more > std::max(1, h->patch.n_nodes / 64)) break;
-                    tiles[q] += more;
-                    tsum += more;
+            // the deep-tile kernel for all of them, or the tensor-memory kernel, which
+            // holds larger tiles
+            bool ok = false;
+            for (const int kind : {HLBM_FV_DEEP, HLBM_FV_TMEM}) {
+                std::vector<int> tl = tiles;
+                int sum = tsum;
+                ok = sum <= sms;
+                for (size_t q = 0; q < g.size() && ok && rc == HLBM_OK; ++q) {
+                    hlbm* h = w->inst[g[q]];
+                    // tiles the kernel cannot hold (its shared memory grows with the
+                    // tile and its halo) are made smaller, a quarter more tiles at a
+                    // time, while the SMs last
+                    for (;;) {
+                        rc = inst_retile(h, tl[q], kind);
+                        if (rc != HLBM_EINVAL) break;
+                        const int more = std::max(1, tl[q] / 4);
+                        if (sum + more > sms || tl[q] + more > std::max(1, h->patch.n_nodes / 64)) break;
+                        tl[q] += more;
+                        sum += more;
+                    }
+                    if (rc == HLBM_EINVAL) {
+                        rc = HLBM_OK;
+                        ok = false;
+                        break;
+                    }
+                    ok = rc == HLBM_OK && h->fv_kind == kind && h->n_tiles == tl[q];
                 }
-                if (rc == HLBM_EINVAL) {
-                    rc = HLBM_OK;
-                    ok = false;
-                    break;
-                }
-                ok = rc == HLBM_OK && h->fv_kind == HLBM_FV_TMEM && h->n_tiles == tiles[q];
+                if (ok || rc != HLBM_OK) break;
             }
             if (rc != HLBM_OK) {
                 w->err = "packing: " + w->inst[g[0]]->err;

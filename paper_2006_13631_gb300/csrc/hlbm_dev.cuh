@@ -606,14 +606,15 @@ template <typename T> void launch_build_ell(const Coef<T>* coef, const int32_t* 
                                             int64_t count, cudaStream_t s);
 template <typename T> int fv_smem_tile_capacity(size_t smem);
 template <typename T> cudaError_t launch_fv_smem(const Dev<T>& d, const StepArgs& a, cudaStream_t s);
-// deep tiles (temporal blocking): rows with at most 7 off-diagonal entries, Dirichlet outer nodes
+// deep tiles (temporal blocking): rows with at most 7 off-diagonal entries
 constexpr int kTmemMaxEntries = 7;  // off-diagonal entries a row may have in the TMEM and deep kernels
 constexpr int kDeepMaxK = 4;  // most sub-steps between exchanges
 constexpr int kDeepCnt = 3 + kDeepMaxK;
 template <typename T> int fv_deep_tmem_slots();          // computed slots a tile may have
+template <typename T> int fv_deep_early();               // own nodes from which a tile updates some ahead
 template <typename T> int fv_deep_row_words();           // words of one row image
 template <typename T> size_t fv_deep_packet_bytes(int n); // exchange packets of n nodes
-template <typename T> size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows);
+template <typename T> size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows, int stars);
 template <typename T> int fv_deep_tile_capacity(size_t smem);
 template <typename T>
 cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>* far, cudaStream_t s);
@@ -625,7 +626,7 @@ template <typename T> void launch_build_deep_rows(const Dev<T>& d, const int32_t
 template <typename T> size_t fv_tmem_smem_bytes(int tile_cap, int halo_cap, int n_sub, int ocap);
 template <typename T> int fv_tmem_tile_capacity(size_t smem);
 template <typename T> cudaError_t launch_fv_tmem(const Dev<T>& d, const StepArgs& a, cudaStream_t s);
-// several solvers' FV sub-steps in one launch of the tensor-memory kernel
+// several solvers' FV sub-steps in one launch of the deep-tile or the tensor-memory kernel
 constexpr int kFvPackMax = 16;
 template <typename T>
 struct FvPack {
@@ -636,6 +637,7 @@ struct FvPack {
     T* g0[kFvPackMax];       // record buffers: sub-step m reads g0 when m is even
     T* g1[kFvPackMax];
 };
+template <typename T> cudaError_t launch_fv_deep_pack(const FvPack<T>& pk, int blocks, size_t smem, cudaStream_t s);
 template <typename T> cudaError_t launch_fv_tmem_pack(const FvPack<T>& pk, int blocks, size_t smem, cudaStream_t s);
 template <typename T> void launch_force(const Dev<T>& d, int64_t t_out, cudaStream_t s);  // 2 launches
 template <typename T> void launch_patch_macro(const Dev<T>& d, double* rho, double* ux, double* uy,

@@ -1224,7 +1224,7 @@ cudaError_t launch_fv_tmem(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // sub-steps (temporal blocking).  A tile holds, as local "slots", its own
 // nodes and K layers of ghost nodes around them: layer j holds the nodes
 // that the updates of layer j-1 read and that are not in earlier layers
-// (outer nodes read nothing).  Sub-step s of a block of K recomputes the
+// (outer nodes read nothing, except with outer_fv).  Sub-step s of a block of K recomputes the
 // own nodes and ghost layers 1 .. K-1-s from the tile's own data, so the
 // tile needs its neighbours' records only once per block.  The arithmetic of
 // a node is that of the other FV kernels (fv_node.cuh, same entry order), so
@@ -1282,6 +1282,15 @@ template <typename T>
 int fv_deep_tmem_slots() {
     return kDeepGroups<T> * kDeepFv<T>;
 }
+// own nodes reading only own nodes from which a tile updates them ahead of the
+// others, while the ghosts are on their way: when they fill the FV warps; fewer
+// are left for after the wait, since one pass over all slots then takes no
+// longer than over a part.  (FP64 from 64 nodes on: the FP64 pipe is busy
+// either way; 25.5 instead of 22.6 us per sub-step on 24 380 nodes.)
+template <typename T>
+int fv_deep_early() {
+    return kDeepFv<T>;
+}
 template <typename T>
 int fv_deep_row_words() {
     return kDeepSlotWords<T>;
@@ -1305,12 +1314,13 @@ struct alignas(16) QuadRow {
 };
 
 struct DeepSmem {
-    size_t buf0, buf1, uv, osnap, rows, gid, kind, send, omap, total;
+    size_t buf0, buf1, uv, osnap, star, rows, gid, kind, send, omap, total;
 };
 
-// quad_rows: computed slots whose rows are kept in shared memory (0: none)
+// quad_rows: computed slots whose rows are kept in shared memory (0: none);
+// stars: outer slots whose interpolated records are kept, twice (outer_fv)
 template <typename T>
-__host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int ocap, int quad_rows) {
+__host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int ocap, int quad_rows, int stars) {
     auto up = [](size_t x) { return (x + 15) / 16 * 16; };
     DeepSmem L;
     size_t o = 0;
@@ -1322,6 +1332,8 @@ __host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int oca
     o = up(o + sizeof(T) * 2 * (size_t)n_sub);
     L.osnap = o;
     o = up(o + sizeof(T) * kSnap * (size_t)ocap);
+    L.star = o;
+    o = up(o + 2 * sizeof(T) * kSR * (size_t)stars);
     L.rows = o;
     o = up(o + sizeof(QuadRow) * (size_t)quad_rows);
     L.gid = o;
@@ -1337,8 +1349,8 @@ __host__ __device__ inline DeepSmem deep_smem_layout(int cap, int n_sub, int oca
 }
 
 template <typename T>
-size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows) {
-    return deep_smem_layout<T>(slot_cap, n_sub, ocap, quad_rows).total;
+size_t fv_deep_smem_bytes(int slot_cap, int n_sub, int ocap, int quad_rows, int stars) {
+    return deep_smem_layout<T>(slot_cap, n_sub, ocap, quad_rows, stars).total;
 }
 
 // ---- packets: one relaxed 128-bit access each (value bits low, tag on top)
@@ -1476,15 +1488,30 @@ __device__ __forceinline__ void adj_record(const Dev<T>& d, int m, int g, bool r
 // image is loaded by every lane of the warp at points where the warp is
 // converged (tcgen05.ld is .sync.aligned); only the arithmetic between the
 // loads is predicated.
-template <typename T, bool kRecord>
+// kOuterFv: outer nodes take eq. postcollision2_u with its FV sums (outer_fv):
+// their row is summed like any other, over the starred values -- star, the
+// interpolated records of this sub-step at outer slots, own one included, and
+// the patch records elsewhere.
+template <typename T, bool kRecord, bool kOuterFv>
 __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* sm, const DeepSmem& L, const T* cur,
                                           T* nxt, uint32_t tslot, bool valid, int x, int m, unsigned char* pkt,
-                                          unsigned tag, bool own_slot) {
+                                          unsigned tag, bool own_slot, const T* star) {
     constexpr int EW = kDeepEntryWords<T>;
-    const int8_t kind = valid ? reinterpret_cast<const int8_t*>(sm + L.kind)[x] : (int8_t)HLBM_NODE_OUTER;
+    const int8_t* kd = reinterpret_cast<const int8_t*>(sm + L.kind);
+    const int16_t* om = reinterpret_cast<const int16_t*>(sm + L.omap);
+    const int8_t kind = valid ? kd[x] : (int8_t)HLBM_NODE_OUTER;
+    const bool outer = kind == HLBM_NODE_OUTER;
+    const bool row = kOuterFv ? valid : !outer;  // the slot's row is summed
+    const T* own_rec = cur + (size_t)kSR * x;
+    if (kOuterFv && outer && valid) own_rec = star + (size_t)kSR * om[x];
+    auto rec_at = [&](int col) {
+        const T* r = cur + (size_t)kSR * col;
+        if (kOuterFv && outer && kd[col] == HLBM_NODE_OUTER) r = star + (size_t)kSR * om[col];
+        return ld_rec(r);
+    };
     Pops<T> P{};
-    if (valid && kind != HLBM_NODE_OUTER) {
-        const RecP<T> own = ld_rec(cur + (size_t)kSR * x);
+    if (row) {
+        const RecP<T> own = ld_rec(own_rec);
         P.A = own.A, P.B = own.B, P.C = own.C, P.D = own.D;
     }
     FvSums<T> acc;
@@ -1495,7 +1522,7 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
         uint32_t hdr[4];
         tmem_ld4(tslot, hdr);
         cP = __uint_as_float(hdr[0]);
-        const int ne = kind != HLBM_NODE_OUTER ? (int)hdr[1] : 0;
+        const int ne = row ? (int)hdr[1] : 0;
         const int nem = (int)__reduce_max_sync(0xffffffffu, (unsigned)ne);
         // two entries per tensor-memory load (one wait for both; entry 7 of
         // the last pair reads the next columns, which no row uses)
@@ -1506,10 +1533,10 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
             tmem_ld8(tslot + EW * (j + 1), e);
             if (j < ne)
                 fv_sums_entry(acc, __uint_as_float(e[0]), __uint_as_float(e[1]), __uint_as_float(e[2]),
-                              ld_rec(cur + (size_t)kSR * (int)e[3]), P);
+                              rec_at((int)e[3]), P);
             if (j + 1 < ne)
                 fv_sums_entry(acc, __uint_as_float(e[4]), __uint_as_float(e[5]), __uint_as_float(e[6]),
-                              ld_rec(cur + (size_t)kSR * (int)e[7]), P);
+                              rec_at((int)e[7]), P);
         }
     } else {
         constexpr int H = kDeepHalf<T>;
@@ -1517,14 +1544,14 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
         uint32_t v[H];
         tmem_ldn<H>(tslot, v);
         cP = from_words<T>(v[0], v[1]);
-        const int ne = kind != HLBM_NODE_OUTER ? (int)v[2] : 0;
+        const int ne = row ? (int)v[2] : 0;
 #pragma unroll
         for (int j = 0; j < E0; ++j) {
             if (j < ne) {
                 T gx, gy, c;
                 int col;
                 deep_entry<T, H>(v, EW * (j + 1), gx, gy, c, col);
-                fv_sums_entry(acc, gx, gy, c, ld_rec(cur + (size_t)kSR * col), P);
+                fv_sums_entry(acc, gx, gy, c, rec_at(col), P);
             }
         }
         __syncwarp();
@@ -1535,18 +1562,17 @@ __device__ __forceinline__ void deep_node(const Dev<T>& d, const unsigned char* 
                 T gx, gy, c;
                 int col;
                 deep_entry<T, H>(v, EW * (j - E0), gx, gy, c, col);
-                fv_sums_entry(acc, gx, gy, c, ld_rec(cur + (size_t)kSR * col), P);
+                fv_sums_entry(acc, gx, gy, c, rec_at(col), P);
             }
         }
     }
     if (!valid) return;
     Pops<T> fn, nq{};
     T mo[3] = {};
-    if (kind == HLBM_NODE_OUTER) {
-        const int q = reinterpret_cast<const int16_t*>(sm + L.omap)[x];
-        fn = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m);
+    if (!row) {
+        fn = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * om[x], 1, m);
     } else {
-        fn = fv_sums_finish(d, acc, cP, ld_rec(cur + (size_t)kSR * x), nq);
+        fn = fv_sums_finish(d, acc, cP, ld_rec(own_rec), nq);
         if (kind == HLBM_NODE_WALL) {
             const T* uv = reinterpret_cast<const T*>(sm + L.uv);
             fv_wall(d, uv[m], uv[d.n_sub + m], fn, mo);
@@ -1817,20 +1843,22 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
     return ok;
 }
 
-// kRecord: also writes what the reverse mode needs of every sub-step (Dev::fv_rec)
-template <typename T, bool kRecord>
-__global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int abort_sh;
-    __shared__ uint32_t tmem_base_sh;
+// The FV sub-steps of tile `tile` of the solver d (one block); k_fv_deep runs
+// one solver, k_fv_deep_pack several.  kRecord: also writes what the reverse
+// mode needs of every sub-step (Dev::fv_rec).
+template <typename T, bool kRecord, bool kOuterFv>
+__device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a, T* g0, T* g1, const FarArgs<T>& far,
+                                             const int tile, unsigned char* sm, int& abort_sh,
+                                             uint32_t& tmem_base_sh) {
     constexpr int NT = kDeepFv<T>, BT = kDeepThreads<T>, G = kDeepGroups<T>, SW = kDeepSlotWords<T>;
-    const int tile = blockIdx.x, tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
     const int s0 = d.deep_ptr[tile];
     const int32_t* cnt = d.deep_cnt + kDeepCnt * tile;
     const int n_a = cnt[0], n_own = cnt[1], n_slot = cnt[2];
     const int K = d.deep_k;
-    const bool quads = sizeof(T) == 8 && d.deep_quads > 0;
-    const DeepSmem L = deep_smem_layout<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, quads ? d.deep_quads : 0);
+    const bool quads = sizeof(T) == 8 && !kOuterFv && d.deep_quads > 0;
+    const DeepSmem L =
+        deep_smem_layout<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, quads ? d.deep_quads : 0, kOuterFv ? d.deep_ocap : 0);
     T* buf0 = reinterpret_cast<T*>(sm + L.buf0);
     T* buf1 = reinterpret_cast<T*>(sm + L.buf1);
     T* uv = reinterpret_cast<T*>(sm + L.uv);
@@ -1914,6 +1942,21 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
         }
         tmem_wait_st();
     }
+    // interpolated records of the outer slots for sub-step m (outer_fv), thread k of n
+    const int n_star = kOuterFv ? d.deep_optr[tile + 1] - d.deep_optr[tile] : 0;
+    auto star_at = [&](int m) { return reinterpret_cast<T*>(sm + L.star) + (m & 1) * (size_t)kSR * d.deep_ocap; };
+    auto make_stars = [&](int m, int k, int n) {
+        for (int q = k; q < n_star; q += n) {
+            const Pops<T> f = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m);
+            T z[3], ux, uy;
+            z_of(f, d.rho0, z, ux, uy);
+            st_rec(star_at(m) + (size_t)kSR * q, rec_of(f, z));
+        }
+    };
+    if constexpr (kOuterFv) {
+        __syncthreads();  // the staged feed
+        make_stars(0, tid, BT);
+    }
     if (tid == 0) abort_sh = 0;
     tmem_fence_before();
     __syncthreads();
@@ -1922,10 +1965,9 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
     if (tid < NT) {
         const int nb0 = d.tile_nb_ptr[tile], nb1 = d.tile_nb_ptr[tile + 1];
         const int64_t xhalf = (int64_t)d.n * kPkts<T> * 16;
-        // own nodes that read only own nodes are updated while the ghosts are on
-        // their way when they fill the FV warps; fewer are left for after the
-        // wait, since one pass over all slots then takes no longer than over a part
-        const int n_early = n_a >= NT && !quads ? n_a : 0;
+        // own nodes that read only own nodes, updated while the ghosts are on
+        // their way (0 where that does not pay: fv_deep_early)
+        const int n_early = quads ? 0 : n_a;
         Quad Q;
         Q.q = tid & 3;
         Q.w = w_of<double>(Q.q < 2 ? 1 : 5);
@@ -1944,13 +1986,16 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                 const bool send = (s == kb - 1) && !final_block && tile != d.stall_tile;
                 const int cs = cnt[3 + s];
                 int lo = 0;
+                // the next sub-step's interpolated records (from the last FV thread down)
+                if (kOuterFv && m + 1 < d.n_sub) make_stars(m + 1, NT - 1 - tid, NT);
                 if (s == 0 && b > 0) {
 #pragma unroll
                     for (int j = 0; j < G; ++j) {
                         const int x = j * NT + tid;
                         const bool v = x < n_early;
                         if (__any_sync(0xffffffffu, v))
-                            deep_node<T, kRecord>(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u, true);
+                            deep_node<T, kRecord, kOuterFv>(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u, true,
+                                                            star_at(m));
                     }
                     bool ok = deep_receive<T, NT>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
                                                   a.xtag + (unsigned)b, NT - 1 - tid);
@@ -2002,10 +2047,10 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
                     const int x = j * NT + tid;
                     const bool v = x >= lo && x < cs;
                     if (__any_sync(0xffffffffu, v))
-                        deep_node<T, kRecord>(
+                        deep_node<T, kRecord, kOuterFv>(
                             d, sm, L, cur, nxt, tslot_of(j), v, x, m,
                             send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out,
-                            x < n_own);
+                            x < n_own, star_at(m));
                 }
                 fv_bar<NT>();
             }
@@ -2040,6 +2085,37 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
     if (warp == 0) tmem_dealloc_512(tbase);
 }
 
+template <typename T, bool kRecord, bool kOuterFv>
+__global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int abort_sh;
+    __shared__ uint32_t tmem_base_sh;
+    fv_deep_body<T, kRecord, kOuterFv>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, tmem_base_sh);
+}
+
+// Several solvers' FV sub-steps in one cooperative launch: block b runs tile
+// b - block0 of the item whose range [block0, next block0) holds b.  Each item
+// keeps its own tables, packets, tags, sub-step count and buffers; items only
+// share the GPU.
+template <typename T>
+__global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep_pack(const __grid_constant__ FvPack<T> pk) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int abort_sh;
+    __shared__ uint32_t tmem_base_sh;
+    int i = 0;
+    while (i + 1 < pk.n && pk.block0[i + 1] <= (int)blockIdx.x) ++i;
+    fv_deep_body<T, false, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<T>{}, (int)blockIdx.x - pk.block0[i], sm,
+                           abort_sh, tmem_base_sh);
+}
+
+template <typename T>
+cudaError_t launch_fv_deep_pack(const FvPack<T>& pk, int blocks, size_t smem, cudaStream_t s) {
+    FvPack<T> p = pk;
+    void* args[] = {&p};
+    return cudaLaunchCooperativeKernel((const void*)k_fv_deep_pack<T>, dim3(blocks), dim3(kDeepThreads<T>), args, smem,
+                                       s);
+}
+
 template <typename T>
 int fv_deep_tile_capacity(size_t smem) {
     if (smem == 0) return 0;
@@ -2048,7 +2124,8 @@ int fv_deep_tile_capacity(size_t smem) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // each block allocates all 512 TMEM columns: only one block per SM
-    for (const void* fn : {(const void*)k_fv_deep<T, false>, (const void*)k_fv_deep<T, true>}) {
+    for (const void* fn : {(const void*)k_fv_deep<T, false, false>, (const void*)k_fv_deep<T, true, false>,
+                           (const void*)k_fv_deep<T, false, true>, (const void*)k_fv_deep_pack<T>}) {
         cudaFuncAttributes fa{};
         if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
             cudaGetLastError();
@@ -2075,8 +2152,11 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
     FarArgs<T> fa{};
     if (far && sizeof(T) == 4) fa = *far;
     void* args[] = {&dd, &aa, &b0, &b1, &fa};
-    const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads);
-    const void* fn = d.fv_rec ? (const void*)k_fv_deep<T, true> : (const void*)k_fv_deep<T, false>;
+    const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads,
+                                               d.outer_fv ? d.deep_ocap : 0);
+    const void* fn = d.outer_fv ? (const void*)k_fv_deep<T, false, true>
+                     : d.fv_rec ? (const void*)k_fv_deep<T, true, false>
+                                : (const void*)k_fv_deep<T, false, false>;
     return cudaLaunchCooperativeKernel(fn, dim3(d.n_tiles), dim3(kDeepThreads<T>), args, smem, s);
 }
 
@@ -3355,10 +3435,12 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template cudaError_t launch_fv_tmem<T>(const Dev<T>&, const StepArgs&, cudaStream_t);                     \
     template cudaError_t launch_fv_tmem_pack<T>(const FvPack<T>&, int, size_t, cudaStream_t);                 \
     template int fv_deep_tmem_slots<T>();                                                                     \
+    template int fv_deep_early<T>();                                                                          \
     template int fv_deep_row_words<T>();                                                                      \
     template size_t fv_deep_packet_bytes<T>(int);                                                             \
-    template size_t fv_deep_smem_bytes<T>(int, int, int, int);                                                \
+    template size_t fv_deep_smem_bytes<T>(int, int, int, int, int);                                                \
     template int fv_deep_tile_capacity<T>(size_t);                                                            \
+    template cudaError_t launch_fv_deep_pack<T>(const FvPack<T>&, int, size_t, cudaStream_t);                 \
     template cudaError_t launch_fv_deep<T>(const Dev<T>&, const StepArgs&, const FarArgs<T>*, cudaStream_t);  \
     template void launch_build_deep_rows<T>(const Dev<T>&, const int32_t*, const int32_t*, int64_t, uint32_t*, \
                                             cudaStream_t);                                                    \

@@ -74,3 +74,35 @@ def test_adjoint_of_a_patch_of_more_nodes_than_resident_quads():
         H.hlbm_destroy(h)
     quotient = (L[1] - L[0]) / (2e-5 * w.tau_s)
     assert abs(g[2] - quotient) <= 1e-5 * abs(quotient)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("mesh_args", [SMALL, MEDIUM, LARGE], ids=["small", "medium", "large"])
+def test_outer_node_sums_agree_bit_for_bit(mesh_args, dtype):
+    """outer_fv: the deep tiles (automatic choice, every exchange interval) and the
+    shared- and global-memory kernels run the same arithmetic."""
+    from paper_2006_13631_gb300 import Solver, hlbm_set_fv_depth
+
+    w = _case(dtype, mesh_args, n_sub=25)
+    w.outer_fv = 1
+    mesh, rho = w.mesh(), w.rho_init()
+    got = []
+    for kern in (1, 2, 0):
+        w.fv_kernel = kern
+        try:
+            s = Solver(w, mesh=mesh, rho_init=rho)
+        except Exception:
+            assert kern == 2 and dtype == "f64"  # tiles too large for the shared-memory kernel
+            continue
+        if kern == 0 and mesh_args is not LARGE:
+            assert s.info()["fv_kernel"] == 4
+        for depth in (1, 2, 3, 4) if s.info()["fv_kernel"] == 4 else (0, 0, 0, 0):
+            if depth:
+                hlbm_set_fv_depth(s.h, depth)
+            s.step(3)
+        assert s.status == 0
+        got.append(tuple(s.fields()) + (s.patch_f(), s.force()[1]))
+        s.close()
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
