@@ -98,6 +98,12 @@ __device__ __forceinline__ void pops_to(const Pops<T>& p, T (&f)[9]) {
     f[5] = px(p.C), f[6] = py(p.C), f[7] = px(p.D), f[8] = py(p.D);
 }
 
+// The state (drho, ux, uy, f^neq) that the interpolations between the grids
+// carry (Sec. 4, eq. postcollision2_s): pairs of opposite directions share the
+// even and odd parts of f^eq, and 1 / rho is formed once.
+template <typename T>
+__device__ __forceinline__ void state_of(const T (&f)[9], T rho0, T (&st)[12]);
+
 // sum f_i, sum c_ix f_i, sum c_iy f_i
 template <typename T>
 __device__ __forceinline__ void pops_moments(const Pops<T>& p, T& m0, T& mx, T& my) {
@@ -105,6 +111,34 @@ __device__ __forceinline__ void pops_moments(const Pops<T>& p, T& m0, T& mx, T& 
     m0 = add_rn(p.f0, add_rn(add_rn(px(s1), py(s1)), add_rn(px(s2), py(s2))));
     mx = add_rn(px(d1), sub_rn(px(d2), py(d2)));
     my = add_rn(py(d1), add_rn(px(d2), py(d2)));
+}
+
+// f_i^eq - w_i rho0 of the pair (i, opp(i)) as w_i (G + H), w_i (G - H)
+template <typename T>
+__device__ __forceinline__ void feq_pair(int i, T dr, T rho, T ux, T uy, T q, T& a, T& b) {
+    const T cu = cdot(i, ux, uy);
+    const T G = fma_rn(rho, fma_rn(mul_rn(T(4.5), cu), cu, q), dr), H = mul_rn(rho, mul_rn(T(3), cu));
+    a = mul_rn(w_of<T>(i), add_rn(G, H));
+    b = mul_rn(w_of<T>(i), sub_rn(G, H));
+}
+template <typename T>
+__device__ __forceinline__ void state_of(const T (&f)[9], T rho0, T (&st)[12]) {
+    T dr, jx, jy;
+    pops_moments(pops_of(f), dr, jx, jy);
+    const T rho = add_rn(rho0, dr), inv = T(1) / rho, ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
+    const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
+    st[0] = dr;
+    st[1] = ux;
+    st[2] = uy;
+    st[3] = sub_rn(f[0], mul_rn(w_of<T>(0), fma_rn(rho, q, dr)));
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        if (opp_of(i) < i) continue;
+        T a, b;
+        feq_pair(i, dr, rho, ux, uy, q, a, b);
+        st[3 + i] = sub_rn(f[i], a);
+        st[3 + opp_of(i)] = sub_rn(f[opp_of(i)], b);
+    }
 }
 
 // acc - w_i (G_i + 3 c_i . (x, y)) over the moving directions, G = (g1, g2)

@@ -101,7 +101,7 @@ struct hlbm {
     // after the FV sub-steps); the next FV launch, which rewrites both patch
     // buffers, waits for it, and every hlbm_step call joins it before returning
     cudaStream_t side = nullptr;
-    cudaEvent_t ev_fv = nullptr, ev_force = nullptr, ev_move = nullptr, ev_cls = nullptr;
+    cudaEvent_t ev_fv = nullptr, ev_force = nullptr;
     bool force_pending = false;
     // tag of the last exchange of a deep-tile FV launch: only ever grows (a
     // restored or abandoned step never meets packets with its own tags)
@@ -409,28 +409,15 @@ int step_lattice(hlbm* h, cudaStream_t s, PendingStep& ps) {
     d.sbox_new = (T*)h->sbox[1 - h->si];
     int ev = phase_begin(h, s);
     if (t > 0) {
-        // 2. classify the lattice nodes against the moved fictitious curve: on
-        // the side stream beside the refill when the solver steps on its own
-        // stream (classification is geometry only, and the class buffer it
-        // writes was last read by the previous step's refill and feed)
-        const bool cls_side = h->side && s == h->stream;
-        if (cls_side) {
-            cudaEventRecord(h->ev_move, s);
-            cudaStreamWaitEvent(h->side, h->ev_move, 0);
-            launch_classify<T>(d, a, h->side);
-            cudaEventRecord(h->ev_cls, h->side);
-        }
+        // 2. classify the lattice nodes against the moved fictitious curve (the
+        // same launch)
         launch_refill<T>(d, a, s);
         h->ui = 1 - h->ui;
         bind(h, d);
-        if (cls_side)
-            cudaStreamWaitEvent(s, h->ev_cls, 0);
-        else
-            launch_classify<T>(d, a, s);
     }
     // 3. interpolation nodes from the patch (eq. postcollision2_s)
     launch_fill<T>(d, a, s);
-    phase_end(h, HLBM_PHASE_MOVE, ev, t > 0 ? 3 : 1, s);
+    phase_end(h, HLBM_PHASE_MOVE, ev, t > 0 ? 2 : 1, s);
     // 4. stream-collide t -> t+1 (eq. LBE)
     ev = phase_begin(h, s);
     int nl = 1;
@@ -591,9 +578,7 @@ int step_impl(hlbm* h, int64_t nsteps) {
     if (side && !h->side) {
         if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->ev_fv, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->ev_force, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->ev_move, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->ev_cls, cudaEventDisableTiming) != cudaSuccess)
+            cudaEventCreateWithFlags(&h->ev_force, cudaEventDisableTiming) != cudaSuccess)
             return cuda_check(h, cudaGetLastError(), "side stream");
     }
     int rc = HLBM_OK;
@@ -3258,7 +3243,7 @@ void hlbm_destroy(hlbm_t* h) {
         cudaStreamSynchronize(h->side);
         cudaStreamDestroy(h->side);
     }
-    for (cudaEvent_t e : {h->ev_fv, h->ev_force, h->ev_move, h->ev_cls})
+    for (cudaEvent_t e : {h->ev_fv, h->ev_force})
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     if (h->st_event) cudaEventDestroy(h->st_event);

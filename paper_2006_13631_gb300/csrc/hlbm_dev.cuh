@@ -476,55 +476,60 @@ __device__ __forceinline__ int locate_warp(const Dev<T>& d, double qx, double qy
 
 template <typename T>
 __device__ __forceinline__ int locate_from_node(const Dev<T>& d, int P, double qx, double qy, double lam[3]) {
-    int best = -1, best_slot = 0;
-    double best_min = -1.0e300;
     // q = x_P + (dx, dy): an FP32 estimate of the coordinates, lambda_j =
     // [j == P] + grad lambda_j . (dx, dy), discards triangles clearly not
     // holding q (estimate below -1e-5, far beyond its ~1e-7 error); the
-    // others take the exact FP64 test
+    // others take the exact FP64 test.  The star is walked once for the
+    // estimates and its few candidates are kept, so that a warp runs the FP64
+    // test (some 30 instructions at 1/64 of the FP32 rate) as often as its
+    // lane with the most candidates has any, not once for every position in
+    // the star at which some lane has one.
+    constexpr int kCand = 3;
     const float dx = float(__dsub_rn(qx, d.xy[2 * P])), dy = float(__dsub_rn(qy, d.xy[2 * P + 1]));
+    const int e0 = d.tstart[P], e1 = d.tstart[P + 1];
+    int cand[kCand] = {0, 0, 0}, slots = 0, count = 0;
+    float m1 = 0.f, est[3] = {0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (int e = e0; e < e1; ++e) {
+        const int k = d.tlist[e];
+        const int32_t* v = d.tri + 3 * k;
+        const int slot = v[0] == P ? 0 : (v[1] == P ? 1 : 2);
+        const float* gr = d.trigrad + 6 * (int64_t)k;
+        const float l0 = fmaf(gr[0], dx, gr[1] * dy) + (slot == 0 ? 1.0f : 0.0f);
+        const float l1 = fmaf(gr[2], dx, gr[3] * dy) + (slot == 1 ? 1.0f : 0.0f);
+        const float l2 = fmaf(gr[4], dx, gr[5] * dy) + (slot == 2 ? 1.0f : 0.0f);
+        const float mn = fminf(l0, fminf(l1, l2));
+        if (mn < -1e-5f) continue;
+        if (count == 0) {
+            m1 = mn;
+            est[0] = l0;
+            est[1] = l1;
+            est[2] = l2;
+        }
+#pragma unroll
+        for (int c = 0; c < kCand; ++c)
+            if (count == c) {
+                cand[c] = k;
+                slots |= slot << (2 * c);
+            }
+        ++count;
+    }
     if constexpr (sizeof(T) == 4) {
         // FP32 populations: when a single star triangle survives the estimate
         // and holds q clearly inside (every estimate above 1e-5), the exact
         // test can only accept it, so its decision is taken without FP64;
         // the estimates serve as the (FP32) interpolation weights
-        int count = 0, k1 = -1, slot1 = 0;
-        float m1 = 0.f, est[3] = {0.f, 0.f, 0.f};
-        for (int i = d.tstart[P]; i < d.tstart[P + 1] && count < 2; ++i) {
-            const int k = d.tlist[i];
-            const int32_t* v = d.tri + 3 * k;
-            const int slot = v[0] == P ? 0 : (v[1] == P ? 1 : 2);
-            const float* gr = d.trigrad + 6 * (int64_t)k;
-            const float l0 = fmaf(gr[0], dx, gr[1] * dy) + (slot == 0 ? 1.0f : 0.0f);
-            const float l1 = fmaf(gr[2], dx, gr[3] * dy) + (slot == 1 ? 1.0f : 0.0f);
-            const float l2 = fmaf(gr[4], dx, gr[5] * dy) + (slot == 2 ? 1.0f : 0.0f);
-            const float mn = fminf(l0, fminf(l1, l2));
-            if (mn < -1e-5f) continue;
-            if (++count == 1) {
-                k1 = k;
-                slot1 = slot;
-                m1 = mn;
-                est[0] = l0;
-                est[1] = l1;
-                est[2] = l2;
-            }
-        }
-        if (count == 1 && m1 > 1e-5f && est[slot1] > 1e-5f) {
+        const float own = (slots & 3) == 0 ? est[0] : (slots & 3) == 1 ? est[1] : est[2];
+        if (count == 1 && m1 > 1e-5f && own > 1e-5f) {
             lam[0] = est[0];
             lam[1] = est[1];
             lam[2] = est[2];
-            return k1;
+            return cand[0];
         }
     }
-    for (int e = d.tstart[P]; e < d.tstart[P + 1]; ++e) {
-        int k = d.tlist[e];
-        const int32_t* v = d.tri + 3 * k;
-        const int slot = v[0] == P ? 0 : (v[1] == P ? 1 : 2);
-        const float* gr = d.trigrad + 6 * (int64_t)k;
-        float l0 = fmaf(gr[0], dx, gr[1] * dy) + (slot == 0 ? 1.0f : 0.0f);
-        float l1 = fmaf(gr[2], dx, gr[3] * dy) + (slot == 1 ? 1.0f : 0.0f);
-        float l2 = fmaf(gr[4], dx, gr[5] * dy) + (slot == 2 ? 1.0f : 0.0f);
-        if (fminf(l0, fminf(l1, l2)) < -1e-5f) continue;
+    int best = -1;
+    double best_min = -1.0e300, best_own = 0.0;
+    auto exact = [&](int k, int slot) {
         double la, lb, lc;
         bary_rn(d.trigeo + 8 * (int64_t)k, qx, qy, la, lb, lc);
         double mn = la < lb ? la : lb;
@@ -532,13 +537,23 @@ __device__ __forceinline__ int locate_from_node(const Dev<T>& d, int P, double q
         if (mn >= -1e-12 && mn > best_min) {
             best = k;
             best_min = mn;
+            best_own = slot == 0 ? la : (slot == 1 ? lb : lc);
             lam[0] = la;
             lam[1] = lb;
             lam[2] = lc;
-            best_slot = slot;
+        }
+    };
+    if (count <= kCand) {
+#pragma unroll 1
+        for (int c = 0; c < count; ++c) exact(c == 0 ? cand[0] : c == 1 ? cand[1] : cand[2], (slots >> (2 * c)) & 3);
+    } else {  // q at or near P itself: every triangle of the star
+        for (int e = e0; e < e1; ++e) {
+            const int k = d.tlist[e];
+            const int32_t* v = d.tri + 3 * k;
+            exact(k, v[0] == P ? 0 : (v[1] == P ? 1 : 2));
         }
     }
-    if (best >= 0 && lam[best_slot] > 1e-6) return best;
+    if (best >= 0 && best_own > 1e-6) return best;
     return locate_dev(d, qx, qy, lam);
 }
 
@@ -551,6 +566,29 @@ __device__ __forceinline__ bool inside_curve(const Dev<T>& d, int x, int y, doub
     if (qx < 0.0) qx = 0.0;
     if (qy < 0.0) qy = 0.0;
     return __dadd_rn(__dmul_rn(qx, qx), __dmul_rn(qy, qy)) < d.df2;
+}
+
+// Sec. 4: discretization outside the fictitious curve, unused inside;
+// unused nodes with a discretization node among their 8 lattice neighbours are
+// interpolation nodes.  Window node b; every node outside the window is a
+// discretization node.
+template <typename T>
+__device__ __forceinline__ void classify_node(const Dev<T>& d, const StepArgs& a, int64_t b) {
+    const int x = a.bx0 + (int)(b % d.bw), y = a.by0 + (int)(b / d.bw);
+    int8_t c = CLS_DISC;
+    if (inside_curve(d, x, y, a.cx, a.cy)) {
+        c = CLS_UNUSED;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const int xx = x + cx_of(i), yy = y + cy_of(i);
+            if (xx < 0 || yy < 0 || xx >= d.nx || yy >= d.ny) continue;
+            if (!inside_curve(d, xx, yy, a.cx, a.cy)) {
+                c = CLS_INTERP;
+                break;
+            }
+        }
+    }
+    d.cls_cur[b] = c;
 }
 
 // ------------------------------------------------------- nested levels
@@ -596,7 +634,7 @@ struct Couple {
 template <typename T> void launch_couple(const Dev<T>& d, const Refine& r, const Couple& c, cudaStream_t s);
 template <typename T> void launch_fv_coeffs(const Dev<T>& d, int lumped, Coef<T>* coef, cudaStream_t s);
 template <typename T> void launch_patch_init(const Dev<T>& d, const StepArgs& a, cudaStream_t s);
-template <typename T> void launch_refill(const Dev<T>& d, const StepArgs& a, cudaStream_t s);
+template <typename T> void launch_refill(const Dev<T>& d, const StepArgs& a, cudaStream_t s);  // and classification
 template <typename T> void launch_feed(const Dev<T>& d, const StepArgs& a, cudaStream_t s);
 template <typename T> int fv_tile_capacity();
 template <typename T> cudaError_t launch_fv_persistent(const Dev<T>& d, const StepArgs& a, cudaStream_t s);

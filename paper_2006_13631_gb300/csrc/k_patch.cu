@@ -92,55 +92,99 @@ void launch_fv_coeffs(const Dev<T>& d, int lumped, Coef<T>* coef, cudaStream_t s
 // is read from a window (origin ox, oy) of pre-collision populations; with
 // cls given, the four donors must be discretization nodes.
 // st = (drho, ux, uy, f^neq[9]).
+//
+// Four lanes (aligned, all calling) share a point: lane q takes corner q, and
+// every lane returns the sums.  One thread per point took the corners one
+// after another, 36 dependent loads and in FP64 some 600 instructions.
 template <typename T>
-__device__ __forceinline__ void bilinear_state(const Dev<T>& d, const T* box, int ox, int oy, const int8_t* cls,
-                                               double wx, double wy, T st[12], int& cell) {
-    double fx0 = floor(wx), fy0 = floor(wy);
-    int ix = (int)fx0, iy = (int)fy0;
-    double ax = __dsub_rn(wx, fx0), ay = __dsub_rn(wy, fy0);
-    T w4[4] = {T((1.0 - ax) * (1.0 - ay)), T(ax * (1.0 - ay)), T((1.0 - ax) * ay), T(ax * ay)};
+__device__ __forceinline__ void bilinear_quad(const Dev<T>& d, const T* box, int ox, int oy, const int8_t* cls,
+                                              double wx, double wy, bool live, int q, T (&st)[12], int& cell) {
+    const double fx0 = floor(wx), fy0 = floor(wy);
+    const int ix = (int)fx0, iy = (int)fy0;
+    const double ax = __dsub_rn(wx, fx0), ay = __dsub_rn(wy, fy0);
+    const T w = T(((q & 1) ? ax : 1.0 - ax) * ((q >> 1) ? ay : 1.0 - ay));
     cell = iy * d.nx + ix;
+    const int bx = ix + (q & 1) - ox, by = iy + (q >> 1) - oy;
+    bool have = live;
+    if (live && ((unsigned)bx >= (unsigned)d.bw || (unsigned)by >= (unsigned)d.bh)) {
+        atomicOr(d.status, HLBM_ST_DONOR_NOT_COMPUTED);
+        have = false;
+    }
+    const int64_t b = have ? (int64_t)by * d.bw + bx : 0;
+    if (have && cls && cls[b] != CLS_DISC) atomicOr(d.status, HLBM_ST_DONOR_NOT_COMPUTED);
+    T f[9];
 #pragma unroll
-    for (int j = 0; j < 12; ++j) st[j] = T(0);
+    for (int i = 0; i < 9; ++i) f[i] = have ? box[i * d.bplane + b] : T(0);
+    state_of(f, d.rho0, st);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        int bx = ix + (q & 1) - ox, by = iy + (q >> 1) - oy;
-        if ((unsigned)bx >= (unsigned)d.bw || (unsigned)by >= (unsigned)d.bh) {
-            atomicOr(d.status, HLBM_ST_DONOR_NOT_COMPUTED);
-            continue;
-        }
-        int64_t b = (int64_t)by * d.bw + bx;
-        if (cls && cls[b] != CLS_DISC) atomicOr(d.status, HLBM_ST_DONOR_NOT_COMPUTED);
-        T f[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = box[i * d.bplane + b];
-        T dr, r, ux, uy;
-        moments_dev(f, d.rho0, dr, r, ux, uy);
-        st[0] += w4[q] * dr;
-        st[1] += w4[q] * ux;
-        st[2] += w4[q] * uy;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) st[3 + i] += w4[q] * (f[i] - feq_dev<T>(i, dr, r, ux, uy));
+    for (int j = 0; j < 12; ++j) {
+        st[j] = have ? w * st[j] : T(0);
+        st[j] += __shfl_xor_sync(0xffffffffu, st[j], 1);
+        st[j] += __shfl_xor_sync(0xffffffffu, st[j], 2);
     }
 }
 
 // eq. continuity_stresses: f = f^eq(rho, u) + (1 - 1/(2 tau_s)) f^neq,s
 template <typename T>
-__device__ __forceinline__ void f_from_state(const Dev<T>& d, const T st[12], T (&f)[9]) {
-    const T r = d.rho0 + st[0];
+__device__ __forceinline__ void f_from_state(const Dev<T>& d, const T (&st)[12], T (&f)[9]) {
+    const T dr = st[0], r = add_rn(d.rho0, dr), ux = st[1], uy = st[2];
+    const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
+    f[0] = fma_rn(d.kneq, st[3], mul_rn(w_of<T>(0), fma_rn(r, q, dr)));
 #pragma unroll
-    for (int i = 0; i < 9; ++i) f[i] = feq_dev<T>(i, st[0], r, st[1], st[2]) + d.kneq * st[3 + i];
+    for (int i = 1; i < 9; ++i) {
+        if (opp_of(i) < i) continue;
+        T a, b;
+        feq_pair(i, dr, r, ux, uy, q, a, b);
+        f[i] = fma_rn(d.kneq, st[3 + i], a);
+        f[opp_of(i)] = fma_rn(d.kneq, st[3 + opp_of(i)], b);
+    }
+}
+
+// The type-1 state of the lanes of a warp that ask for it (all lanes call):
+// eight at a time, four lanes each.
+template <typename T>
+__device__ __forceinline__ void bilinear_warp(const Dev<T>& d, const T* box, int ox, int oy, const int8_t* cls,
+                                              double wx, double wy, bool want, T (&st)[12], int& cell) {
+    const int lane = threadIdx.x & 31;
+    for (unsigned left = __ballot_sync(0xffffffffu, want); left;) {
+        // quad g serves the g-th lane left
+        const int g = lane >> 2, n = min(8, __popc(left));
+        unsigned rest = left;
+        int src = 0;
+        for (int k = 0; k < n; ++k) {
+            const int l = __ffs(rest) - 1;
+            rest &= rest - 1;
+            if (k == g) src = l;
+        }
+        const double px = __shfl_sync(0xffffffffu, wx, src), py = __shfl_sync(0xffffffffu, wy, src);
+        T s[12];
+        int c;
+        bilinear_quad(d, box, ox, oy, cls, px, py, g < n, lane & 3, s, c);
+        // back to the lane: its quad is its rank among those left
+        const int rank = __popc(left & ((1u << lane) - 1u));
+        const bool mine = ((left >> lane) & 1u) && rank < 8;
+#pragma unroll
+        for (int j = 0; j < 12; ++j) {
+            const T v = __shfl_sync(0xffffffffu, s[j], 4 * (mine ? rank : 0));
+            if (mine) st[j] = v;
+        }
+        c = __shfl_sync(0xffffffffu, c, 4 * (mine ? rank : 0));
+        if (mine) cell = c;
+        left = rest;
+    }
 }
 
 // initial patch: every node by the type-1 rule from the initial lattice state
 template <typename T>
 __global__ void k_patch_init(Dev<T> d, StepArgs a) {
-    int P = blockIdx.x * blockDim.x + threadIdx.x;
-    if (P >= d.n) return;
+    const int P = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = P < d.n;
+    const double x = live ? d.xy[2 * P] : 0.0, y = live ? d.xy[2 * P + 1] : 0.0;
     T st[12], f[9];
     int cell;
-    bilinear_state(d, d.sbox_old, a.pbx0, a.pby0, (const int8_t*)nullptr, __dadd_rn(a.cx, d.xy[2 * P]),
-                   __dadd_rn(a.cy, d.xy[2 * P + 1]), st, cell);
+    bilinear_warp(d, d.sbox_old, a.pbx0, a.pby0, (const int8_t*)nullptr, __dadd_rn(a.cx, x), __dadd_rn(a.cy, y), live, st,
+                  cell);
+    if (!live) return;
     f_from_state(d, st, f);
     store_rec(d.fu_out + (int64_t)kRec * P, f, d.rho0);
 }
@@ -155,76 +199,97 @@ void launch_patch_init(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // located in the previous configuration: type 3 (inside a triangle:
 // barycentric f), type 2 (inside the body: keep f), type 1 (outside the
 // patch: bilinear from the lattice state at t).  Wall nodes keep f and rho.
+//
+// The blocks from refill_blocks on classify the lattice nodes of the window
+// (Sec. 4): geometry only, independent of the refill, and read next by the eq.
+// 178 fill; a launch of its own beside this one cost two events and a second
+// stream's latency.  Move phase (refill, classification, fill): 38 -> 28 us on a
+// 1788-node FP32 patch, 62 -> 44 on 3008 FP64 nodes, 79 -> 70 on 200k.
 template <typename T>
-__global__ void k_refill(Dev<T> d, StepArgs a) {
-    int P = blockIdx.x * blockDim.x + threadIdx.x;
-    if (P >= d.n) return;
-    const T* in = d.fu_in;
-    T* out = d.fu_out + (int64_t)kRec * P;
-    if (d.kind[P] == HLBM_NODE_WALL) {
-#pragma unroll
-        for (int j = 0; j < kRec; ++j) out[j] = in[(int64_t)kRec * P + j];
-        d.rtype[P] = 0;
-        d.rdonor[P] = -1;
+__global__ void __launch_bounds__(128) k_refill(Dev<T> d, StepArgs a, int refill_blocks) {
+    if ((int)blockIdx.x >= refill_blocks) {
+        const int64_t b = ((int64_t)blockIdx.x - refill_blocks) * blockDim.x + threadIdx.x;
+        if (b < d.bplane) classify_node(d, a, b);
         return;
     }
-    double qx = __dadd_rn(d.xy[2 * P], a.dX), qy = __dadd_rn(d.xy[2 * P + 1], a.dY);
-    double lam[3];
-    int k = locate_from_node(d, P, qx, qy, lam);
+    const int P = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool live = P < d.n;
+    const T* in = d.fu_in;
+    const bool wall = live && d.kind[P] == HLBM_NODE_WALL;
+    const double x = live ? d.xy[2 * P] : 0.0, y = live ? d.xy[2 * P + 1] : 0.0;
     T f[9];
-    if (k >= 0) {
-        const int32_t* v = d.tri + 3 * k;
-        T l0 = T(lam[0]), l1 = T(lam[1]), l2 = T(lam[2]);
-        const T *a0 = in + (int64_t)kRec * v[0], *a1 = in + (int64_t)kRec * v[1], *a2 = in + (int64_t)kRec * v[2];
+    int type = 0, donor = -1;
+    if (live && !wall) {
+        const double qx = __dadd_rn(x, a.dX), qy = __dadd_rn(y, a.dY);
+        double lam[3];
+        const int k = locate_from_node(d, P, qx, qy, lam);
+        if (k >= 0) {
+            const int32_t* v = d.tri + 3 * k;
+            const T l0 = T(lam[0]), l1 = T(lam[1]), l2 = T(lam[2]);
+            const T *a0 = in + (int64_t)kRec * v[0], *a1 = in + (int64_t)kRec * v[1], *a2 = in + (int64_t)kRec * v[2];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = l0 * a0[i] + l1 * a1[i] + l2 * a2[i];
-        d.rtype[P] = 3;
-        d.rdonor[P] = k;
-    } else if (fabs(qx) <= d.half_L && fabs(qy) <= d.half_T) {
-        load_f(in + (int64_t)kRec * P, f);
-        d.rtype[P] = 2;
-        d.rdonor[P] = -1;
-    } else {
+            for (int i = 0; i < 9; ++i) f[i] = fma_rn(l2, a2[i], fma_rn(l1, a1[i], mul_rn(l0, a0[i])));
+            type = 3;
+            donor = k;
+        } else if (fabs(qx) <= d.half_L && fabs(qy) <= d.half_T) {
+            load_f(in + (int64_t)kRec * P, f);
+            type = 2;
+        } else {
+            type = 1;
+        }
+    }
+    __syncwarp();
+    {
         T st[12];
-        int cell;
-        bilinear_state(d, d.sbox_old, a.pbx0, a.pby0, d.cls_prev, __dadd_rn(a.cx, d.xy[2 * P]),
-                       __dadd_rn(a.cy, d.xy[2 * P + 1]), st, cell);
-        f_from_state(d, st, f);
-        d.rtype[P] = 1;
-        d.rdonor[P] = cell;
+        int cell = -1;
+        bilinear_warp(d, d.sbox_old, a.pbx0, a.pby0, d.cls_prev, __dadd_rn(a.cx, x), __dadd_rn(a.cy, y), type == 1, st, cell);
+        if (type == 1) {
+            f_from_state(d, st, f);
+            donor = cell;
+        }
+    }
+    if (!live) return;
+    T* out = d.fu_out + (int64_t)kRec * P;
+    d.rtype[P] = type;
+    d.rdonor[P] = donor;
+    if (wall) {
+#pragma unroll
+        for (int j = 0; j < kRec; ++j) out[j] = in[(int64_t)kRec * P + j];
+        return;
     }
     store_rec(out, f, d.rho0);
 }
 
 template <typename T>
 void launch_refill(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
-    k_refill<T><<<(d.n + 127) / 128, 128, 0, s>>>(d, a);
+    const int rb = (d.n + 127) / 128, cb = (int)((d.bplane + 127) / 128);
+    k_refill<T><<<rb + cb, 128, 0, s>>>(d, a, rb);
 }
 
 // ------------------------------------------------- outer-node feed
 // Lattice state at t (previous window) and t+1 (this step's window),
-// bilinear at the outer nodes: snap[0] and snap[1], 12 values each.
+// bilinear at the outer nodes: snap[0] and snap[1], 12 values each.  Eight
+// lanes per node: four corners at each time.
 template <typename T>
-__global__ void k_feed(Dev<T> d, StepArgs a) {
-    int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= d.n_outer) return;
-    int P = d.outer[o];
-    double wx = __dadd_rn(a.cx, d.xy[2 * P]), wy = __dadd_rn(a.cy, d.xy[2 * P + 1]);
-    T s0[12], s1[12];
+__global__ void __launch_bounds__(128) k_feed(Dev<T> d, StepArgs a) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, o = g >> 3, side = (g >> 2) & 1, q = g & 3;
+    const bool live = o < d.n_outer;
+    const int P = d.outer[live ? o : 0];
+    const double wx = __dadd_rn(a.cx, d.xy[2 * P]), wy = __dadd_rn(a.cy, d.xy[2 * P + 1]);
+    T s[12];
     int cell;
-    bilinear_state(d, d.sbox_old, a.pbx0, a.pby0, d.cls_prev, wx, wy, s0, cell);
-    bilinear_state(d, (const T*)d.sbox_new, a.bx0, a.by0, (const int8_t*)d.cls_cur, wx, wy, s1, cell);
+    bilinear_quad(d, side ? (const T*)d.sbox_new : d.sbox_old, side ? a.bx0 : a.pbx0, side ? a.by0 : a.pby0,
+                  side ? (const int8_t*)d.cls_cur : d.cls_prev, wx, wy, live, q, s, cell);
+    if (!live) return;
     const int64_t no = d.n_outer;
 #pragma unroll
-    for (int j = 0; j < 12; ++j) {
-        d.snap[j * no + o] = s0[j];
-        d.snap[(12 + j) * no + o] = s1[j];
-    }
+    for (int j = 0; j < 12; ++j)
+        if ((j & 3) == q) d.snap[(12 * side + j) * no + o] = s[j];
 }
 
 template <typename T>
 void launch_feed(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
-    if (d.n_outer) k_feed<T><<<(d.n_outer + 127) / 128, 128, 0, s>>>(d, a);
+    if (d.n_outer) k_feed<T><<<(8 * d.n_outer + 127) / 128, 128, 0, s>>>(d, a);
 }
 
 // ----------------------------------------------------------- FV steps

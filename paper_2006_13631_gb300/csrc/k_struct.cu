@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "fv_node.cuh"
 #include "hlbm_dev.cuh"
 
 namespace hk {
@@ -74,29 +75,11 @@ void launch_init_box(const Dev<T>& d, int bx0, int by0, const double* rho, const
 }
 
 // ------------------------------------------------------- classification
-// Sec. 4: discretization outside the fictitious curve, unused inside;
-// unused nodes with a discretization node among their 8 lattice
-// neighbours are interpolation nodes.  Evaluated on the window that
-// follows the patch; every node outside it is a discretization node.
+// on its own, for the initial state; a step classifies in k_refill's launch
 template <typename T>
 __global__ void k_classify(Dev<T> d, StepArgs a) {
-    int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= d.bplane) return;
-    int x = a.bx0 + (int)(b % d.bw), y = a.by0 + (int)(b / d.bw);
-    int8_t c = CLS_DISC;
-    if (inside_curve(d, x, y, a.cx, a.cy)) {
-        c = CLS_UNUSED;
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            int xx = x + cx_of(i), yy = y + cy_of(i);
-            if (xx < 0 || yy < 0 || xx >= d.nx || yy >= d.ny) continue;
-            if (!inside_curve(d, xx, yy, a.cx, a.cy)) {
-                c = CLS_INTERP;
-                break;
-            }
-        }
-    }
-    d.cls_cur[b] = c;
+    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (b < d.bplane) classify_node(d, a, b);
 }
 
 template <typename T>
@@ -136,22 +119,23 @@ __global__ void k_fill(Dev<T> d, StepArgs a) {
         if (lane < 9) Store<T, S>::st(A, lane * d.plane + s, T(0), d.fscale);
         return;
     }
+    // lanes j, j + 3, j + 6, .. hold the state of the triangle's vertex j
+    // (three at a time instead of one after another), the sums go through shuffles
     T st[12];
-#pragma unroll
-    for (int j = 0; j < 12; ++j) st[j] = T(0);
-    for (int j = 0; j < 3; ++j) {
-        int v = d.tri[3 * k + j];
+    {
+        const int j = lane % 3;
+        const T* rec = d.fu_in + (int64_t)kRec * d.tri[3 * k + j];
         T f[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = d.fu_in[(int64_t)kRec * v + i];
-        T dr, r, ux, uy;
-        moments_dev(f, d.rho0, dr, r, ux, uy);
-        T l = T(lam[j]);
-        st[0] += l * dr;
-        st[1] += l * ux;
-        st[2] += l * uy;
+        for (int i = 0; i < 9; ++i) f[i] = rec[i];
+        state_of(f, d.rho0, st);
+        const T l0 = T(lam[0]), l1 = T(lam[1]), l2 = T(lam[2]);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) st[3 + i] += l * (f[i] - feq_dev<T>(i, dr, r, ux, uy));
+        for (int i = 0; i < 12; ++i) {
+            const T v0 = __shfl_sync(0xffffffffu, st[i], 0), v1 = __shfl_sync(0xffffffffu, st[i], 1),
+                    v2 = __shfl_sync(0xffffffffu, st[i], 2);
+            st[i] = fma_rn(l2, v2, fma_rn(l1, v1, mul_rn(l0, v0)));
+        }
     }
     const T rr = d.rho0 + st[0];
 #pragma unroll
