@@ -464,6 +464,9 @@ bool far_args(hlbm* h, const PendingStep& ps, FarArgs<T>& far) {
     if (!h->overlap || sizeof(T) != 4 || h->dtype != HLBM_F32 || h->fv_kind != HLBM_FV_DEEP || !h->lv.empty() ||
         h->motion.kind == HLBM_MOTION_INDUCED)
         return false;
+    // with two lanes per node the FV blocks have no lattice warps: the SMs
+    // without a tile run the lattice, when they are enough to end before the FV
+    if (d.deep_duo && 4 * (d.deep_sms - h->n_tiles) < d.deep_sms) return false;
     double X, Y;
     motion_pos(h->motion, ps.a.t + 1, &X, &Y);
     int bx0, by0;
@@ -477,7 +480,7 @@ bool far_args(hlbm* h, const PendingStep& ps, FarArgs<T>& far) {
     far.ex1 = h->far_rect[2];
     far.ey1 = h->far_rect[3];
     far.n_seg = (d.nx + 63) / 64;
-    h->far_rows = std::max(1, std::min(d.ny, (int)std::lround(h->overlap_share * d.ny)));
+    h->far_rows = d.deep_duo ? d.ny : std::max(1, std::min(d.ny, (int)std::lround(h->overlap_share * d.ny)));
     far.n_chunks = h->far_rows * far.n_seg;
     far.next = h->far_next;
     return true;
@@ -882,6 +885,8 @@ int build_tiles(hlbm* h, int n_tiles_req, int kind = HLBM_FV_AUTO) {
         d.deep_slot_cap = deep.slot_cap;
         d.deep_ocap = std::max(deep.ocap, 1);
         d.deep_quads = deep_quads;
+        d.deep_duo = deep.comp_cap <= fv_deep_duo_slots<T>();
+        d.deep_sms = sms;
         if (deep.oslot.empty()) deep.oslot.push_back(0);
         d.deep_ptr = (int32_t*)track(upload(h, deep.ptr.data(), deep.ptr.size(), &rc));
         d.deep_cnt = (int32_t*)track(upload(h, deep.cnt.data(), deep.cnt.size(), &rc));

@@ -224,6 +224,8 @@ struct Dev {
     int deep_slot_cap;          // most slots of a tile (own nodes and every ghost layer)
     int deep_ocap;              // most outer nodes among a tile's slots
     int deep_quads;             // FP64: four lanes per node, rows in shared memory for this many computed slots (0: off)
+    int deep_duo;               // FP32: two lanes per node
+    int deep_sms;               // SMs of the device
     const int32_t* deep_ptr;    // [n_tiles + 1]: first slot of each tile in the slot arrays
     const int32_t* deep_cnt;    // [n_tiles][kDeepCnt]: n_a, n_own, n_slot, then the slots computed at block sub-step s
     const int32_t* deep_gid;    // per slot: node id
@@ -649,6 +651,7 @@ constexpr int kTmemMaxEntries = 7;  // off-diagonal entries a row may have in th
 constexpr int kDeepMaxK = 4;  // most sub-steps between exchanges
 constexpr int kDeepCnt = 3 + kDeepMaxK;
 template <typename T> int fv_deep_tmem_slots();          // computed slots a tile may have
+template <typename T> int fv_deep_duo_slots();           // computed slots up to which two lanes share a node (0: never)
 template <typename T> int fv_deep_early();               // own nodes from which a tile updates some ahead
 template <typename T> int fv_deep_row_words();           // words of one row image
 template <typename T> size_t fv_deep_packet_bytes(int n); // exchange packets of n nodes

@@ -8,6 +8,8 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <utility>
+#include <vector>
 
 #include "fv_node.cuh"
 #include "hlbm_dev.cuh"
@@ -1805,7 +1807,191 @@ __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned c
     }
 }
 
-// One chunk of the next lattice step's stream-collide (FarArgs, FP32
+// ---- FP32 pairs of lanes.  With one node per thread the few warps of a small
+// tile have nothing to overlap the update's chain of some 500 instructions
+// with: 1.85 us of a sub-step's 2.3 on a 2588-node patch (63 own nodes per
+// tile), 1.0 / K more for the exchange.  Where a tile's computed slots fit, two
+// lanes share a node: lane 0 holds the pairs A, B (axes) and E, lane 1 C, D
+// (diagonals) and F, each with its share of the row in registers; the sums
+// over directions take one shuffle.  Every value is formed by the expression
+// of fv_node.cuh, so the bits are those of a node per lane.
+constexpr int kDuoThreads = 768;  // 80 registers a thread
+constexpr int kDuoSlots = kDuoThreads / 2;
+struct Duo {
+    int q;                             // lane of the pair
+    Pr<float> w, dt1, iv1, dt2, iv2;  // minus the weights; the update's signed factors
+};
+struct DuoRow {
+    Pr<float> k[kTmemMaxEntries];  // (gx, gy) on lane 0, (gx + gy, gx - gy) on lane 1; 0 past the row's end
+    float c[kTmemMaxEntries];
+    int col[kTmemMaxEntries];
+    float cP;
+};
+__device__ __forceinline__ Pr<float> duo_zero() { return pk(0.0f, 0.0f); }
+__device__ __forceinline__ float duo_other(float v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+// (x, y) on lane 0, (x + y, y - x) on lane 1
+__device__ __forceinline__ Pr<float> duo_axes(const Duo& Q, float x, float y) {
+    return pk(Q.q ? add_rn(x, y) : x, Q.q ? sub_rn(y, x) : y);
+}
+// moments of the set whose pairs (a, b) each lane holds, f0 in lane 0's e
+__device__ __forceinline__ void duo_moments(const Duo& Q, Pr<float> a, Pr<float> b, float e, float& m0, float& mx,
+                                            float& my) {
+    const Pr<float> s = padd(a, b), dd = psub(a, b);
+    const float t = add_rn(px(s), py(s));
+    const float vx = Q.q ? sub_rn(px(dd), py(dd)) : px(dd), vy = Q.q ? add_rn(px(dd), py(dd)) : py(dd);
+    const float f0 = __shfl_sync(0xffffffffu, e, 0, 2), t2 = duo_other(t), wx = duo_other(vx), wy = duo_other(vy);
+    m0 = add_rn(f0, add_rn(t, t2));
+    mx = add_rn(vx, wx);
+    my = add_rn(vy, wy);
+}
+// the pairs minus w (G +- 3 c . (x, y))
+__device__ __forceinline__ void duo_sub_lin(const Duo& Q, Pr<float> G, float x, float y, Pr<float>& a, Pr<float>& b) {
+    const Pr<float> H = pmul(pk(3.0f, 3.0f), duo_axes(Q, x, y));
+    a = pfma(Q.w, padd(G, H), a);
+    b = pfma(Q.w, psub(G, H), b);
+}
+
+template <bool kRecord, bool kOuterFv>
+__device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned char* sm, const DeepSmem& L,
+                                         const float* cur, float* nxt, const Duo& Q, const DuoRow& R, bool valid, int x,
+                                         int m, unsigned char* pkt, unsigned tag, bool own_slot, const float* star) {
+    const int q = Q.q, ia = 4 * q, ie = 8 + 2 * q;
+    const int8_t* kd = reinterpret_cast<const int8_t*>(sm + L.kind);
+    const int16_t* om = reinterpret_cast<const int16_t*>(sm + L.omap);
+    const int8_t kind = valid ? kd[x] : (int8_t)HLBM_NODE_OUTER;
+    const bool outer = kind == HLBM_NODE_OUTER;
+    const bool row = kOuterFv ? valid : !outer;
+    auto pairs = [&](const float* p, Pr<float>& a, Pr<float>& b, Pr<float>& e) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + ia);
+        a.v = v.x;
+        b.v = v.y;
+        e.v = *reinterpret_cast<const unsigned long long*>(p + ie);
+    };
+    float* rec = nullptr;
+    if constexpr (kRecord) {
+        if (valid && own_slot) rec = d.fv_rec + ((int64_t)m * d.n + reinterpret_cast<const int32_t*>(sm + L.gid)[x]) * kAdjRec;
+    }
+    Pr<float> a = duo_zero(), b = a, e = a;
+    if (__any_sync(0xffffffffu, row)) {
+        const float* own = cur + (size_t)kSR * (valid ? x : 0);
+        if (kOuterFv && outer && valid) own = star + (size_t)kSR * om[x];
+        Pr<float> Pa, Pb, Pe, Sa = a, Sb = a, Ca = a, Cb = a, Ce = a;
+        pairs(own, Pa, Pb, Pe);
+#pragma unroll
+        for (int j = 0; j < kTmemMaxEntries; ++j) {
+            const float* r = cur + (size_t)kSR * R.col[j];
+            if (kOuterFv && outer && kd[R.col[j]] == HLBM_NODE_OUTER) r = star + (size_t)kSR * om[R.col[j]];
+            Pr<float> fa, fb, fe;
+            pairs(r, fa, fb, fe);
+            const Pr<float> cc = pk(R.c[j], R.c[j]);
+            Sa = pfma(R.k[j], psub(fa, Pa), Sa);
+            Sb = pfma(R.k[j], psub(fb, Pb), Sb);
+            Ca = pfma(cc, fa, Ca);
+            Cb = pfma(cc, fb, Cb);
+            Ce = pfma(cc, fe, Ce);
+        }
+        const Pr<float> cP = pk(R.cP, R.cP);
+        Ca = pfma(cP, Pa, Ca);
+        Cb = pfma(cP, Pb, Cb);
+        Ce = pfma(cP, Pe, Ce);
+        // collision sums: lane 0 has (Cf_0, Z0), lane 1 (Z1, Z2)
+        float dr, jx, jy, n0 = px(Ce);
+        duo_moments(Q, Ca, Cb, n0, dr, jx, jy);
+        const float zo = py(Ce), zx = duo_other(zo), Z0 = q ? zx : zo, Z2 = q ? zo : zx;
+        const float zs = add_rn(Z0, Z2), q0 = fma_rn(-1.5f, zs, dr);
+        const Pr<float> u = pk(q ? fma_rn(2.0f, px(Ce), zs) : Z0, q ? fma_rn(-2.0f, px(Ce), zs) : Z2);
+        duo_sub_lin(Q, pfma(pk(4.5f, 4.5f), u, pk(q0, q0)), jx, jy, Ca, Cb);
+        n0 = fma_rn(-w_of<float>(0), q0, n0);
+        float m0, mx, my;
+        duo_moments(Q, Ca, Cb, n0, m0, mx, my);
+        duo_sub_lin(Q, pk(m0, m0), mx, my, Ca, Cb);
+        n0 = fma_rn(-w_of<float>(0), m0, n0);
+        a = pfma(Q.dt1, pfma(Q.iv1, Ca, Sa), Pa);
+        b = pfma(Q.dt2, pfma(Q.iv2, Cb, Sb), Pb);
+        float f0 = fma_rn(d.dt_u, mul_rn(-d.inv_tau_u, n0), px(Pe));
+        const bool wall = kind == HLBM_NODE_WALL;
+        if constexpr (kRecord) {
+            if (rec && row) {
+                *reinterpret_cast<ulonglong2*>(rec + ia) = make_ulonglong2(Ca.v, Cb.v);
+                if (q == 0) rec[kAdjN0] = n0;
+            }
+        }
+        if (__any_sync(0xffffffffu, wall)) {
+            const float* uv = reinterpret_cast<const float*>(sm + L.uv);
+            const float U = uv[m], V = uv[d.n_sub + m];
+            duo_moments(Q, a, b, f0, dr, jx, jy);
+            const float rho = add_rn(d.rho0, dr), inv = 1.0f / rho;
+            const float ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
+            const float dx = sub_rn(U, ux), dy = sub_rn(V, uy), sx = add_rn(U, ux), sy = add_rn(V, uy);
+            const float bb = mul_rn(-1.5f, fma_rn(dx, sx, mul_rn(dy, sy)));
+            const Pr<float> dv = duo_axes(Q, dx, dy);
+            const Pr<float> G = pfma(pmul(pk(4.5f, 4.5f), dv), duo_axes(Q, sx, sy), pk(bb, bb)), H = pmul(pk(3.0f, 3.0f), dv);
+            const float wr = mul_rn(q ? w_of<float>(5) : w_of<float>(1), rho);
+            if constexpr (kRecord) {
+                if (rec && wall) {
+                    if (q == 0) rec[kAdjWall] = rho;
+                    rec[kAdjWall + 1 + q] = q ? uy : ux;
+                }
+            }
+            if (wall) {
+                a = pfma(pk(wr, wr), padd(G, H), a);
+                b = pfma(pk(wr, wr), psub(G, H), b);
+                f0 = fma_rn(mul_rn(w_of<float>(0), rho), bb, f0);
+            }
+        }
+        e = pk(f0, 0.0f);
+    }
+    if (valid && !row) {
+        const float* sn = reinterpret_cast<const float*>(sm + L.osnap) + kSnap * om[x];
+        const float th = float(m + 1) / float(d.n_sub), t0 = sub_rn(1.0f, th);
+        auto at = [&](int j) { return fma_rn(t0, sn[j], mul_rn(th, sn[12 + j])); };
+        const float dr = at(0), ux = at(1), uy = at(2), rho = add_rn(d.rho0, dr);
+        const float qq = mul_rn(-1.5f, fma_rn(ux, ux, mul_rn(uy, uy)));
+        const Pr<float> c = duo_axes(Q, ux, uy), rr = pk(rho, rho), kk = pk(d.kneq, d.kneq);
+        const float wl = q ? w_of<float>(5) : w_of<float>(1);
+        const Pr<float> w = pk(wl, wl);
+        const Pr<float> G = pfma(rr, pfma(pmul(pk(4.5f, 4.5f), c), c, pk(qq, qq)), pk(dr, dr)),
+                        H = pmul(rr, pmul(pk(3.0f, 3.0f), c));
+        a = pfma(kk, pk(at(4 + ia), at(5 + ia)), pmul(w, padd(G, H)));
+        b = pfma(kk, pk(at(6 + ia), at(7 + ia)), pmul(w, psub(G, H)));
+        e = pk(fma_rn(d.kneq, at(3), mul_rn(w_of<float>(0), fma_rn(rho, qq, dr))), 0.0f);
+    }
+    __syncwarp();
+    float dr, jx, jy;
+    duo_moments(Q, a, b, px(e), dr, jx, jy);
+    const float inv = 1.0f / add_rn(d.rho0, dr), ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
+    e = q ? pk(mul_rn(jx, uy), mul_rn(jy, uy)) : pk(px(e), mul_rn(jx, ux));
+    if constexpr (kRecord) {
+        if (rec && m + 1 < d.n_sub) rec[(int64_t)d.n * kAdjRec + kAdjU + q] = q ? uy : ux;
+    }
+    if (!valid) return;
+    float* o = nxt + (size_t)kSR * x;
+    *reinterpret_cast<ulonglong2*>(o + ia) = make_ulonglong2(a.v, b.v);
+    *reinterpret_cast<unsigned long long*>(o + ie) = e.v;
+    if (pkt) {  // packets 2 q, 2 q + 1: (a, b.x), (b.y, e)
+        const unsigned long long t = (unsigned long long)tag << 32;
+        auto w = [](float v) { return (unsigned long long)__float_as_uint(v); };
+        st_packet(pkt + 32 * q, a.v, t | w(px(b)));
+        st_packet(pkt + 32 * q + 16, w(py(b)) | (w(px(e)) << 32), t | w(py(e)));
+    }
+}
+__device__ __forceinline__ void take_packet_duo(float* dst, int c, const Packet& k) {
+    const int q = c >> 1;
+    const float v0 = __uint_as_float((unsigned)k.lo), v1 = __uint_as_float((unsigned)(k.lo >> 32)),
+                v2 = __uint_as_float((unsigned)k.hi);
+    if (c & 1) {
+        dst[4 * q + 3] = v0;
+        dst[8 + 2 * q] = v1;
+        dst[9 + 2 * q] = v2;
+    } else {
+        dst[4 * q] = v0;
+        dst[4 * q + 1] = v1;
+        dst[4 * q + 2] = v2;
+    }
+}
+
+// One chunk of the next lattice step's stream-collide (FarArgs, FP32'''
+
 // storage) on the lattice warps: row y = c / n_seg, nodes [64 seg,
 // 64 seg + 64), two per lane.  The pull and BGK arithmetic of a node is that
 // of k_stream_collide (the same pulled values through bgk_dev; edge nodes
@@ -1867,6 +2053,18 @@ __device__ __forceinline__ void far_chunk(const Dev<float>& d, const FarArgs<flo
     }
 }
 
+// lattice warps: chunks of the next step's stream-collide until none is left
+__device__ __forceinline__ void far_chunks(const Dev<float>& d, const FarArgs<float>& far) {
+    const int lane = threadIdx.x & 31;
+    for (; far.n_chunks > 0;) {
+        int c = 0;
+        if (lane == 0) c = (int)atomicAdd(far.next, 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= far.n_chunks) break;
+        far_chunk(d, far, c, lane);
+    }
+}
+
 // the FV warps' barrier (named barrier 1; the lattice warps never join it)
 template <int N>
 __device__ __forceinline__ void fv_bar() {
@@ -1878,7 +2076,7 @@ __device__ __forceinline__ void fv_bar() {
 // fewest nodes) takes packets k, k + N, ...  Each is polled until its tag is
 // the exchange's, a bounded number of times; false when a wait ran out or
 // another tile gave up.
-template <typename T, int N>
+template <typename T, int N, bool kDuo>
 __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned char* xb, const int32_t* gid, T* cur,
                                              int n_own, int n_slot, unsigned tag, int k) {
     constexpr int PK = kPkts<T>;
@@ -1903,7 +2101,10 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
             }
             v = ld_packet(src);
         }
-        take_packet(cur + (size_t)kSR * sl, c, v);
+        if constexpr (kDuo)
+            take_packet_duo(cur + (size_t)kSR * sl, c, v);
+        else
+            take_packet(cur + (size_t)kSR * sl, c, v);
     }
     return ok;
 }
@@ -1911,11 +2112,13 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
 // The FV sub-steps of tile `tile` of the solver d (one block); k_fv_deep runs
 // one solver, k_fv_deep_pack several.  kRecord: also writes what the reverse
 // mode needs of every sub-step (Dev::fv_rec).
-template <typename T, bool kRecord, bool kOuterFv>
+// kDuo (FP32): two lanes per node, no tensor memory, no lattice warps.
+template <typename T, bool kRecord, bool kOuterFv, bool kDuo>
 __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a, T* g0, T* g1, const FarArgs<T>& far,
                                              const int tile, unsigned char* sm, int& abort_sh,
                                              uint32_t& tmem_base_sh) {
-    constexpr int NT = kDeepFv<T>, BT = kDeepThreads<T>, G = kDeepGroups<T>, SW = kDeepSlotWords<T>;
+    constexpr int NT = kDuo ? kDuoThreads : kDeepFv<T>, BT = kDuo ? kDuoThreads : kDeepThreads<T>;
+    constexpr int G = kDeepGroups<T>, SW = kDeepSlotWords<T>;
     const int tid = threadIdx.x, warp = tid >> 5;
     const int s0 = d.deep_ptr[tile];
     const int32_t* cnt = d.deep_cnt + kDeepCnt * tile;
@@ -1933,16 +2136,30 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
     int16_t* om = reinterpret_cast<int16_t*>(sm + L.omap);
     // ---- tensor memory: all 512 columns; warp w reads lanes 32 (w % 4) ..
     // and, for its slot group j, the columns SW (j NT / 128 + w / 4) ..
-    if (warp == 0) tmem_alloc_512(&tmem_base_sh);
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
-    const uint32_t tbase = tmem_base_sh;
+    uint32_t tbase = 0;
+    if constexpr (!kDuo) {
+        if (warp == 0) tmem_alloc_512(&tmem_base_sh);
+        tmem_fence_before();
+        __syncthreads();
+        tmem_fence_after();
+        tbase = tmem_base_sh;
+    }
     auto tslot_of = [&](int j) {
         return tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(SW * (j * (NT / 128) + (warp >> 2)));
     };
     // ---- set-up: wall velocity per sub-step, slot tables, records of every
     // slot at sub-step 0, the outer nodes' feed, the row images
+    [[maybe_unused]] DuoRow R;
+    [[maybe_unused]] Duo Q2;
+    if constexpr (kDuo) {
+        Q2.q = tid & 1;
+        const float w = Q2.q ? -w_of<float>(5) : -w_of<float>(1), dt = d.dt_u, iv = d.inv_tau_u;
+        Q2.w = pk(w, w);
+        Q2.dt1 = pk(dt, Q2.q ? -dt : dt);
+        Q2.iv1 = pk(-iv, Q2.q ? iv : -iv);
+        Q2.dt2 = pk(-dt, Q2.q ? dt : -dt);
+        Q2.iv2 = pk(iv, Q2.q ? -iv : iv);
+    }
     for (int m = tid; m < d.n_sub; m += BT) wall_velocity(d, a, m, uv[m], uv[d.n_sub + m]);
     for (int x = tid; x < n_slot; x += BT) {
         const int g = d.deep_gid[s0 + x];
@@ -1993,8 +2210,24 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                 }
             }
         }
+        if constexpr (kDuo) {
+            // pairs of lanes: this lane's share of its row, in registers
+            const int x = tid >> 1;
+            const bool have = x < n_comp;
+            const uint4 h = have ? rows[(int64_t)(SW / 4) * x] : make_uint4(0u, 0u, 0u, 0u);
+            R.cP = __uint_as_float(h.x);
+#pragma unroll
+            for (int j = 0; j < kTmemMaxEntries; ++j) {
+                const bool in_row = have && j < (int)h.y;
+                const uint4 u = in_row ? rows[(int64_t)(SW / 4) * x + 1 + j] : make_uint4(0u, 0u, 0u, 0u);
+                const float gx = __uint_as_float(u.x), gy = __uint_as_float(u.y);
+                R.k[j] = Q2.q ? pk(add_rn(gx, gy), sub_rn(gx, gy)) : pk(gx, gy);
+                R.c[j] = __uint_as_float(u.z);
+                R.col[j] = in_row ? (int)u.w : (have ? x : 0);
+            }
+        }
 #pragma unroll 1
-        for (int j = 0; j < G && tid < NT && !quads; ++j) {
+        for (int j = 0; j < G && tid < NT && !quads && !kDuo; ++j) {
             const int x = j * NT + tid;
             const bool have = x < n_comp;
             const uint32_t ts = tslot_of(j);
@@ -2005,7 +2238,7 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                 tmem_st4(ts + 4 * w4, u.x, u.y, u.z, u.w);
             }
         }
-        tmem_wait_st();
+        if constexpr (!kDuo) tmem_wait_st();
     }
     // interpolated records of the outer slots for sub-step m (outer_fv), thread k of n
     const int n_star = kOuterFv ? d.deep_optr[tile + 1] - d.deep_optr[tile] : 0;
@@ -2023,16 +2256,16 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
         make_stars(0, tid, BT);
     }
     if (tid == 0) abort_sh = 0;
-    tmem_fence_before();
+    if constexpr (!kDuo) tmem_fence_before();
     __syncthreads();
-    tmem_fence_after();
+    if constexpr (!kDuo) tmem_fence_after();
     const unsigned long long base = (unsigned long long)a.t * (unsigned long long)d.n_sub;
     if (tid < NT) {
         const int nb0 = d.tile_nb_ptr[tile], nb1 = d.tile_nb_ptr[tile + 1];
         const int64_t xhalf = (int64_t)d.n * kPkts<T> * 16;
         // own nodes that read only own nodes, updated while the ghosts are on
         // their way (0 where that does not pay: fv_deep_early)
-        const int n_early = quads ? 0 : n_a;
+        const int n_early = quads || kDuo ? 0 : n_a;
         Quad Q;
         Q.q = tid & 3;
         Q.w = w_of<double>(Q.q < 2 ? 1 : 5);
@@ -2055,14 +2288,16 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                 if (kOuterFv && m + 1 < d.n_sub) make_stars(m + 1, NT - 1 - tid, NT);
                 if (s == 0 && b > 0) {
 #pragma unroll
-                    for (int j = 0; j < G; ++j) {
+                    for (int j = 0; j < G && !kDuo; ++j) {
                         const int x = j * NT + tid;
                         const bool v = x < n_early;
-                        if (__any_sync(0xffffffffu, v))
-                            deep_node<T, kRecord, kOuterFv>(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u, true,
-                                                            star_at(m));
+                        if constexpr (!kDuo) {
+                            if (__any_sync(0xffffffffu, v))
+                                deep_node<T, kRecord, kOuterFv>(d, sm, L, cur, nxt, tslot_of(j), v, x, m, nullptr, 0u,
+                                                                true, star_at(m));
+                        }
                     }
-                    bool ok = deep_receive<T, NT>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
+                    bool ok = deep_receive<T, NT, kDuo>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
                                                   a.xtag + (unsigned)b, NT - 1 - tid);
                     // tiles that read this one but are not read by it: their reads of
                     // the packets about to be overwritten are behind their counter
@@ -2107,15 +2342,26 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                             x < n_own);
                     }
                 }
-#pragma unroll
-                for (int j = 0; j < G && !quads; ++j) {
-                    const int x = j * NT + tid;
-                    const bool v = x >= lo && x < cs;
+                if constexpr (kDuo) {
+                    const int x = tid >> 1;
+                    const bool v = x < cs;
                     if (__any_sync(0xffffffffu, v))
-                        deep_node<T, kRecord, kOuterFv>(
-                            d, sm, L, cur, nxt, tslot_of(j), v, x, m,
+                        duo_node<kRecord, kOuterFv>(
+                            d, sm, L, cur, nxt, Q2, R, v, x, m,
                             send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out,
                             x < n_own, star_at(m));
+                }
+#pragma unroll
+                for (int j = 0; j < G && !quads && !kDuo; ++j) {
+                    const int x = j * NT + tid;
+                    const bool v = x >= lo && x < cs;
+                    if constexpr (!kDuo) {
+                        if (__any_sync(0xffffffffu, v))
+                            deep_node<T, kRecord, kOuterFv>(
+                                d, sm, L, cur, nxt, tslot_of(j), v, x, m,
+                                send && v && x < n_own && sd[x] ? xout + (int64_t)gid[x] * kPkts<T> * 16 : nullptr, tag_out,
+                                x < n_own, star_at(m));
+                    }
                 }
                 fv_bar<NT>();
             }
@@ -2133,21 +2379,15 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
             st4(o + 8, v1.w, v2.y, v2.z, v2.w);
         }
     } else if constexpr (sizeof(T) == 4) {
-        // lattice warps: chunks of the next step's stream-collide until none is left
-        const int lane = tid & 31;
-        for (; far.n_chunks > 0;) {
-            int c = 0;
-            if (lane == 0) c = (int)atomicAdd(far.next, 1u);
-            c = __shfl_sync(0xffffffffu, c, 0);
-            if (c >= far.n_chunks) break;
-            far_chunk(d, far, c, lane);
-        }
+        far_chunks(d, far);
     }
     // ---- release TMEM (also after an abort: every warp is past its last tcgen05.ld)
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
-    if (warp == 0) tmem_dealloc_512(tbase);
+    if constexpr (!kDuo) {
+        tmem_fence_before();
+        __syncthreads();
+        tmem_fence_after();
+        if (warp == 0) tmem_dealloc_512(tbase);
+    }
 }
 
 template <typename T, bool kRecord, bool kOuterFv>
@@ -2155,7 +2395,7 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int abort_sh;
     __shared__ uint32_t tmem_base_sh;
-    fv_deep_body<T, kRecord, kOuterFv>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, tmem_base_sh);
+    fv_deep_body<T, kRecord, kOuterFv, false>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, tmem_base_sh);
 }
 
 // Several solvers' FV sub-steps in one cooperative launch: block b runs tile
@@ -2169,16 +2409,53 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep_pack(const __gri
     __shared__ uint32_t tmem_base_sh;
     int i = 0;
     while (i + 1 < pk.n && pk.block0[i + 1] <= (int)blockIdx.x) ++i;
-    fv_deep_body<T, false, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<T>{}, (int)blockIdx.x - pk.block0[i], sm,
+    fv_deep_body<T, false, false, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<T>{}, (int)blockIdx.x - pk.block0[i], sm,
                            abort_sh, tmem_base_sh);
+}
+
+// FP32 patches whose tiles' computed slots fit pairs of lanes.  Blocks past
+// the tiles run the next step's stream-collide away from the patch (FarArgs) on
+// all their warps.
+template <bool kRecord, bool kOuterFv>
+__global__ void __launch_bounds__(kDuoThreads, 1) k_fv_duo(Dev<float> d, StepArgs a, float* g0, float* g1,
+                                                           FarArgs<float> far) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int abort_sh;
+    uint32_t none = 0;
+    if ((int)blockIdx.x >= d.n_tiles)
+        far_chunks(d, far);
+    else
+        fv_deep_body<float, kRecord, kOuterFv, true>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, none);
+}
+__global__ void __launch_bounds__(kDuoThreads, 1) k_fv_duo_pack(const __grid_constant__ FvPack<float> pk) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int abort_sh;
+    uint32_t none = 0;
+    int i = 0;
+    while (i + 1 < pk.n && pk.block0[i + 1] <= (int)blockIdx.x) ++i;
+    fv_deep_body<float, false, false, true>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<float>{},
+                                            (int)blockIdx.x - pk.block0[i], sm, abort_sh, none);
 }
 
 template <typename T>
 cudaError_t launch_fv_deep_pack(const FvPack<T>& pk, int blocks, size_t smem, cudaStream_t s) {
     FvPack<T> p = pk;
     void* args[] = {&p};
-    return cudaLaunchCooperativeKernel((const void*)k_fv_deep_pack<T>, dim3(blocks), dim3(kDeepThreads<T>), args, smem,
-                                       s);
+    const void* fn = (const void*)k_fv_deep_pack<T>;
+    int threads = kDeepThreads<T>;
+    if constexpr (sizeof(T) == 4) {
+        bool duo = true;
+        for (int k = 0; k < pk.n; ++k) duo = duo && pk.d[k].deep_duo;
+        if (duo) {
+            fn = (const void*)k_fv_duo_pack;
+            threads = kDuoThreads;
+        }
+    }
+    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(threads), args, smem, s);
+}
+template <typename T>
+int fv_deep_duo_slots() {
+    return sizeof(T) == 4 ? kDuoSlots : 0;
 }
 
 template <typename T>
@@ -2189,8 +2466,15 @@ int fv_deep_tile_capacity(size_t smem) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // each block allocates all 512 TMEM columns: only one block per SM
+    std::vector<std::pair<const void*, int>> fns;
     for (const void* fn : {(const void*)k_fv_deep<T, false, false>, (const void*)k_fv_deep<T, true, false>,
-                           (const void*)k_fv_deep<T, false, true>, (const void*)k_fv_deep_pack<T>}) {
+                           (const void*)k_fv_deep<T, false, true>, (const void*)k_fv_deep_pack<T>})
+        fns.push_back({fn, kDeepThreads<T>});
+    if constexpr (sizeof(T) == 4)
+        for (const void* fn : {(const void*)k_fv_duo<false, false>, (const void*)k_fv_duo<true, false>,
+                               (const void*)k_fv_duo<false, true>, (const void*)k_fv_duo_pack})
+            fns.push_back({fn, kDuoThreads});
+    for (const auto& [fn, threads] : fns) {
         cudaFuncAttributes fa{};
         if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
             cudaGetLastError();
@@ -2202,7 +2486,7 @@ int fv_deep_tile_capacity(size_t smem) {
             cudaGetLastError();
             return 0;
         }
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kDeepThreads<T>, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem);
         if (per != 1) return 0;
     }
     return sms;
@@ -2222,7 +2506,17 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
     const void* fn = d.outer_fv ? (const void*)k_fv_deep<T, false, true>
                      : d.fv_rec ? (const void*)k_fv_deep<T, true, false>
                                 : (const void*)k_fv_deep<T, false, false>;
-    return cudaLaunchCooperativeKernel(fn, dim3(d.n_tiles), dim3(kDeepThreads<T>), args, smem, s);
+    int threads = kDeepThreads<T>, blocks = d.n_tiles;
+    if constexpr (sizeof(T) == 4) {
+        if (d.deep_duo) {
+            fn = d.outer_fv ? (const void*)k_fv_duo<false, true>
+                 : d.fv_rec ? (const void*)k_fv_duo<true, false>
+                            : (const void*)k_fv_duo<false, false>;
+            threads = kDuoThreads;
+            if (fa.n_chunks > 0) blocks = std::max(blocks, d.deep_sms);  // the other SMs run the lattice
+        }
+    }
+    return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(threads), args, smem, s);
 }
 
 // Row image of computed slot i: header (C_PP, entry count), then the
@@ -3500,6 +3794,7 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template cudaError_t launch_fv_tmem<T>(const Dev<T>&, const StepArgs&, cudaStream_t);                     \
     template cudaError_t launch_fv_tmem_pack<T>(const FvPack<T>&, int, size_t, cudaStream_t);                 \
     template int fv_deep_tmem_slots<T>();                                                                     \
+    template int fv_deep_duo_slots<T>();                                                                      \
     template int fv_deep_early<T>();                                                                          \
     template int fv_deep_row_words<T>();                                                                      \
     template size_t fv_deep_packet_bytes<T>(int);                                                             \
