@@ -838,7 +838,9 @@ int build_tiles(hlbm* h, int n_tiles_req, int kind = HLBM_FV_AUTO) {
         for (int K = depth; K >= 1 && !deep_ok; --K) {
             if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), fv_deep_early<T>(), deep)) continue;
             // FP64, few computed slots: four lanes per node
-            const int ocap1 = std::max(deep.ocap, 1);
+            deep.slot_cap = fv_deep_cap<T>(deep.slot_cap);
+            deep.ocap = fv_deep_cap<T>(std::max(deep.ocap, 1));
+            const int ocap1 = deep.ocap;
             deep_quads = sizeof(T) == 8 && h->patch.outer_fv == 0 && deep.comp_cap <= kDeepQuadMax ? deep.comp_cap : 0;
             deep_ok = deep.slot_cap < 65536 &&
                       fv_deep_tile_capacity<T>(fv_deep_smem_bytes<T>(deep.slot_cap, h->patch.n_sub, ocap1, deep_quads,

@@ -651,6 +651,7 @@ constexpr int kTmemMaxEntries = 7;  // off-diagonal entries a row may have in th
 constexpr int kDeepMaxK = 4;  // most sub-steps between exchanges
 constexpr int kDeepCnt = 3 + kDeepMaxK;
 template <typename T> int fv_deep_tmem_slots();          // computed slots a tile may have
+template <typename T> int fv_deep_cap(int n);            // slots to lay out for n
 template <typename T> int fv_deep_duo_slots();           // computed slots up to which two lanes share a node (0: never)
 template <typename T> int fv_deep_early();               // own nodes from which a tile updates some ahead
 template <typename T> int fv_deep_row_words();           // words of one row image

@@ -1824,9 +1824,21 @@ struct Duo {
 struct DuoRow {
     Pr<float> k[kTmemMaxEntries];  // (gx, gy) on lane 0, (gx + gy, gx - gy) on lane 1; 0 past the row's end
     float c[kTmemMaxEntries];
-    int col[kTmemMaxEntries];
+    int col[kTmemMaxEntries];      // 4 times the slot
     float cP;
 };
+// Records of cap slots: the pairs A, B of every slot, then C, D, then E, F (cap
+// is 4 modulo 8, so that the two lanes of four neighbouring slots read eight
+// different bank quads; records of 48 bytes gave two-way conflicts: 52 % of the
+// shared-memory cycles of the 45k-node patch's sub-steps)
+__host__ __device__ constexpr int duo_cap(int n) { return (n + 3) / 8 * 8 + 4; }
+__device__ __forceinline__ int duo_ab(int cap, int q) { return 4 * q * cap; }
+__device__ __forceinline__ int duo_ef(int cap, int q) { return 8 * cap + 2 * q; }
+__device__ __forceinline__ void duo_put(float* buf, int cap, int x, const RecP<float>& r) {
+    *reinterpret_cast<ulonglong2*>(buf + 4 * x) = make_ulonglong2(r.A.v, r.B.v);
+    *reinterpret_cast<ulonglong2*>(buf + 4 * cap + 4 * x) = make_ulonglong2(r.C.v, r.D.v);
+    *reinterpret_cast<ulonglong2*>(buf + 8 * cap + 4 * x) = make_ulonglong2(r.E.v, r.F.v);
+}
 __device__ __forceinline__ Pr<float> duo_zero() { return pk(0.0f, 0.0f); }
 __device__ __forceinline__ float duo_other(float v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
 // (x, y) on lane 0, (x + y, y - x) on lane 1
@@ -1855,17 +1867,18 @@ template <bool kRecord, bool kOuterFv>
 __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned char* sm, const DeepSmem& L,
                                          const float* cur, float* nxt, const Duo& Q, const DuoRow& R, bool valid, int x,
                                          int m, unsigned char* pkt, unsigned tag, bool own_slot, const float* star) {
-    const int q = Q.q, ia = 4 * q, ie = 8 + 2 * q;
+    const int q = Q.q, ia = 4 * q;
     const int8_t* kd = reinterpret_cast<const int8_t*>(sm + L.kind);
     const int16_t* om = reinterpret_cast<const int16_t*>(sm + L.omap);
     const int8_t kind = valid ? kd[x] : (int8_t)HLBM_NODE_OUTER;
     const bool outer = kind == HLBM_NODE_OUTER;
     const bool row = kOuterFv ? valid : !outer;
-    auto pairs = [&](const float* p, Pr<float>& a, Pr<float>& b, Pr<float>& e) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p + ia);
+    const int cap = d.deep_slot_cap;
+    auto pairs = [&](const float* ab, const float* ef, Pr<float>& a, Pr<float>& b, Pr<float>& e) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(ab);
         a.v = v.x;
         b.v = v.y;
-        e.v = *reinterpret_cast<const unsigned long long*>(p + ie);
+        e.v = *reinterpret_cast<const unsigned long long*>(ef);
     };
     float* rec = nullptr;
     if constexpr (kRecord) {
@@ -1873,16 +1886,25 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
     }
     Pr<float> a = duo_zero(), b = a, e = a;
     if (__any_sync(0xffffffffu, row)) {
-        const float* own = cur + (size_t)kSR * (valid ? x : 0);
-        if (kOuterFv && outer && valid) own = star + (size_t)kSR * om[x];
+        const float *ab = cur + duo_ab(cap, q), *ef = cur + duo_ef(cap, q);
+        const float *sab = nullptr, *sef = nullptr;  // interpolated records (outer_fv)
+        const int own = 4 * (valid ? x : 0);
         Pr<float> Pa, Pb, Pe, Sa = a, Sb = a, Ca = a, Cb = a, Ce = a;
-        pairs(own, Pa, Pb, Pe);
+        if (kOuterFv && outer && valid) {
+            sab = star + duo_ab(d.deep_ocap, q), sef = star + duo_ef(d.deep_ocap, q);
+            pairs(sab + 4 * om[x], sef + 4 * om[x], Pa, Pb, Pe);
+        } else {
+            pairs(ab + own, ef + own, Pa, Pb, Pe);
+        }
 #pragma unroll
         for (int j = 0; j < kTmemMaxEntries; ++j) {
-            const float* r = cur + (size_t)kSR * R.col[j];
-            if (kOuterFv && outer && kd[R.col[j]] == HLBM_NODE_OUTER) r = star + (size_t)kSR * om[R.col[j]];
             Pr<float> fa, fb, fe;
-            pairs(r, fa, fb, fe);
+            if (kOuterFv && outer && valid && kd[R.col[j] >> 2] == HLBM_NODE_OUTER) {
+                const int o = 4 * om[R.col[j] >> 2];
+                pairs(sab + o, sef + o, fa, fb, fe);
+            } else {
+                pairs(ab + R.col[j], ef + R.col[j], fa, fb, fe);
+            }
             const Pr<float> cc = pk(R.c[j], R.c[j]);
             Sa = pfma(R.k[j], psub(fa, Pa), Sa);
             Sb = pfma(R.k[j], psub(fb, Pb), Sb);
@@ -1965,9 +1987,8 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
         if (rec && m + 1 < d.n_sub) rec[(int64_t)d.n * kAdjRec + kAdjU + q] = q ? uy : ux;
     }
     if (!valid) return;
-    float* o = nxt + (size_t)kSR * x;
-    *reinterpret_cast<ulonglong2*>(o + ia) = make_ulonglong2(a.v, b.v);
-    *reinterpret_cast<unsigned long long*>(o + ie) = e.v;
+    *reinterpret_cast<ulonglong2*>(nxt + duo_ab(cap, q) + 4 * x) = make_ulonglong2(a.v, b.v);
+    *reinterpret_cast<unsigned long long*>(nxt + duo_ef(cap, q) + 4 * x) = e.v;
     if (pkt) {  // packets 2 q, 2 q + 1: (a, b.x), (b.y, e)
         const unsigned long long t = (unsigned long long)tag << 32;
         auto w = [](float v) { return (unsigned long long)__float_as_uint(v); };
@@ -1975,18 +1996,19 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
         st_packet(pkt + 32 * q + 16, w(py(b)) | (w(px(e)) << 32), t | w(py(e)));
     }
 }
-__device__ __forceinline__ void take_packet_duo(float* dst, int c, const Packet& k) {
+__device__ __forceinline__ void take_packet_duo(float* buf, int cap, int x, int c, const Packet& k) {
     const int q = c >> 1;
+    float *ab = buf + duo_ab(cap, q) + 4 * x, *ef = buf + duo_ef(cap, q) + 4 * x;
     const float v0 = __uint_as_float((unsigned)k.lo), v1 = __uint_as_float((unsigned)(k.lo >> 32)),
                 v2 = __uint_as_float((unsigned)k.hi);
     if (c & 1) {
-        dst[4 * q + 3] = v0;
-        dst[8 + 2 * q] = v1;
-        dst[9 + 2 * q] = v2;
+        ab[3] = v0;
+        ef[0] = v1;
+        ef[1] = v2;
     } else {
-        dst[4 * q] = v0;
-        dst[4 * q + 1] = v1;
-        dst[4 * q + 2] = v2;
+        ab[0] = v0;
+        ab[1] = v1;
+        ab[2] = v2;
     }
 }
 
@@ -2102,7 +2124,7 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
             v = ld_packet(src);
         }
         if constexpr (kDuo)
-            take_packet_duo(cur + (size_t)kSR * sl, c, v);
+            take_packet_duo(cur, d.deep_slot_cap, sl, c, v);
         else
             take_packet(cur + (size_t)kSR * sl, c, v);
     }
@@ -2170,9 +2192,15 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
         const T* r = g0 + (int64_t)kRec * g;
         T* o = buf0 + (size_t)kSR * x;
         const Vec4<T> v0 = ld4(r), v1 = ld4(r + 4), v2 = ld4(r + 8);
+        T *o1 = o + 4, *o2 = o + 8;
+        if constexpr (kDuo) {
+            o = buf0 + 4 * x;
+            o1 = o + 4 * d.deep_slot_cap;
+            o2 = o1 + 4 * d.deep_slot_cap;
+        }
         st4(o, v0.y, v0.z, v0.w, v1.x);
-        st4(o + 4, v1.y, v1.z, v1.w, v2.x);
-        st4(o + 8, v0.x, v2.y, v2.z, v2.w);
+        st4(o1, v1.y, v1.z, v1.w, v2.x);
+        st4(o2, v0.x, v2.y, v2.z, v2.w);
     }
     __syncthreads();
     {
@@ -2223,7 +2251,7 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                 const float gx = __uint_as_float(u.x), gy = __uint_as_float(u.y);
                 R.k[j] = Q2.q ? pk(add_rn(gx, gy), sub_rn(gx, gy)) : pk(gx, gy);
                 R.c[j] = __uint_as_float(u.z);
-                R.col[j] = in_row ? (int)u.w : (have ? x : 0);
+                R.col[j] = 4 * (in_row ? (int)u.w : (have ? x : 0));
             }
         }
 #pragma unroll 1
@@ -2248,7 +2276,10 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
             const Pops<T> f = fv_outer_from(d, reinterpret_cast<const T*>(sm + L.osnap) + kSnap * q, 1, m);
             T z[3], ux, uy;
             z_of(f, d.rho0, z, ux, uy);
-            st_rec(star_at(m) + (size_t)kSR * q, rec_of(f, z));
+            if constexpr (kDuo)
+                duo_put(star_at(m), d.deep_ocap, q, rec_of(f, z));
+            else
+                st_rec(star_at(m) + (size_t)kSR * q, rec_of(f, z));
         }
     };
     if constexpr (kOuterFv) {
@@ -2371,9 +2402,14 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
         // the state after the last completed sub-step, in index order
         const T* fin = (m & 1) ? buf1 : buf0;
         for (int x = tid; x < n_own; x += NT) {
-            const T* r = fin + (size_t)kSR * x;
+            const T *r = fin + (size_t)kSR * x, *r1 = r + 4, *r2 = r + 8;
+            if constexpr (kDuo) {
+                r = fin + 4 * x;
+                r1 = r + 4 * d.deep_slot_cap;
+                r2 = r1 + 4 * d.deep_slot_cap;
+            }
             T* o = g1 + (int64_t)kRec * gid[x];
-            const Vec4<T> v0 = ld4(r), v1 = ld4(r + 4), v2 = ld4(r + 8);
+            const Vec4<T> v0 = ld4(r), v1 = ld4(r1), v2 = ld4(r2);
             st4(o, v2.x, v0.x, v0.y, v0.z);
             st4(o + 4, v0.w, v1.x, v1.y, v1.z);
             st4(o + 8, v1.w, v2.y, v2.z, v2.w);
@@ -2452,6 +2488,10 @@ cudaError_t launch_fv_deep_pack(const FvPack<T>& pk, int blocks, size_t smem, cu
         }
     }
     return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(threads), args, smem, s);
+}
+template <typename T>
+int fv_deep_cap(int n) {
+    return sizeof(T) == 4 ? duo_cap(n) : n;
 }
 template <typename T>
 int fv_deep_duo_slots() {
@@ -3794,6 +3834,7 @@ void launch_adj_refill(const Dev<T>& d, const StepArgs& a, const T* lPm, T* lP0,
     template cudaError_t launch_fv_tmem<T>(const Dev<T>&, const StepArgs&, cudaStream_t);                     \
     template cudaError_t launch_fv_tmem_pack<T>(const FvPack<T>&, int, size_t, cudaStream_t);                 \
     template int fv_deep_tmem_slots<T>();                                                                     \
+    template int fv_deep_cap<T>(int);                                                                         \
     template int fv_deep_duo_slots<T>();                                                                      \
     template int fv_deep_early<T>();                                                                          \
     template int fv_deep_row_words<T>();                                                                      \
