@@ -1324,8 +1324,8 @@ cudaError_t launch_fv_tmem(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // threads of two slots that load a row in two halves.  The FP32 block has
 // 256 more threads (8 warps) that run the next lattice step's stream-collide
 // away from the patch (FarArgs) while the FV warps step the patch.
-template <typename T>
-constexpr int kDeepThreads = sizeof(T) == 4 ? 1024 : 512;  // block size
+template <typename T, bool kFar>
+constexpr int kDeepThreads = sizeof(T) == 4 ? (kFar ? 1024 : 768) : 512;  // block size
 template <typename T>
 constexpr int kDeepFv = sizeof(T) == 4 ? 768 : 512;  // FV threads: warps 0 .. kDeepFv / 32 - 1
 template <typename T>
@@ -2093,14 +2093,28 @@ __device__ __forceinline__ void fv_bar() {
     asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory");
 }
 
+// the same, and whether any of them calls it with bad
+template <int N>
+__device__ __forceinline__ bool fv_bar_or(bool bad) {
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred q, 1, %2, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((int)bad), "n"(N)
+        : "memory");
+    return r != 0;
+}
+// a barrier of the last n FV threads (named barrier 2)
+__device__ __forceinline__ void late_bar(int n) { asm volatile("bar.sync 2, %0;" ::"r"(n) : "memory"); }
+
 // Receives the ghost records of one exchange into the ghost slots of buffer
 // cur: thread k of N (counted from the last FV thread, whose warps have the
 // fewest nodes) takes packets k, k + N, ...  Each is polled until its tag is
 // the exchange's, a bounded number of times; false when a wait ran out or
 // another tile gave up.
-template <typename T, int N, bool kDuo>
+template <typename T, bool kDuo>
 __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned char* xb, const int32_t* gid, T* cur,
-                                             int n_own, int n_slot, unsigned tag, int k) {
+                                             int n_own, int n_slot, unsigned tag, int k, int N) {
     constexpr int PK = kPkts<T>;
     const int np = (n_slot - n_own) * PK;
     bool ok = true;
@@ -2135,11 +2149,11 @@ __device__ __forceinline__ bool deep_receive(const Dev<T>& d, const unsigned cha
 // one solver, k_fv_deep_pack several.  kRecord: also writes what the reverse
 // mode needs of every sub-step (Dev::fv_rec).
 // kDuo (FP32): two lanes per node, no tensor memory, no lattice warps.
-template <typename T, bool kRecord, bool kOuterFv, bool kDuo>
+template <typename T, bool kRecord, bool kOuterFv, bool kDuo, bool kFar>
 __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a, T* g0, T* g1, const FarArgs<T>& far,
                                              const int tile, unsigned char* sm, int& abort_sh,
                                              uint32_t& tmem_base_sh) {
-    constexpr int NT = kDuo ? kDuoThreads : kDeepFv<T>, BT = kDuo ? kDuoThreads : kDeepThreads<T>;
+    constexpr int NT = kDuo ? kDuoThreads : kDeepFv<T>, BT = kDuo ? kDuoThreads : kDeepThreads<T, kFar>;
     constexpr int G = kDeepGroups<T>, SW = kDeepSlotWords<T>;
     const int tid = threadIdx.x, warp = tid >> 5;
     const int s0 = d.deep_ptr[tile];
@@ -2297,6 +2311,10 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
         // own nodes that read only own nodes, updated while the ghosts are on
         // their way (0 where that does not pay: fv_deep_early)
         const int n_early = quads || kDuo ? 0 : n_a;
+        // first thread of the warps that have slots left after the early part
+        // (they lie in the second group: n_a fills the first)
+        constexpr bool kSplit = !kDuo && sizeof(T) == 4;
+        const int late0 = kSplit && n_early > 0 ? min(NT - 32, (n_early - NT) / 32 * 32) : 0;
         Quad Q;
         Q.q = tid & 3;
         Q.w = w_of<double>(Q.q < 2 ? 1 : 5);
@@ -2315,6 +2333,7 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                 const bool send = (s == kb - 1) && !final_block && tile != d.stall_tile;
                 const int cs = cnt[3 + s];
                 int lo = 0;
+                bool ok = true;
                 // the next sub-step's interpolated records (from the last FV thread down)
                 if (kOuterFv && m + 1 < d.n_sub) make_stars(m + 1, NT - 1 - tid, NT);
                 if (s == 0 && b > 0) {
@@ -2328,36 +2347,47 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                                                                 true, star_at(m));
                         }
                     }
-                    bool ok = deep_receive<T, NT, kDuo>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
-                                                  a.xtag + (unsigned)b, NT - 1 - tid);
-                    // tiles that read this one but are not read by it: their reads of
-                    // the packets about to be overwritten are behind their counter
-                    for (int e = nb0 + tid; e < nb1 && ok; e += NT) {
-                        const unsigned long long* pc = d.progress + d.tile_nb[e];
-                        long spins = 0;
-                        while (ld_acquire(pc) < base + m) {
-                            if (*(volatile unsigned*)d.abort_flag) {
-                                ok = false;
-                                break;
+                    // FP32, after an early part: the warps with slots left receive and go
+                    // on while the others still update, with a barrier of their own
+                    if (tid >= late0) {
+                        const int nr = kSplit ? NT - late0 : NT;
+                        ok = deep_receive<T, kDuo>(d, d.deep_x + (b & 1) * xhalf, gid, cur, n_own, n_slot,
+                                                   a.xtag + (unsigned)b, NT - 1 - tid, nr);
+                        // tiles that read this one but are not read by it: their reads of
+                        // the packets about to be overwritten are behind their counter
+                        for (int e = nb0 + tid - late0; e < nb1 && ok; e += nr) {
+                            const unsigned long long* pc = d.progress + d.tile_nb[e];
+                            long spins = 0;
+                            while (ld_acquire(pc) < base + m) {
+                                if (*(volatile unsigned*)d.abort_flag) {
+                                    ok = false;
+                                    break;
+                                }
+                                if (++spins > d.spin_limit) {
+                                    atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
+                                    atomicExch(d.abort_flag, 1u);
+                                    ok = false;
+                                    break;
+                                }
                             }
-                            if (++spins > d.spin_limit) {
-                                atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
-                                atomicExch(d.abort_flag, 1u);
-                                ok = false;
+                        }
+                        if constexpr (kSplit) {
+                            late_bar(nr);
+                        } else {
+                            if (!ok) abort_sh = 1;
+                            fv_bar<NT>();
+                            if (abort_sh) {
+                                aborted = true;
                                 break;
                             }
                         }
                     }
-                    if (!ok) abort_sh = 1;
-                    fv_bar<NT>();
-                    if (abort_sh) {
-                        aborted = true;
-                        break;
-                    }
                     // a block of one sub-step ends here: the nodes updated early are sent
-                    // only now, after the receive (which frees the packets they overwrite)
-                    if (send) {
-                        for (int x = tid; x < n_early; x += NT)
+                    // only after the receive (which frees the packets they overwrite)
+                    if (send && n_early > 0) {
+                        bool bad = false;
+                        if constexpr (kSplit) bad = fv_bar_or<NT>(!ok);
+                        for (int x = tid; x < n_early && !bad; x += NT)
                             if (sd[x])
                                 send_record(xout + (int64_t)gid[x] * kPkts<T> * 16, ld_rec(nxt + (size_t)kSR * x), tag_out);
                     }
@@ -2394,7 +2424,12 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
                                 x < n_own, star_at(m));
                     }
                 }
-                fv_bar<NT>();
+                if (kSplit && s == 0 && b > 0) {
+                    aborted = fv_bar_or<NT>(!ok);  // a wait ran out: the sub-step's results are dropped
+                    if (aborted) break;
+                } else {
+                    fv_bar<NT>();
+                }
             }
             if (!aborted && !final_block && d.deep_pub[tile] && tid == NT - 1 && tile != d.stall_tile)
                 st_release(d.progress + tile, base + m);
@@ -2414,7 +2449,7 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
             st4(o + 4, v0.w, v1.x, v1.y, v1.z);
             st4(o + 8, v1.w, v2.y, v2.z, v2.w);
         }
-    } else if constexpr (sizeof(T) == 4) {
+    } else if constexpr (kFar) {
         far_chunks(d, far);
     }
     // ---- release TMEM (also after an abort: every warp is past its last tcgen05.ld)
@@ -2426,12 +2461,12 @@ __device__ __forceinline__ void fv_deep_body(const Dev<T>& d, const StepArgs& a,
     }
 }
 
-template <typename T, bool kRecord, bool kOuterFv>
-__global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
+template <typename T, bool kRecord, bool kOuterFv, bool kFar>
+__global__ void __launch_bounds__(kDeepThreads<T, kFar>, 1) k_fv_deep(Dev<T> d, StepArgs a, T* g0, T* g1, FarArgs<T> far) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int abort_sh;
     __shared__ uint32_t tmem_base_sh;
-    fv_deep_body<T, kRecord, kOuterFv, false>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, tmem_base_sh);
+    fv_deep_body<T, kRecord, kOuterFv, false, kFar>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, tmem_base_sh);
 }
 
 // Several solvers' FV sub-steps in one cooperative launch: block b runs tile
@@ -2439,14 +2474,14 @@ __global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep(Dev<T> d, StepAr
 // keeps its own tables, packets, tags, sub-step count and buffers; items only
 // share the GPU.
 template <typename T>
-__global__ void __launch_bounds__(kDeepThreads<T>, 1) k_fv_deep_pack(const __grid_constant__ FvPack<T> pk) {
+__global__ void __launch_bounds__(kDeepThreads<T, false>, 1) k_fv_deep_pack(const __grid_constant__ FvPack<T> pk) {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int abort_sh;
     __shared__ uint32_t tmem_base_sh;
     int i = 0;
     while (i + 1 < pk.n && pk.block0[i + 1] <= (int)blockIdx.x) ++i;
-    fv_deep_body<T, false, false, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<T>{}, (int)blockIdx.x - pk.block0[i], sm,
-                           abort_sh, tmem_base_sh);
+    fv_deep_body<T, false, false, false, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<T>{}, (int)blockIdx.x - pk.block0[i], sm,
+                                                abort_sh, tmem_base_sh);
 }
 
 // FP32 patches whose tiles' computed slots fit pairs of lanes.  Blocks past
@@ -2461,7 +2496,7 @@ __global__ void __launch_bounds__(kDuoThreads, 1) k_fv_duo(Dev<float> d, StepArg
     if ((int)blockIdx.x >= d.n_tiles)
         far_chunks(d, far);
     else
-        fv_deep_body<float, kRecord, kOuterFv, true>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, none);
+        fv_deep_body<float, kRecord, kOuterFv, true, false>(d, a, g0, g1, far, blockIdx.x, sm, abort_sh, none);
 }
 __global__ void __launch_bounds__(kDuoThreads, 1) k_fv_duo_pack(const __grid_constant__ FvPack<float> pk) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -2469,7 +2504,7 @@ __global__ void __launch_bounds__(kDuoThreads, 1) k_fv_duo_pack(const __grid_con
     uint32_t none = 0;
     int i = 0;
     while (i + 1 < pk.n && pk.block0[i + 1] <= (int)blockIdx.x) ++i;
-    fv_deep_body<float, false, false, true>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<float>{},
+    fv_deep_body<float, false, false, true, false>(pk.d[i], pk.a[i], pk.g0[i], pk.g1[i], FarArgs<float>{},
                                             (int)blockIdx.x - pk.block0[i], sm, abort_sh, none);
 }
 
@@ -2478,7 +2513,7 @@ cudaError_t launch_fv_deep_pack(const FvPack<T>& pk, int blocks, size_t smem, cu
     FvPack<T> p = pk;
     void* args[] = {&p};
     const void* fn = (const void*)k_fv_deep_pack<T>;
-    int threads = kDeepThreads<T>;
+    int threads = kDeepThreads<T, false>;
     if constexpr (sizeof(T) == 4) {
         bool duo = true;
         for (int k = 0; k < pk.n; ++k) duo = duo && pk.d[k].deep_duo;
@@ -2507,9 +2542,12 @@ int fv_deep_tile_capacity(size_t smem) {
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // each block allocates all 512 TMEM columns: only one block per SM
     std::vector<std::pair<const void*, int>> fns;
-    for (const void* fn : {(const void*)k_fv_deep<T, false, false>, (const void*)k_fv_deep<T, true, false>,
-                           (const void*)k_fv_deep<T, false, true>, (const void*)k_fv_deep_pack<T>})
-        fns.push_back({fn, kDeepThreads<T>});
+    for (const void* fn : {(const void*)k_fv_deep<T, false, false, false>, (const void*)k_fv_deep<T, true, false, false>,
+                           (const void*)k_fv_deep<T, false, true, false>, (const void*)k_fv_deep_pack<T>})
+        fns.push_back({fn, kDeepThreads<T, false>});
+    if constexpr (sizeof(T) == 4)
+        for (const void* fn : {(const void*)k_fv_deep<T, false, false, true>, (const void*)k_fv_deep<T, false, true, true>})
+            fns.push_back({fn, kDeepThreads<T, true>});
     if constexpr (sizeof(T) == 4)
         for (const void* fn : {(const void*)k_fv_duo<false, false>, (const void*)k_fv_duo<true, false>,
                                (const void*)k_fv_duo<false, true>, (const void*)k_fv_duo_pack})
@@ -2543,11 +2581,15 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
     void* args[] = {&dd, &aa, &b0, &b1, &fa};
     const size_t smem = fv_deep_smem_bytes<T>(d.deep_slot_cap, d.n_sub, d.deep_ocap, d.deep_quads,
                                                d.outer_fv ? d.deep_ocap : 0);
-    const void* fn = d.outer_fv ? (const void*)k_fv_deep<T, false, true>
-                     : d.fv_rec ? (const void*)k_fv_deep<T, true, false>
-                                : (const void*)k_fv_deep<T, false, false>;
-    int threads = kDeepThreads<T>, blocks = d.n_tiles;
+    const void* fn = d.outer_fv ? (const void*)k_fv_deep<T, false, true, false>
+                     : d.fv_rec ? (const void*)k_fv_deep<T, true, false, false>
+                                : (const void*)k_fv_deep<T, false, false, false>;
+    int threads = kDeepThreads<T, false>, blocks = d.n_tiles;
     if constexpr (sizeof(T) == 4) {
+        if (fa.n_chunks > 0 && !d.fv_rec) {
+            fn = d.outer_fv ? (const void*)k_fv_deep<T, false, true, true> : (const void*)k_fv_deep<T, false, false, true>;
+            threads = kDeepThreads<T, true>;
+        }
         if (d.deep_duo) {
             fn = d.outer_fv ? (const void*)k_fv_duo<false, true>
                  : d.fv_rec ? (const void*)k_fv_duo<true, false>
