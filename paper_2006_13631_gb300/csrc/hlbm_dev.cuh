@@ -117,28 +117,33 @@ __device__ __forceinline__ T feq_dev(int i, T drho, T rho, T ux, T uy) {
 }
 
 // BGK relaxation of a deviation set (eq. LBE's collision with tau_s):
-// out_i = f_i - omega (f_i - f_i^eq), with f_i^eq - w_i rho0 = w_i (G +- H)
-// for the pair i, opp(i) (c_opp = -c_i): G = drho + rho (4.5 (c.u)^2 -
-// 1.5 u^2), H = 3 rho c.u.  The same numbers as feq_dev up to rounding, in
-// fewer operations; the relaxation keeps the form that rounds only the
-// small non-equilibrium part.  rho0 may be given scaled by a power of two
-// together with f.  Explicitly rounded: the lattice is collided by more
-// than one kernel, which must agree bit for bit.
+// out_i = f_i - omega (f_i - f_i^eq), with f_i^eq - w_i rho0 = w_i (G +- 3 rho c.u)
+// for the pair i, opp(i) (c_opp = -c_i), G = drho + rho (4.5 (c.u)^2 - 1.5 u^2).
+// The same numbers as feq_dev up to rounding, in fewer operations; the
+// relaxation keeps the form that rounds only the small non-equilibrium part.
+// rho0 may be given scaled by a power of two together with f.  Explicitly
+// rounded, and no product is the operand of a sum, so that nothing is left to
+// contract: the lattice is collided by more than one kernel, a node at a time or
+// two (bgk_pair in fv_node.cuh), which must agree bit for bit.
 template <typename T>
 __device__ __forceinline__ void bgk_dev(const T (&f)[9], T rho0, T omega, T (&out)[9]) {
-    T dr, r, ux, uy;
-    moments_dev(f, rho0, dr, r, ux, uy);
-    const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
-    out[0] = fma_rn(-omega, sub_rn(f[0], mul_rn(w_of<T>(0), fma_rn(r, q, dr))), f[0]);
+    T dr = f[0], jx = T(0), jy = T(0);
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
-        if (opp_of(i) < i) continue;  // each pair once, from its lower index
-        const int j = opp_of(i);
-        const T cu = cdot(i, ux, uy);
-        const T G = fma_rn(r, fma_rn(mul_rn(T(4.5), cu), cu, q), dr);
-        const T H = mul_rn(r, mul_rn(T(3), cu));
-        out[i] = fma_rn(-omega, sub_rn(f[i], mul_rn(w_of<T>(i), add_rn(G, H))), f[i]);
-        out[j] = fma_rn(-omega, sub_rn(f[j], mul_rn(w_of<T>(j), sub_rn(G, H))), f[j]);
+        dr = add_rn(dr, f[i]);
+        jx = add_cx(i, jx, f[i]);
+        jy = add_cy(i, jy, f[i]);
+    }
+    const T r = add_rn(rho0, dr), inv = T(1) / r, r3 = mul_rn(T(3), r);
+    const T c[4] = {mul_rn(jx, inv), mul_rn(jy, inv), mul_rn(add_rn(jx, jy), inv), mul_rn(sub_rn(jy, jx), inv)};
+    const T q = mul_rn(T(-1.5), fma_rn(c[0], c[0], mul_rn(c[1], c[1])));
+    out[0] = fma_rn(-omega, fma_rn(-w_of<T>(0), fma_rn(r, q, dr), f[0]), f[0]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = k < 2 ? k + 1 : k + 3, j = opp_of(i);  // 1, 2, 5, 6
+        const T G = fma_rn(r, fma_rn(mul_rn(T(4.5), c[k]), c[k], q), dr);
+        out[i] = fma_rn(-omega, fma_rn(-w_of<T>(i), fma_rn(r3, c[k], G), f[i]), f[i]);
+        out[j] = fma_rn(-omega, fma_rn(-w_of<T>(i), fma_rn(-r3, c[k], G), f[j]), f[j]);
     }
 }
 

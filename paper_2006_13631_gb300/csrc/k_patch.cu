@@ -2051,16 +2051,14 @@ __device__ __forceinline__ void far_chunk(const Dev<float>& d, const FarArgs<flo
     }
     if (!mine) return;
     if (interior) {
-        float f[9], o0[9], o1[9];
+        Pr<float> f[9], o[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = cx_of(i) == 0 ? p[i].x : (cx_of(i) == 1 ? edge[i] : p[i].y);
-        bgk_dev(f, d.rho0, omega, o0);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = cx_of(i) == 0 ? p[i].y : (cx_of(i) == 1 ? p[i].x : edge[i]);
-        bgk_dev(f, d.rho0, omega, o1);
+        for (int i = 0; i < 9; ++i)
+            f[i] = cx_of(i) == 0 ? pk(p[i].x, p[i].y) : (cx_of(i) == 1 ? pk(edge[i], p[i].x) : pk(p[i].y, edge[i]));
+        bgk_pair(f, d.rho0, omega, o);
         const int64_t s0 = (int64_t)y * d.pitch + x0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(B + i * d.plane + s0) = make_float2(o0[i], o1[i]);
+        for (int i = 0; i < 9; ++i) *reinterpret_cast<unsigned long long*>(B + i * d.plane + s0) = o[i].v;
     } else {
         for (int k = 0; k < 2; ++k) {
             const int x = x0 + k;
