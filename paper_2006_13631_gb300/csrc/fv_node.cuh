@@ -80,34 +80,6 @@ __device__ __forceinline__ Pr<double> pfma(Pr<double> a, Pr<double> b, Pr<double
     return Pr<double>{__fma_rn(a.a, b.a, c.a), __fma_rn(a.b, b.b, c.b)};
 }
 
-// bgk_dev (hlbm_dev.cuh) of two FP32 nodes, one in each half of the pairs: the
-// same operation on every element in the same order, so the same bits, in half
-// the instructions: for the lattice warps beside the FV warps, which are short of
-// issue slots.  (In k_stream_collide it changes nothing in FP32, bound by HBM,
-// and costs the 2-byte lattices 7 %: 122.8 against 114.6 us at 4096^2.)
-__device__ __forceinline__ void bgk_pair(const Pr<float> (&f)[9], float rho0, float omega, Pr<float> (&out)[9]) {
-    auto both = [](float v) { return pk(v, v); };
-    Pr<float> dr = f[0], jx = both(0.0f), jy = both(0.0f);
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        dr = padd(dr, f[i]);
-        if (cx_of(i) != 0) jx = cx_of(i) > 0 ? padd(jx, f[i]) : psub(jx, f[i]);
-        if (cy_of(i) != 0) jy = cy_of(i) > 0 ? padd(jy, f[i]) : psub(jy, f[i]);
-    }
-    const Pr<float> r = padd(both(rho0), dr), inv = pk(1.0f / px(r), 1.0f / py(r));
-    const Pr<float> r3 = pmul(both(3.0f), r), m3 = pmul(both(-3.0f), r), no = both(-omega);
-    const Pr<float> c[4] = {pmul(jx, inv), pmul(jy, inv), pmul(padd(jx, jy), inv), pmul(psub(jy, jx), inv)};
-    const Pr<float> q = pmul(both(-1.5f), pfma(c[0], c[0], pmul(c[1], c[1])));
-    out[0] = pfma(no, pfma(both(-w_of<float>(0)), pfma(r, q, dr), f[0]), f[0]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = k < 2 ? k + 1 : k + 3, j = opp_of(i);
-        const Pr<float> G = pfma(r, pfma(pmul(both(4.5f), c[k]), c[k], q), dr), w = both(-w_of<float>(i));
-        out[i] = pfma(no, pfma(w, pfma(r3, c[k], G), f[i]), f[i]);
-        out[j] = pfma(no, pfma(w, pfma(m3, c[k], G), f[j]), f[j]);
-    }
-}
-
 // the eight moving populations of a set, and its rest population
 template <typename T>
 struct Pops {
@@ -133,12 +105,40 @@ template <typename T>
 __device__ __forceinline__ void state_of(const T (&f)[9], T rho0, T (&st)[12]);
 
 // sum f_i, sum c_ix f_i, sum c_iy f_i
-template <typename T>
-__device__ __forceinline__ void pops_moments(const Pops<T>& p, T& m0, T& mx, T& my) {
-    const Pr<T> s1 = padd(p.A, p.B), d1 = psub(p.A, p.B), s2 = padd(p.C, p.D), d2 = psub(p.C, p.D);
+__device__ __forceinline__ void pops_moments(const Pops<float>& p, float& m0, float& mx, float& my) {
+    float f[9];
+    pops_to(p, f);
+    m0 = f[0];
+    mx = my = 0.0f;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        m0 = add_rn(m0, f[i]);
+        mx = add_cx(i, mx, f[i]);
+        my = add_cy(i, my, f[i]);
+    }
+}
+__device__ __forceinline__ void pops_moments(const Pops<double>& p, double& m0, double& mx, double& my) {
+    const Pr<double> s1 = padd(p.A, p.B), d1 = psub(p.A, p.B), s2 = padd(p.C, p.D), d2 = psub(p.C, p.D);
     m0 = add_rn(p.f0, add_rn(add_rn(px(s1), py(s1)), add_rn(px(s2), py(s2))));
     mx = add_rn(px(d1), sub_rn(px(d2), py(d2)));
     my = add_rn(py(d1), add_rn(px(d2), py(d2)));
+}
+
+// (f_i^eq - w_i rho0) / w_i of the directions with c . u = c (x) and of their
+// opposites (y): drho + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u^2)
+__device__ __forceinline__ void feq_x(Pr<float> c, float dr, float rho, float usq, Pr<float>& x, Pr<float>& y) {
+    const Pr<float> e = pmul(pmul(pk(4.5f, 4.5f), c), c), u = pk(usq, usq), m = pk(-1.5f, -1.5f), r = pk(rho, rho), d = pk(dr, dr);
+    x = pfma(r, pfma(m, u, pfma(pk(3.0f, 3.0f), c, e)), d);
+    y = pfma(r, pfma(m, u, pfma(pk(-3.0f, -3.0f), c, e)), d);
+}
+// all of them, as a set: the axes' and the diagonals' pairs, and the rest one
+__device__ __forceinline__ Pops<float> feq_x(float dr, float rho, float ux, float uy) {
+    const float usq = fma_rn(ux, ux, mul_rn(uy, uy));
+    Pops<float> X;
+    feq_x(pk(ux, uy), dr, rho, usq, X.A, X.B);
+    feq_x(pk(add_rn(ux, uy), sub_rn(uy, ux)), dr, rho, usq, X.C, X.D);
+    X.f0 = fma_rn(rho, mul_rn(-1.5f, usq), dr);
+    return X;
 }
 
 // f_i^eq - w_i rho0 of the pair (i, opp(i)) as w_i (G + H), w_i (G - H)
@@ -154,10 +154,17 @@ __device__ __forceinline__ void state_of(const T (&f)[9], T rho0, T (&st)[12]) {
     T dr, jx, jy;
     pops_moments(pops_of(f), dr, jx, jy);
     const T rho = add_rn(rho0, dr), inv = T(1) / rho, ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
-    const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
     st[0] = dr;
     st[1] = ux;
     st[2] = uy;
+    if constexpr (sizeof(T) == 4) {
+        T x[9];
+        pops_to(feq_x(dr, rho, ux, uy), x);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) st[3 + i] = fma_rn(-w_of<T>(i), x[i], f[i]);
+        return;
+    }
+    const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
     st[3] = sub_rn(f[0], mul_rn(w_of<T>(0), fma_rn(rho, q, dr)));
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
@@ -169,7 +176,22 @@ __device__ __forceinline__ void state_of(const T (&f)[9], T rho0, T (&st)[12]) {
     }
 }
 
-// acc - w_i (G_i + 3 c_i . (x, y)) over the moving directions, G = (g1, g2)
+// FP32: acc - w_i (4.5 Q_i + 3 c_i . (x, y) + g) with Q the quadratic part (qa on
+// the axes, qd on the diagonals) when kQuad
+template <bool kQuad>
+__device__ __forceinline__ void pops_sub_lin(Pops<float>& p, float g, float x, float y, Pr<float> qa, Pr<float> qd) {
+    const Pr<float> w1 = pk(-w_of<float>(1), -w_of<float>(1)), w5 = pk(-w_of<float>(5), -w_of<float>(5));
+    const Pr<float> h = pk(4.5f, 4.5f), t = pk(3.0f, 3.0f), m = pk(-3.0f, -3.0f), gg = pk(g, g);
+    const Pr<float> ca = pk(x, y), cd = pk(add_rn(x, y), sub_rn(y, x));
+    Pr<float> A = pfma(t, ca, gg), B = pfma(m, ca, gg), C = pfma(t, cd, gg), D = pfma(m, cd, gg);
+    if (kQuad) A = pfma(h, qa, A), B = pfma(h, qa, B), C = pfma(h, qd, C), D = pfma(h, qd, D);
+    p.A = pfma(w1, A, p.A);
+    p.B = pfma(w1, B, p.B);
+    p.C = pfma(w5, C, p.C);
+    p.D = pfma(w5, D, p.D);
+}
+
+// FP64: acc - w_i (G_i + 3 c_i . (x, y)) over the moving directions, G = (g1, g2)
 // on the axes x and y and (g5, g6) on the diagonals (1, 1) and (-1, 1)
 template <typename T>
 __device__ __forceinline__ void pops_sub_lin(Pops<T>& p, Pr<T> ga, Pr<T> gd, T x, T y) {
@@ -194,9 +216,15 @@ __device__ __forceinline__ void z_of(const Pops<T>& p, T rho0, T (&z)[3], T& ux,
     const T inv = T(1) / add_rn(rho0, dr);
     ux = mul_rn(jx, inv);
     uy = mul_rn(jy, inv);
-    z[0] = mul_rn(jx, ux);
-    z[1] = mul_rn(jx, uy);
-    z[2] = mul_rn(jy, uy);
+    if constexpr (sizeof(T) == 4) {
+        z[0] = mul_rn(mul_rn(jx, jx), inv);
+        z[1] = mul_rn(mul_rn(jx, jy), inv);
+        z[2] = mul_rn(mul_rn(jy, jy), inv);
+    } else {
+        z[0] = mul_rn(jx, ux);
+        z[1] = mul_rn(jx, uy);
+        z[2] = mul_rn(jy, uy);
+    }
 }
 template <typename T>
 __device__ __forceinline__ void z_of(const T (&f)[9], T rho0, T (&z)[3]) {
@@ -267,13 +295,21 @@ __device__ __forceinline__ Pops<T> fv_sums_finish(const Dev<T>& d, FvSums<T>& s,
     // sum_k C_Pk (f^eq_k,i - w_i rho0): quadratic part Z0, Z2 on the axes and
     // Z0 + Z2 +- 2 Z1 on the diagonals
     const T zs = add_rn(Z0, Z2), q0 = fma_rn(T(-1.5), zs, dr);
-    const Pr<T> q = pk(q0, q0), h = pk(T(4.5), T(4.5));
-    pops_sub_lin(n, pfma(h, pk(Z0, Z2), q), pfma(h, pk(fma_rn(T(2), Z1, zs), fma_rn(T(-2), Z1, zs)), q), jx, jy);
+    if constexpr (sizeof(T) == 4) {
+        const Pr<T> qd = pk(add_rn(fma_rn(T(2), Z1, Z0), Z2), add_rn(fma_rn(T(-2), Z1, Z0), Z2));
+        pops_sub_lin<true>(n, q0, jx, jy, pk(Z0, Z2), qd);
+    } else {
+        const Pr<T> q = pk(q0, q0), h = pk(T(4.5), T(4.5));
+        pops_sub_lin(n, pfma(h, pk(Z0, Z2), q), pfma(h, pk(fma_rn(T(2), Z1, zs), fma_rn(T(-2), Z1, zs)), q), jx, jy);
+    }
     n.f0 = fma_rn(-w_of<T>(0), q0, n.f0);
     T m0, mx, my;
     pops_moments(n, m0, mx, my);
     const Pr<T> mm = pk(m0, m0);
-    pops_sub_lin(n, mm, mm, mx, my);
+    if constexpr (sizeof(T) == 4)
+        pops_sub_lin<false>(n, m0, mx, my, mm, mm);
+    else
+        pops_sub_lin(n, mm, mm, mx, my);
     n.f0 = fma_rn(-w_of<T>(0), m0, n.f0);
     // f_P + dt_u (S - n / tau_u)
     const T iv = d.inv_tau_u, dt = d.dt_u;
@@ -287,7 +323,8 @@ __device__ __forceinline__ Pops<T> fv_sums_finish(const Dev<T>& d, FvSums<T>& s,
 }
 
 // wall nodes: impose the lamina velocity, keep the non-equilibrium part:
-// f_i += w_i rho (3 c_i.(U - u) + 4.5 ((c_i.U)^2 - (c_i.u)^2) - 1.5 (U^2 - u^2)),
+// f_i += f_i^eq(rho, U) - f_i^eq(rho, u); in FP64
+// w_i rho (3 c_i.(U - u) + 4.5 ((c_i.U)^2 - (c_i.u)^2) - 1.5 (U^2 - u^2)),
 // the squares as products of sums and differences
 // (the update's moments rho, u go to mo)
 template <typename T>
@@ -299,6 +336,16 @@ __device__ __forceinline__ void fv_wall(const Dev<T>& d, T U, T V, Pops<T>& p, T
     mo[0] = rho;
     mo[1] = ux;
     mo[2] = uy;
+    if constexpr (sizeof(T) == 4) {
+        const Pops<T> X = feq_x(dr, rho, U, V), Y = feq_x(dr, rho, ux, uy);
+        auto add = [](T wi, Pr<T> x, Pr<T> y, Pr<T> f) { return padd(f, pfma(pk(wi, wi), x, pmul(pk(-wi, -wi), y))); };
+        p.A = add(w_of<T>(1), X.A, Y.A, p.A);
+        p.B = add(w_of<T>(1), X.B, Y.B, p.B);
+        p.C = add(w_of<T>(5), X.C, Y.C, p.C);
+        p.D = add(w_of<T>(5), X.D, Y.D, p.D);
+        p.f0 = add_rn(p.f0, fma_rn(w_of<T>(0), X.f0, mul_rn(-w_of<T>(0), Y.f0)));
+        return;
+    }
     const T dx = sub_rn(U, ux), dy = sub_rn(V, uy), sx = add_rn(U, ux), sy = add_rn(V, uy);
     const T b = mul_rn(T(-1.5), fma_rn(dx, sx, mul_rn(dy, sy)));
     const Pr<T> bb = pk(b, b), h = pk(T(4.5), T(4.5)), three = pk(T(3), T(3));
@@ -322,6 +369,17 @@ __device__ __forceinline__ Pops<T> fv_outer_from(const Dev<T>& d, const T* sn, i
     const T th = T(m + 1) / T(d.n_sub), t0 = sub_rn(T(1), th);
     auto at = [&](int j) { return fma_rn(t0, sn[j * stride], mul_rn(th, sn[(12 + j) * stride])); };
     const T dr = at(0), ux = at(1), uy = at(2), rho = add_rn(d.rho0, dr);
+    if constexpr (sizeof(T) == 4) {
+        const Pops<T> X = feq_x(dr, rho, ux, uy);
+        auto f = [&](T wi, Pr<T> x, int j) { return pfma(pk(d.kneq, d.kneq), pk(at(j), at(j + 1)), pmul(pk(wi, wi), x)); };
+        Pops<T> p;
+        p.A = f(w_of<T>(1), X.A, 4);
+        p.B = f(w_of<T>(1), X.B, 6);
+        p.C = f(w_of<T>(5), X.C, 8);
+        p.D = f(w_of<T>(5), X.D, 10);
+        p.f0 = fma_rn(d.kneq, at(3), mul_rn(w_of<T>(0), X.f0));
+        return p;
+    }
     const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
     const Pr<T> rr = pk(rho, rho), qq = pk(q, q), h = pk(T(4.5), T(4.5)), three = pk(T(3), T(3)), kk = pk(d.kneq, d.kneq);
     const Pr<T> ca = pk(ux, uy), cd = pk(add_rn(ux, uy), sub_rn(uy, ux)), dd = pk(dr, dr);

@@ -117,16 +117,37 @@ __device__ __forceinline__ T feq_dev(int i, T drho, T rho, T ux, T uy) {
 }
 
 // BGK relaxation of a deviation set (eq. LBE's collision with tau_s):
-// out_i = f_i - omega (f_i - f_i^eq), with f_i^eq - w_i rho0 = w_i (G +- 3 rho c.u)
-// for the pair i, opp(i) (c_opp = -c_i), G = drho + rho (4.5 (c.u)^2 - 1.5 u^2).
-// The same numbers as feq_dev up to rounding, in fewer operations; the
-// relaxation keeps the form that rounds only the small non-equilibrium part.
-// rho0 may be given scaled by a power of two together with f.  Explicitly
-// rounded, and no product is the operand of a sum, so that nothing is left to
-// contract: the lattice is collided by more than one kernel, a node at a time or
-// two (bgk_pair in fv_node.cuh), which must agree bit for bit.
+// out_i = f_i - omega (f_i - f_i^eq), with f_i^eq - w_i rho0 = w_i (G +- H)
+// for the pair i, opp(i) (c_opp = -c_i): G = drho + rho (4.5 (c.u)^2 -
+// 1.5 u^2), H = 3 rho c.u.  The same numbers as feq_dev up to rounding, in
+// fewer operations; the relaxation keeps the form that rounds only the
+// small non-equilibrium part.  rho0 may be given scaled by a power of two
+// together with f.  Explicitly rounded: the lattice is collided by more
+// than one kernel, which must agree bit for bit.
+// FP64 takes a shorter form (products that feed sums as multiply-adds, 3 rho
+// shared, 9 operations a pair instead of 15): its stream-collide is bound by
+// the FP64 issue rate, 2997 -> 2572 us at 4096^2.  In FP32 it is bound by HBM
+// (180 us either way), and another rounding of every node would show in the
+// 2-byte lattices at the size of their storage error.
 template <typename T>
 __device__ __forceinline__ void bgk_dev(const T (&f)[9], T rho0, T omega, T (&out)[9]) {
+    if constexpr (sizeof(T) == 4) {
+        T dr, r, ux, uy;
+        moments_dev(f, rho0, dr, r, ux, uy);
+        const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
+        out[0] = fma_rn(-omega, sub_rn(f[0], mul_rn(w_of<T>(0), fma_rn(r, q, dr))), f[0]);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            if (opp_of(i) < i) continue;  // each pair once, from its lower index
+            const int j = opp_of(i);
+            const T cu = cdot(i, ux, uy);
+            const T G = fma_rn(r, fma_rn(mul_rn(T(4.5), cu), cu, q), dr);
+            const T H = mul_rn(r, mul_rn(T(3), cu));
+            out[i] = fma_rn(-omega, sub_rn(f[i], mul_rn(w_of<T>(i), add_rn(G, H))), f[i]);
+            out[j] = fma_rn(-omega, sub_rn(f[j], mul_rn(w_of<T>(j), sub_rn(G, H))), f[j]);
+        }
+        return;
+    }
     T dr = f[0], jx = T(0), jy = T(0);
 #pragma unroll
     for (int i = 1; i < 9; ++i) {

@@ -118,11 +118,17 @@ __device__ __forceinline__ void bilinear_quad(const Dev<T>& d, const T* box, int
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = have ? box[i * d.bplane + b] : T(0);
     state_of(f, d.rho0, st);
+    // the sum in corner order
+    const T wq = have ? w : T(0);
+    T w4[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w4[c] = __shfl_sync(0xffffffffu, wq, c, 4);
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
-        st[j] = have ? w * st[j] : T(0);
-        st[j] += __shfl_xor_sync(0xffffffffu, st[j], 1);
-        st[j] += __shfl_xor_sync(0xffffffffu, st[j], 2);
+        T v[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = __shfl_sync(0xffffffffu, st[j], c, 4);
+        st[j] = fma_rn(w4[3], v[3], fma_rn(w4[2], v[2], fma_rn(w4[1], v[1], mul_rn(w4[0], v[0]))));
     }
 }
 
@@ -130,6 +136,13 @@ __device__ __forceinline__ void bilinear_quad(const Dev<T>& d, const T* box, int
 template <typename T>
 __device__ __forceinline__ void f_from_state(const Dev<T>& d, const T (&st)[12], T (&f)[9]) {
     const T dr = st[0], r = add_rn(d.rho0, dr), ux = st[1], uy = st[2];
+    if constexpr (sizeof(T) == 4) {
+        T x[9];
+        pops_to(feq_x(dr, r, ux, uy), x);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = fma_rn(d.kneq, st[3 + i], mul_rn(w_of<T>(i), x[i]));
+        return;
+    }
     const T q = mul_rn(T(-1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
     f[0] = fma_rn(d.kneq, st[3], mul_rn(w_of<T>(0), fma_rn(r, q, dr)));
 #pragma unroll
@@ -230,7 +243,7 @@ __global__ void __launch_bounds__(128) k_refill(Dev<T> d, StepArgs a, int refill
             const T l0 = T(lam[0]), l1 = T(lam[1]), l2 = T(lam[2]);
             const T *a0 = in + (int64_t)kRec * v[0], *a1 = in + (int64_t)kRec * v[1], *a2 = in + (int64_t)kRec * v[2];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = fma_rn(l2, a2[i], fma_rn(l1, a1[i], mul_rn(l0, a0[i])));
+            for (int i = 0; i < 9; ++i) f[i] = fma_rn(l2, a2[i], fma_rn(l0, a0[i], mul_rn(l1, a1[i])));
             type = 3;
             donor = k;
         } else if (fabs(qx) <= d.half_L && fabs(qy) <= d.half_T) {
@@ -1845,22 +1858,27 @@ __device__ __forceinline__ float duo_other(float v) { return __shfl_xor_sync(0xf
 __device__ __forceinline__ Pr<float> duo_axes(const Duo& Q, float x, float y) {
     return pk(Q.q ? add_rn(x, y) : x, Q.q ? sub_rn(y, x) : y);
 }
-// moments of the set whose pairs (a, b) each lane holds, f0 in lane 0's e
-__device__ __forceinline__ void duo_moments(const Duo& Q, Pr<float> a, Pr<float> b, float e, float& m0, float& mx,
-                                            float& my) {
-    const Pr<float> s = padd(a, b), dd = psub(a, b);
-    const float t = add_rn(px(s), py(s));
-    const float vx = Q.q ? sub_rn(px(dd), py(dd)) : px(dd), vy = Q.q ? add_rn(px(dd), py(dd)) : py(dd);
-    const float f0 = __shfl_sync(0xffffffffu, e, 0, 2), t2 = duo_other(t), wx = duo_other(vx), wy = duo_other(vy);
-    m0 = add_rn(f0, add_rn(t, t2));
-    mx = add_rn(vx, wx);
-    my = add_rn(vy, wy);
+// moments of the set whose pairs (a, b) each lane holds, f0 in lane 0's e: the
+// sums run over directions 0 .. 4 on lane 0, then 5 .. 8 on lane 1
+__device__ __forceinline__ void duo_moments(Pr<float> a, Pr<float> b, float e, float& m0, float& mx, float& my) {
+    auto from = [](float v, int lane) { return __shfl_sync(0xffffffffu, v, lane, 2); };
+    const float f1 = px(a), f2 = py(a), f3 = px(b), f4 = py(b);
+    m0 = from(add_rn(add_rn(add_rn(add_rn(e, f1), f2), f3), f4), 0);
+    mx = from(sub_rn(f1, f3), 0);
+    my = from(sub_rn(f2, f4), 0);
+    m0 = from(add_rn(add_rn(add_rn(add_rn(m0, f1), f2), f3), f4), 1);
+    mx = from(add_rn(sub_rn(sub_rn(add_rn(mx, f1), f2), f3), f4), 1);
+    my = from(sub_rn(sub_rn(add_rn(add_rn(my, f1), f2), f3), f4), 1);
 }
-// the pairs minus w (G +- 3 c . (x, y))
-__device__ __forceinline__ void duo_sub_lin(const Duo& Q, Pr<float> G, float x, float y, Pr<float>& a, Pr<float>& b) {
-    const Pr<float> H = pmul(pk(3.0f, 3.0f), duo_axes(Q, x, y));
-    a = pfma(Q.w, padd(G, H), a);
-    b = pfma(Q.w, psub(G, H), b);
+// the pairs minus w (g + 3 c . (x, y) + 4.5 Q)
+template <bool kQuad>
+__device__ __forceinline__ void duo_sub_lin(const Duo& Q, float g, float x, float y, Pr<float> quad, Pr<float>& a,
+                                            Pr<float>& b) {
+    const Pr<float> c = duo_axes(Q, x, y), gg = pk(g, g), h = pk(4.5f, 4.5f);
+    Pr<float> A = pfma(pk(3.0f, 3.0f), c, gg), B = pfma(pk(-3.0f, -3.0f), c, gg);
+    if (kQuad) A = pfma(h, quad, A), B = pfma(h, quad, B);
+    a = pfma(Q.w, A, a);
+    b = pfma(Q.w, B, b);
 }
 
 template <bool kRecord, bool kOuterFv>
@@ -1918,15 +1936,15 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
         Ce = pfma(cP, Pe, Ce);
         // collision sums: lane 0 has (Cf_0, Z0), lane 1 (Z1, Z2)
         float dr, jx, jy, n0 = px(Ce);
-        duo_moments(Q, Ca, Cb, n0, dr, jx, jy);
+        duo_moments(Ca, Cb, n0, dr, jx, jy);
         const float zo = py(Ce), zx = duo_other(zo), Z0 = q ? zx : zo, Z2 = q ? zo : zx;
         const float zs = add_rn(Z0, Z2), q0 = fma_rn(-1.5f, zs, dr);
-        const Pr<float> u = pk(q ? fma_rn(2.0f, px(Ce), zs) : Z0, q ? fma_rn(-2.0f, px(Ce), zs) : Z2);
-        duo_sub_lin(Q, pfma(pk(4.5f, 4.5f), u, pk(q0, q0)), jx, jy, Ca, Cb);
+        const Pr<float> u = pk(q ? add_rn(fma_rn(2.0f, px(Ce), Z0), Z2) : Z0, q ? add_rn(fma_rn(-2.0f, px(Ce), Z0), Z2) : Z2);
+        duo_sub_lin<true>(Q, q0, jx, jy, u, Ca, Cb);
         n0 = fma_rn(-w_of<float>(0), q0, n0);
         float m0, mx, my;
-        duo_moments(Q, Ca, Cb, n0, m0, mx, my);
-        duo_sub_lin(Q, pk(m0, m0), mx, my, Ca, Cb);
+        duo_moments(Ca, Cb, n0, m0, mx, my);
+        duo_sub_lin<false>(Q, m0, mx, my, Ca, Ca, Cb);
         n0 = fma_rn(-w_of<float>(0), m0, n0);
         a = pfma(Q.dt1, pfma(Q.iv1, Ca, Sa), Pa);
         b = pfma(Q.dt2, pfma(Q.iv2, Cb, Sb), Pb);
@@ -1941,14 +1959,15 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
         if (__any_sync(0xffffffffu, wall)) {
             const float* uv = reinterpret_cast<const float*>(sm + L.uv);
             const float U = uv[m], V = uv[d.n_sub + m];
-            duo_moments(Q, a, b, f0, dr, jx, jy);
+            duo_moments(a, b, f0, dr, jx, jy);
             const float rho = add_rn(d.rho0, dr), inv = 1.0f / rho;
             const float ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
-            const float dx = sub_rn(U, ux), dy = sub_rn(V, uy), sx = add_rn(U, ux), sy = add_rn(V, uy);
-            const float bb = mul_rn(-1.5f, fma_rn(dx, sx, mul_rn(dy, sy)));
-            const Pr<float> dv = duo_axes(Q, dx, dy);
-            const Pr<float> G = pfma(pmul(pk(4.5f, 4.5f), dv), duo_axes(Q, sx, sy), pk(bb, bb)), H = pmul(pk(3.0f, 3.0f), dv);
-            const float wr = mul_rn(q ? w_of<float>(5) : w_of<float>(1), rho);
+            const float usq = fma_rn(ux, ux, mul_rn(uy, uy)), Usq = fma_rn(U, U, mul_rn(V, V));
+            const float wl = q ? w_of<float>(5) : w_of<float>(1), w0 = w_of<float>(0);
+            Pr<float> Xa, Xb, Ya, Yb;
+            feq_x(duo_axes(Q, U, V), dr, rho, Usq, Xa, Xb);
+            feq_x(duo_axes(Q, ux, uy), dr, rho, usq, Ya, Yb);
+            const float X0 = fma_rn(rho, mul_rn(-1.5f, Usq), dr), Y0 = fma_rn(rho, mul_rn(-1.5f, usq), dr);
             if constexpr (kRecord) {
                 if (rec && wall) {
                     if (q == 0) rec[kAdjWall] = rho;
@@ -1956,9 +1975,9 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
                 }
             }
             if (wall) {
-                a = pfma(pk(wr, wr), padd(G, H), a);
-                b = pfma(pk(wr, wr), psub(G, H), b);
-                f0 = fma_rn(mul_rn(w_of<float>(0), rho), bb, f0);
+                a = padd(a, pfma(pk(wl, wl), Xa, pmul(pk(-wl, -wl), Ya)));
+                b = padd(b, pfma(pk(wl, wl), Xb, pmul(pk(-wl, -wl), Yb)));
+                f0 = add_rn(f0, fma_rn(w0, X0, mul_rn(-w0, Y0)));
             }
         }
         e = pk(f0, 0.0f);
@@ -1968,21 +1987,19 @@ __device__ __forceinline__ void duo_node(const Dev<float>& d, const unsigned cha
         const float th = float(m + 1) / float(d.n_sub), t0 = sub_rn(1.0f, th);
         auto at = [&](int j) { return fma_rn(t0, sn[j], mul_rn(th, sn[12 + j])); };
         const float dr = at(0), ux = at(1), uy = at(2), rho = add_rn(d.rho0, dr);
-        const float qq = mul_rn(-1.5f, fma_rn(ux, ux, mul_rn(uy, uy)));
-        const Pr<float> c = duo_axes(Q, ux, uy), rr = pk(rho, rho), kk = pk(d.kneq, d.kneq);
-        const float wl = q ? w_of<float>(5) : w_of<float>(1);
-        const Pr<float> w = pk(wl, wl);
-        const Pr<float> G = pfma(rr, pfma(pmul(pk(4.5f, 4.5f), c), c, pk(qq, qq)), pk(dr, dr)),
-                        H = pmul(rr, pmul(pk(3.0f, 3.0f), c));
-        a = pfma(kk, pk(at(4 + ia), at(5 + ia)), pmul(w, padd(G, H)));
-        b = pfma(kk, pk(at(6 + ia), at(7 + ia)), pmul(w, psub(G, H)));
-        e = pk(fma_rn(d.kneq, at(3), mul_rn(w_of<float>(0), fma_rn(rho, qq, dr))), 0.0f);
+        const float usq = fma_rn(ux, ux, mul_rn(uy, uy)), wl = q ? w_of<float>(5) : w_of<float>(1);
+        const Pr<float> w = pk(wl, wl), kk = pk(d.kneq, d.kneq);
+        Pr<float> Xa, Xb;
+        feq_x(duo_axes(Q, ux, uy), dr, rho, usq, Xa, Xb);
+        a = pfma(kk, pk(at(4 + ia), at(5 + ia)), pmul(w, Xa));
+        b = pfma(kk, pk(at(6 + ia), at(7 + ia)), pmul(w, Xb));
+        e = pk(fma_rn(d.kneq, at(3), mul_rn(w_of<float>(0), fma_rn(rho, mul_rn(-1.5f, usq), dr))), 0.0f);
     }
     __syncwarp();
     float dr, jx, jy;
-    duo_moments(Q, a, b, px(e), dr, jx, jy);
+    duo_moments(a, b, px(e), dr, jx, jy);
     const float inv = 1.0f / add_rn(d.rho0, dr), ux = mul_rn(jx, inv), uy = mul_rn(jy, inv);
-    e = q ? pk(mul_rn(jx, uy), mul_rn(jy, uy)) : pk(px(e), mul_rn(jx, ux));
+    e = q ? pk(mul_rn(mul_rn(jx, jy), inv), mul_rn(mul_rn(jy, jy), inv)) : pk(px(e), mul_rn(mul_rn(jx, jx), inv));
     if constexpr (kRecord) {
         if (rec && m + 1 < d.n_sub) rec[(int64_t)d.n * kAdjRec + kAdjU + q] = q ? uy : ux;
     }
@@ -2051,14 +2068,16 @@ __device__ __forceinline__ void far_chunk(const Dev<float>& d, const FarArgs<flo
     }
     if (!mine) return;
     if (interior) {
-        Pr<float> f[9], o[9];
+        float f[9], o0[9], o1[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
-            f[i] = cx_of(i) == 0 ? pk(p[i].x, p[i].y) : (cx_of(i) == 1 ? pk(edge[i], p[i].x) : pk(p[i].y, edge[i]));
-        bgk_pair(f, d.rho0, omega, o);
+        for (int i = 0; i < 9; ++i) f[i] = cx_of(i) == 0 ? p[i].x : (cx_of(i) == 1 ? edge[i] : p[i].y);
+        bgk_dev(f, d.rho0, omega, o0);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = cx_of(i) == 0 ? p[i].y : (cx_of(i) == 1 ? p[i].x : edge[i]);
+        bgk_dev(f, d.rho0, omega, o1);
         const int64_t s0 = (int64_t)y * d.pitch + x0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) *reinterpret_cast<unsigned long long*>(B + i * d.plane + s0) = o[i].v;
+        for (int i = 0; i < 9; ++i) *reinterpret_cast<float2*>(B + i * d.plane + s0) = make_float2(o0[i], o1[i]);
     } else {
         for (int k = 0; k < 2; ++k) {
             const int x = x0 + k;
