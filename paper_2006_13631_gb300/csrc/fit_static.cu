@@ -11,7 +11,8 @@
 // That array (kFitBlocks x 8 doubles) exists on every GPU that loads the
 // library and stays there until the process exits.  All calls on a device
 // share it and it keeps the last call's contents; every slot a call reads
-// is written earlier in the same call, so nothing has to be cleared, but
+// is written earlier in the same call, or is the count of finished blocks,
+// which each launch leaves at zero, so nothing has to be cleared, but
 // calls whose work overlaps on the GPU (different streams, or different host
 // threads) race on it and must be serialised by the caller.
 #include <cuda_runtime.h>
@@ -32,7 +33,7 @@ constexpr int64_t kFitMaxSamples = (int64_t)1 << 26;
 constexpr int kMaxDevices = 64;
 
 // partial sums of each block (5 used by the first pass, 1 by the residual
-// pass) and, in the last row, the final results
+// pass) and, in the last row, the final results and the count of blocks done
 static __device__ __align__(256) double g_fit_scratch[(kFitBlocks + 1) * 8];
 
 // Device address of g_fit_scratch per device, with the unique id of the
@@ -91,11 +92,52 @@ cudaError_t scratch_address(double** out) {
     return cudaSuccess;
 }
 
+// Sum of a per-thread value over the block, in every thread of warp 0's lane 0:
+// a shuffle tree per warp, then one over the warps' sums.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = threadIdx.x < kFitThreads / 32 ? sh[threadIdx.x] : 0.0;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int w = kFitThreads / 64; w > 0; w >>= 1) v += __shfl_down_sync(0xffffffffu, v, w);
+    }
+    __syncthreads();
+    return v;
+}
+
+// Whether this block is the last of the grid to get here, its partial sums and
+// every other block's being visible then.  The counter (the scratch array's
+// last slot) is zero between launches: the last block puts it back.
+__device__ __forceinline__ bool last_block(double* scratch, bool& last_sh) {
+    if (threadIdx.x == 0) {
+        unsigned* ticket = reinterpret_cast<unsigned*>(scratch + 8 * kFitBlocks + 7);
+        __threadfence();
+        last_sh = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last_sh) *ticket = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    return last_sh;
+}
+
 // Per-block sums over samples t0..t1 of s^2, s c, c^2, F s, F c with
-// s = sin(w t), c = cos(w t), F = samples[t * stride].
+// s = sin(w t), c = cos(w t), F = samples[t * stride]; the last block adds
+// them in a fixed order and solves the 2x2 normal equations: a, b into the
+// result row, and in its slot 3 whether the system is regular.
+// With s = sin(w t), c = cos(w t), s^2 + c^2 = 1, so S_ss + S_cc is the sample
+// count n and det = S_ss S_cc - S_sc^2 <= n^2 / 4; det below 1e-12 n^2 means
+// the two columns are (nearly) dependent, e.g. w a multiple of pi, where
+// sin(w t) vanishes at every integer t.
+// Bound by the FP64 issue rate (a sincos is some 50 FP64 instructions, one per 19
+// cycles and SM): one block per SM.  102 400 samples took 116 us in four
+// launches, 25 blocks and serial sums of the partials.
 __global__ void __launch_bounds__(kFitThreads) k_fit_partials(const double* samples, int64_t stride, int64_t t0,
                                                              int64_t t1, double omega, double* scratch) {
-    __shared__ double sh[5][kFitThreads];
+    __shared__ double sh[kFitThreads / 32];
+    __shared__ bool last_sh;
     double acc[5] = {0, 0, 0, 0, 0};
     for (int64_t t = t0 + blockIdx.x * (int64_t)kFitThreads + threadIdx.x; t <= t1;
          t += (int64_t)gridDim.x * kFitThreads) {
@@ -108,38 +150,29 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_partials(const double* samp
         acc[3] += F * s;
         acc[4] += F * c;
     }
-    for (int j = 0; j < 5; ++j) sh[j][threadIdx.x] = acc[j];
-    __syncthreads();
-    for (int w = kFitThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int j = 0; j < 5; ++j) sh[j][threadIdx.x] += sh[j][threadIdx.x + w];
-        __syncthreads();
+    for (int j = 0; j < 5; ++j) {
+        const double v = block_sum(acc[j], sh);
+        if (threadIdx.x == 0) scratch[8 * blockIdx.x + j] = v;
     }
-    if (threadIdx.x < 5) scratch[8 * blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
+    if (!last_block(scratch, last_sh)) return;
+    double s[5];
+    for (int j = 0; j < 5; ++j)
+        s[j] = block_sum(threadIdx.x < gridDim.x ? __ldcg(scratch + 8 * threadIdx.x + j) : 0.0, sh);
+    if (threadIdx.x == 0) {
+        const double det = s[0] * s[2] - s[1] * s[1];
+        const double n = s[0] + s[2];
+        double* res = scratch + 8 * kFitBlocks;
+        res[0] = (s[3] * s[2] - s[4] * s[1]) / det;
+        res[1] = (s[4] * s[0] - s[3] * s[1]) / det;
+        res[3] = (isfinite(det) && det > 1e-12 * n * n) ? 1.0 : 0.0;
+    }
 }
 
-// Fixed-order sum of the block partials, then the 2x2 normal equations:
-// a, b into the result row, and in its slot 3 whether the system is regular.
-// With s = sin(w t), c = cos(w t), s^2 + c^2 = 1, so S_ss + S_cc is the sample
-// count n and det = S_ss S_cc - S_sc^2 <= n^2 / 4; det below 1e-12 n^2 means
-// the two columns are (nearly) dependent, e.g. w a multiple of pi, where
-// sin(w t) vanishes at every integer t.
-__global__ void k_fit_solve(int nblocks, double* scratch) {
-    if (threadIdx.x != 0) return;
-    double s[5] = {0, 0, 0, 0, 0};
-    for (int b = 0; b < nblocks; ++b)
-        for (int j = 0; j < 5; ++j) s[j] += scratch[8 * b + j];
-    const double det = s[0] * s[2] - s[1] * s[1];
-    const double n = s[0] + s[2];
-    double* res = scratch + 8 * kFitBlocks;
-    res[0] = (s[3] * s[2] - s[4] * s[1]) / det;
-    res[1] = (s[4] * s[0] - s[3] * s[1]) / det;
-    res[3] = (isfinite(det) && det > 1e-12 * n * n) ? 1.0 : 0.0;
-}
-
+// the residual's sum of squares, likewise
 __global__ void __launch_bounds__(kFitThreads) k_fit_resid_partials(const double* samples, int64_t stride, int64_t t0,
                                                                    int64_t t1, double omega, double* scratch) {
-    __shared__ double sh[kFitThreads];
+    __shared__ double sh[kFitThreads / 32];
+    __shared__ bool last_sh;
     const double* res = scratch + 8 * kFitBlocks;
     const double a = res[0], b = res[1];
     double acc = 0.0;
@@ -150,20 +183,11 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_resid_partials(const double
         const double e = samples[t * stride] - (a * s + b * c);
         acc += e * e;
     }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kFitThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) scratch[8 * blockIdx.x + 5] = sh[0];
-}
-
-__global__ void k_fit_rms(int nblocks, int64_t count, double* scratch) {
-    if (threadIdx.x != 0) return;
-    double r2 = 0.0;
-    for (int b = 0; b < nblocks; ++b) r2 += scratch[8 * b + 5];
-    scratch[8 * kFitBlocks + 2] = sqrt(r2 / (double)count);
+    acc = block_sum(acc, sh);
+    if (threadIdx.x == 0) scratch[8 * blockIdx.x + 5] = acc;
+    if (!last_block(scratch, last_sh)) return;
+    const double r2 = block_sum(threadIdx.x < gridDim.x ? __ldcg(scratch + 8 * threadIdx.x + 5) : 0.0, sh);
+    if (threadIdx.x == 0) scratch[8 * kFitBlocks + 2] = sqrt(r2 / (double)(t1 - t0 + 1));
 }
 
 }  // namespace
@@ -186,13 +210,14 @@ extern "C" int hlbm_fit_static(const double* samples, int64_t stride, int64_t t0
     }
     double* scratch = nullptr;
     if (scratch_address(&scratch) != cudaSuccess) return HLBM_ECUDA;
-    const int nblocks = (int)((count + kFitThreads * 16 - 1) / (kFitThreads * 16)) < kFitBlocks
-                            ? (int)((count + kFitThreads * 16 - 1) / (kFitThreads * 16))
-                            : kFitBlocks;
+    int dev = 0, sms = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return HLBM_ECUDA;
+    const int64_t most = sms < kFitBlocks ? sms : kFitBlocks, need = (count + kFitThreads - 1) / kFitThreads;
+    const int nblocks = (int)(need < most ? need : most);
     k_fit_partials<<<nblocks, kFitThreads, 0, s>>>(samples, stride, t0, t1, omega, scratch);
-    k_fit_solve<<<1, 32, 0, s>>>(nblocks, scratch);
     k_fit_resid_partials<<<nblocks, kFitThreads, 0, s>>>(samples, stride, t0, t1, omega, scratch);
-    k_fit_rms<<<1, 32, 0, s>>>(nblocks, count, scratch);
     // a rejected launch must not let the read-back return the previous
     // call's results, which the shared array still holds
     e = cudaGetLastError();
