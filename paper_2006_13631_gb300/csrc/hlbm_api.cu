@@ -49,7 +49,7 @@ struct hlbm {
     std::vector<void*> tile_blocks;  // device tables of the current FV tiling
     bool use_smem = false;      // a tile kernel (else the global-memory kernel)
     int fv_kind = HLBM_FV_GLOBAL;  // HLBM_FV_* in use
-    int fv_depth = 2;              // deep tiles: sub-steps between exchanges asked for (the largest that fits up to it)
+    int fv_depth = 0;              // deep tiles: sub-steps between exchanges asked for (the largest that fits up to it; 0: default_depth)
     double mxmin = 0, mxmax = 0, mymin = 0, mymax = 0;
     int nnz = 0, nseg = 0;
 
@@ -752,11 +752,26 @@ int default_tiles(int n, int sms) {
     return std::max(1, std::min(sms, (n + least - 1) / least));
 }
 
-// Computed slots of an FP64 tile up to which four lanes share a node (K = 2;
-// FV us per sub-step with quads / with a node per lane: 7.2 / 15.5 on 3008
-// nodes (152 tiles of at most 76 slots), 9.0 / 15.6 on 5464, 11.7 / 15.6 on
-// 9096, 16.8 / 18.1 on 13 188 (205 slots, about 150 computed); beyond, a quad
-// warp's larger total of FP64 instructions costs more than it hides).
+// Sub-steps between two exchanges of the deep tiles: 2, where the ghost layer
+// recomputed in between costs less than an exchange (some 1 us).  An FP64 tile
+// of more than 18 nodes is bound by the SM's FP64 issue rate, and the ghosts
+// are work: FV us per sub-step with K = 1 / K = 2 at 16 nodes per tile 6.92 /
+// 6.80 (1344 nodes), 7.21 / 6.89 (2280); above, 7.14 / 7.27 (2748 nodes, 19
+// per tile), 7.13 / 7.25 (3008), 7.21 / 7.87 (3920), 7.48 / 8.93 (5464), 9.9 /
+// 11.8 (9096), 13.0 / 16.8 (13 188), 21.1 / 22.6 (24 380).  With outer_fv the
+// update is a node per lane, whose chain the ghosts hide in: 16.9 / 15.0 (5464).
+// FP32 with 1 / 2 / 3: 2.09 / 1.60 / 1.57 (2588 nodes), 2.26 / 2.00 / 2.05
+// (24 380), 2.69 / 2.43 / 2.37 (45 304).
+template <typename T>
+int default_depth(int tile_cap, int outer_fv) {
+    return sizeof(T) == 8 && tile_cap > 18 && !outer_fv ? 1 : 2;
+}
+
+// Computed slots of an FP64 tile up to which four lanes share a node (FV us
+// per sub-step with quads / with a node per lane: 7.2 / 15.5 on 3008 nodes and
+// 11.7 / 15.6 on 9096, K = 2; with K = 1 21.8 / 21.2 on 24 380 nodes (161 per
+// tile), 29.2 / 27.7 on 35 256: there the quads' larger total of FP64
+// instructions costs more than it hides).
 constexpr int kDeepQuadMax = 160;
 
 // FV tiles: equal ranges of the Morton-ordered nodes.  The shared-memory
@@ -833,8 +848,10 @@ int build_tiles(hlbm* h, int n_tiles_req, int kind = HLBM_FV_AUTO) {
     bool deep_ok = false;
     int deep_quads = 0;
     if ((want == HLBM_FV_AUTO || (want == HLBM_FV_DEEP && h->patch.outer_fv == 0)) && max_row - 1 <= 7) {
-        // a pack of FP64 solvers fills the SMs' FP64 pipes, and recomputed ghosts cost more than exchanges
-        const int depth = kind != HLBM_FV_AUTO && sizeof(T) == 8 ? 1 : std::min(h->fv_depth, kDeepMaxK);
+        // a pack of FP64 solvers fills the SMs' FP64 pipes, as large tiles do
+        const int depth = kind != HLBM_FV_AUTO && sizeof(T) == 8 ? 1
+                          : h->fv_depth > 0                      ? std::min(h->fv_depth, kDeepMaxK)
+                                                                 : default_depth<T>(tile_cap, h->patch.outer_fv);
         for (int K = depth; K >= 1 && !deep_ok; --K) {
             if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), fv_deep_early<T>(), deep)) continue;
             // FP64, few computed slots: four lanes per node

@@ -106,3 +106,34 @@ def test_outer_node_sums_agree_bit_for_bit(mesh_args, dtype):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b)
+
+
+# the sizes next to each line of the dispatch: FP64 tiles of 18 and of 19 nodes
+# (exchange interval 2 and 1), of at most 160 and of 161 (four lanes per node or
+# one), FP32 tiles of few computed slots and of more than 384 (two lanes or one)
+@pytest.mark.parametrize("dtype,n_L,n_layers,h1,nodes,depth", [
+    ("f64", 75, 14, 0.3, 2716, 2), ("f64", 78, 14, 0.25, 2748, 1), ("f64", 240, 40, 0.08, None, 1),
+    ("f64", 250, 40, 0.08, 24380, 1), ("f32", 74, 13, 0.3, 2436, 2), ("f32", 400, 50, 0.06, 46600, 2),
+    ("f32", 420, 55, 0.06, 54612, 2)])
+def test_deep_forms_agree_bit_for_bit(dtype, n_L, n_layers, h1, nodes, depth):
+    """The forms of the deep kernel and the global-memory kernel run the same
+    arithmetic: equal fields after a few steps."""
+    from paper_2006_13631_gb300 import Solver
+
+    w = _case(dtype, dict(n_L=n_L, n_T=2, n_layers=n_layers, h1=h1, d_out=4.0), n_sub=25)
+    mesh, rho = w.mesh(), w.rho_init()
+    assert nodes is None or mesh.n_nodes == nodes
+    got = []
+    for kern in (1, 0):
+        w.fv_kernel = kern
+        s = Solver(w, mesh=mesh, rho_init=rho)
+        if kern == 0:
+            assert s.info()["fv_kernel"] == 4
+            if s.info()["n_tiles"] == 152:
+                assert s.info()["fv_depth"] == depth
+        s.step(4)
+        assert s.status == 0
+        got.append(tuple(s.fields()) + (s.patch_f(), s.force()[1]))
+        s.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
