@@ -338,8 +338,9 @@ int hlbm_set_fv_depth(hlbm_t* h, int32_t depth);
  * motion, the FV launch of step t also runs step t+1's stream-collide of
  * every lattice node outside step t+1's window and the nodes pulling from it
  * (the only nodes that step t+1's relocation, classification and eq. 178
- * feed change), on warps of its own; step t+1's stream-collide then covers
- * that rectangle alone.  The results are the same bits either way.  Across
+ * feed change), on warps of its own, or where the patch leaves SMs without
+ * a tile, on those; step t+1's stream-collide then covers that rectangle
+ * alone.  The results are the same bits either way.  Across
  * hlbm_step calls the precomputed part is kept (hlbm_load, hlbm_clear_status
  * and an injected lattice fault drop it).  enable = 0 runs each step's
  * stream-collide whole, before its FV launch. */
@@ -348,8 +349,8 @@ int hlbm_set_overlap(hlbm_t* h, int32_t enable);
 /* The share (0, 1] of the lattice rows, from y = 0, whose part away from the
  * patch the FV launch streams under the overlap; the next step's
  * stream-collide covers the other rows with its rectangle (default 0.85:
- * the FV launch then ends about when its far lattice does).  Results do not
- * change.  HLBM_EINVAL outside (0, 1]. */
+ * the FV launch then ends about when its far lattice does; SMs without a
+ * tile take every row).  Results do not change.  HLBM_EINVAL outside (0, 1]. */
 int hlbm_set_overlap_share(hlbm_t* h, double share);
 
 /* Per-phase device time, measured with CUDA events recorded on the
@@ -394,10 +395,10 @@ int hlbm_sweep_fv_time(hlbm_sweep_t* w, int64_t nsteps, double* fv_ms);
  * the same precision whose sub-step counts lie within 25 % of each other,
  * up to 16, are retiled so that together they take one block per SM, and
  * each lattice step runs their FV sub-steps in one cooperative launch of the
- * tensor-memory kernel (each solver keeps its own tables, counters and
- * buffers).  Solvers with outer_fv = 1 or a forced fv_kernel stay alone.
- * A group whose tiles the tensor-memory kernel cannot hold even with more,
- * smaller tiles stays unpacked.  enable = 0 undoes it (the tuner's tiling,
+ * deep-tile kernel, or of the tensor-memory kernel where the tiles are too
+ * large for it (each solver keeps its own tables, counters and buffers).
+ * Solvers with outer_fv = 1 or a forced fv_kernel stay alone.  A group whose
+ * tiles neither can hold even with more, smaller tiles stays unpacked.  enable = 0 undoes it (the tuner's tiling,
  * or the default one before hlbm_sweep_tune).  n_packs (may be NULL) receives
  * the number of packs.  Results do not change: a node's arithmetic does not
  * depend on its tile or launch.  hlbm_sweep_tune after this call undoes it. */

@@ -1318,7 +1318,7 @@ cudaError_t launch_fv_tmem(const Dev<T>& d, const StepArgs& a, cudaStream_t s) {
 // (with the counters and cp.async copies of the other kernels, 3.8 us per
 // sub-step on a 2588-node FP32 patch at K = 2, 3.7 on 45 304 nodes and 28 on
 // 3008 FP64 nodes; with the packets and the pair arithmetic 2.4, 2.6 and
-// 17.7).  Tags are unique over the solver's life
+// 17.7, and with several lanes per node, below, 1.6, 2.4 and 7.1).  Tags are unique over the solver's life
 // (StepArgs::xtag), so a packet left by an earlier launch is never taken for
 // a new one.  Packets alternate between two buffers; a tile overwrites the
 // packets of exchange e when it sends exchange e + 2, after having received
@@ -1366,7 +1366,7 @@ int fv_deep_tmem_slots() {
 // others, while the ghosts are on their way: when they fill the FV warps; fewer
 // are left for after the wait, since one pass over all slots then takes no
 // longer than over a part.  (FP64 from 64 nodes on: the FP64 pipe is busy
-// either way; 25.5 instead of 22.6 us per sub-step on 24 380 nodes.)
+// either way; 25.5 instead of 22.6 us per sub-step on 24 380 nodes, K = 2.)
 template <typename T>
 int fv_deep_early() {
     return kDeepFv<T>;
@@ -1826,8 +1826,9 @@ __device__ __forceinline__ void quad_node(const Dev<double>& d, const unsigned c
 // tile), 1.0 / K more for the exchange.  Where a tile's computed slots fit, two
 // lanes share a node: lane 0 holds the pairs A, B (axes) and E, lane 1 C, D
 // (diagonals) and F, each with its share of the row in registers; the sums
-// over directions take one shuffle.  Every value is formed by the expression
-// of fv_node.cuh, so the bits are those of a node per lane.
+// over directions take one shuffle: 1.6 us per sub-step on that patch, 2.4 on
+// 45 304 nodes.  Every value is formed by the expression of fv_node.cuh, so the
+// bits are those of a node per lane.
 constexpr int kDuoThreads = 768;  // 80 registers a thread
 constexpr int kDuoSlots = kDuoThreads / 2;
 struct Duo {
