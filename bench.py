@@ -198,6 +198,7 @@ _KERNEL_SOURCES = {
                         "// ---------------------------------------------------------------- geometry")],
     "fv_deep": [("k_patch.cu", "// ----------------------------------------------------------- FV steps",
                  "// ------------------------------------------------------------- force"),
+                ("fv_node.cuh", "// Arithmetic of one patch node's FV update", "}  // namespace hk"),
                 ("hlbm_dev.cuh", "// ---------------------------------------------------------------- D2Q9",
                  "// ---------------------------------------------------------------- layout"),
                 ("hlbm_dev.cuh", "// ---------------------------------------------------------------- lattice storage",
