@@ -2015,6 +2015,7 @@ int adj_snapshot(hlbm* h, AdjCkpt& c, bool restore) {
         h->si = c.si;
         h->ui = c.ui;
         h->fi = c.fi;
+        h->far_ready = false;  // the successor buffer holds what a later step wrote
     }
     auto cp = [&](void* dst, const void* src, size_t n) { return cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToDevice, s); };
     cudaError_t e;
