@@ -11,9 +11,9 @@
 // That array (kFitBlocks x 8 doubles) exists on every GPU that loads the
 // library and stays there until the process exits.  All calls on a device
 // share it and it keeps the last call's contents; every slot a call reads
-// is written earlier in the same call, or is the count of finished blocks,
-// which each launch leaves at zero, so nothing has to be cleared, but
-// calls whose work overlaps on the GPU (different streams, or different host
+// is written earlier in the same call, the counts of finished blocks by the
+// memset that begins it, so that no call depends on how an earlier one ended.
+// Calls whose work overlaps on the GPU (different streams, or different host
 // threads) race on it and must be serialised by the caller.
 #include <cuda_runtime.h>
 
@@ -31,9 +31,11 @@ constexpr int kFitBlocks = 256;      // blocks of the partial-sum passes
 constexpr int kFitThreads = 256;
 constexpr int64_t kFitMaxSamples = (int64_t)1 << 26;
 constexpr int kMaxDevices = 64;
+constexpr int kFitSumsDone = 8 * kFitBlocks + 6, kFitResidDone = kFitSumsDone + 1;  // the counts' slots
 
 // partial sums of each block (5 used by the first pass, 1 by the residual
-// pass) and, in the last row, the final results and the count of blocks done
+// pass) and, in the last row, the final results and the two passes' counts of
+// blocks done
 static __device__ __align__(256) double g_fit_scratch[(kFitBlocks + 1) * 8];
 
 // Device address of g_fit_scratch per device, with the unique id of the
@@ -109,14 +111,11 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 // Whether this block is the last of the grid to get here, its partial sums and
-// every other block's being visible then.  The counter (the scratch array's
-// last slot) is zero between launches: the last block puts it back.
-__device__ __forceinline__ bool last_block(double* scratch, bool& last_sh) {
+// every other block's being visible then.  The pass's counter starts at zero.
+__device__ __forceinline__ bool last_block(double* scratch, int counter, bool& last_sh) {
     if (threadIdx.x == 0) {
-        unsigned* ticket = reinterpret_cast<unsigned*>(scratch + 8 * kFitBlocks + 7);
         __threadfence();
-        last_sh = atomicAdd(ticket, 1u) == gridDim.x - 1;
-        if (last_sh) *ticket = 0u;
+        last_sh = atomicAdd(reinterpret_cast<unsigned*>(scratch + counter), 1u) == gridDim.x - 1;
         __threadfence();
     }
     __syncthreads();
@@ -132,8 +131,9 @@ __device__ __forceinline__ bool last_block(double* scratch, bool& last_sh) {
 // the two columns are (nearly) dependent, e.g. w a multiple of pi, where
 // sin(w t) vanishes at every integer t.
 // Bound by the FP64 issue rate (a sincos is some 50 FP64 instructions, one per 19
-// cycles and SM): one block per SM.  102 400 samples took 116 us in four
-// launches, 25 blocks and serial sums of the partials.
+// cycles and SM): one block per SM.  A call on 102 400 samples takes 52 us (116
+// in four launches with 25 blocks and serial sums of the partials), some 1.5 of
+// them the memset of the counts.
 __global__ void __launch_bounds__(kFitThreads) k_fit_partials(const double* samples, int64_t stride, int64_t t0,
                                                              int64_t t1, double omega, double* scratch) {
     __shared__ double sh[kFitThreads / 32];
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_partials(const double* samp
         const double v = block_sum(acc[j], sh);
         if (threadIdx.x == 0) scratch[8 * blockIdx.x + j] = v;
     }
-    if (!last_block(scratch, last_sh)) return;
+    if (!last_block(scratch, kFitSumsDone, last_sh)) return;
     double s[5];
     for (int j = 0; j < 5; ++j)
         s[j] = block_sum(threadIdx.x < gridDim.x ? __ldcg(scratch + 8 * threadIdx.x + j) : 0.0, sh);
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kFitThreads) k_fit_resid_partials(const double
     }
     acc = block_sum(acc, sh);
     if (threadIdx.x == 0) scratch[8 * blockIdx.x + 5] = acc;
-    if (!last_block(scratch, last_sh)) return;
+    if (!last_block(scratch, kFitResidDone, last_sh)) return;
     const double r2 = block_sum(threadIdx.x < gridDim.x ? __ldcg(scratch + 8 * threadIdx.x + 5) : 0.0, sh);
     if (threadIdx.x == 0) scratch[8 * kFitBlocks + 2] = sqrt(r2 / (double)(t1 - t0 + 1));
 }
@@ -216,6 +216,7 @@ extern "C" int hlbm_fit_static(const double* samples, int64_t stride, int64_t t0
         return HLBM_ECUDA;
     const int64_t most = sms < kFitBlocks ? sms : kFitBlocks, need = (count + kFitThreads - 1) / kFitThreads;
     const int nblocks = (int)(need < most ? need : most);
+    cudaMemsetAsync(scratch + kFitSumsDone, 0, 2 * sizeof(double), s);
     k_fit_partials<<<nblocks, kFitThreads, 0, s>>>(samples, stride, t0, t1, omega, scratch);
     k_fit_resid_partials<<<nblocks, kFitThreads, 0, s>>>(samples, stride, t0, t1, omega, scratch);
     // a rejected launch must not let the read-back return the previous
