@@ -153,7 +153,10 @@ void* dev_alloc(hlbm* h, size_t bytes) {
     } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
         p = nullptr;
     }
-    if (p) h->blocks.push_back(p);
+    if (p)
+        h->blocks.push_back(p);
+    else
+        cudaGetLastError();  // reported as a null pointer, and not again after the next launch
     return p;
 }
 
