@@ -32,7 +32,8 @@ def _stale(target, deps):
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT, exist_ok=True)
-    headers = [os.path.join(CSRC, "hlbm_dev.cuh"), os.path.join(CSRC, "fv_node.cuh"), os.path.join(ROOT, "include", "hlbm.h")]
+    headers = [os.path.join(CSRC, h) for h in ("hlbm_dev.cuh", "fv_node.cuh", "adj_node.cuh", "partition.h")]
+    headers.append(os.path.join(ROOT, "include", "hlbm.h"))
     nvcc = _nvcc()
     jobs = []
     objs = []
