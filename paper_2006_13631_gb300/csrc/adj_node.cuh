@@ -3,8 +3,8 @@
 //
 // Reverse mode of one lattice step, with every decision of the forward step
 // held fixed (node classes, refill types, donor cells and triangles: the map
-// is smooth in the states and parameters between decisions).  All adjoints
-// are FP64.  Notation: for a deviation set f (f_i = f'_i), rho = rho0 + dr,
+// is smooth in the states and parameters between decisions).  Adjoints have the
+// population type; a parameter's sum takes every product in FP64.  Notation: for a deviation set f (f_i = f'_i), rho = rho0 + dr,
 // u = j / rho; the equilibrium's derivatives are
 //   d feq_i / d dr |_u = A_i = w_i (1 + 3 c.u + 4.5 (c.u)^2 - 1.5 u^2),
 //   d feq_i / d u      = B_i = w_i rho (3 c_i + 9 (c.u) c_i - 3 u),
@@ -122,13 +122,11 @@ __device__ __forceinline__ void ffsT(const R (&st)[12], R rho0, R k, const R (&l
     const R rho = rho0 + st[0];
     R a, bx, by;
     feq_ab(st[1], st[2], lf, a, bx, by);
-    R dot = R(0);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         ls[3 + i] = k * lf[i];
-        dot += lf[i] * st[3 + i];
+        lk += double(lf[i] * st[3 + i]);
     }
-    lk += double(dot);
     ls[0] = a;
     ls[1] = rho * bx;
     ls[2] = rho * by;
@@ -181,7 +179,8 @@ __device__ __forceinline__ void aq_feq(const AQuad<T>& Q, T ux, T uy, T la, T lb
 
 // What a quad holds of its node: at outer nodes the lattice state at t and
 // t + 1 (drho, ux, uy, f^neq of the lane's pair and f^neq_0) and the sums of
-// its adjoint (the lane's share: its pair, and f^neq_0 with drho, ux or uy)
+// its adjoint (the lane's share: its pair, and f^neq_0 with drho, ux or uy);
+// kq: in FP32, the lane's products of the sum of kneq at the latest sub-step
 template <typename T>
 struct ANode {
     int k;
@@ -189,6 +188,7 @@ struct ANode {
     bool valid;
     T s0[6], s1[6];
     T g0[4], g1[4];
+    T kq[3];
 };
 // what sub-step m's record gives the lane: its collision sums and the wall moments
 template <typename T>
@@ -198,7 +198,8 @@ struct ARec {
 
 // psi at the quad's node for a sub-step (time fraction th, wall velocity U, V,
 // record r) from the adjoint (la, lb, l0) of the state after it, the outer
-// nodes' feed adjoint, and the parameter terms (1/tau_u, kneq, wall velocity)
+// nodes' feed adjoint, and the parameter terms (1/tau_u, wall velocity, kneq; in
+// FP32 that of kneq is left to adj_kneq)
 template <typename T>
 __device__ __forceinline__ void adj_psi(const Dev<T>& d, const AQuad<T>& Q, ANode<T>& N, const ARec<T>& r, T th, T U, T V,
                                         T la, T lb, T l0, T& pa, T& pb, T& p0, T& l_inv, double& l_kneq, T& l_v) {
@@ -232,12 +233,30 @@ __device__ __forceinline__ void adj_psi(const Dev<T>& d, const AQuad<T>& Q, ANod
                 N.g0[j] += t0 * v[j];
                 N.g1[j] += th * v[j];
             }
-            l_kneq += double(la * st[3] + lb * st[4] + (Q.q == 0 ? l0 * st[5] : T(0)));
+            if constexpr (sizeof(T) == 4) {
+                N.kq[0] = la * st[3];
+                N.kq[1] = lb * st[4];
+                N.kq[2] = Q.q == 0 ? l0 * st[5] : T(0);
+            } else {
+                l_kneq += la * st[3] + lb * st[4] + (Q.q == 0 ? l0 * st[5] : T(0));
+            }
             pa = pb = p0 = T(0);
         }
     }
     if (!N.valid) return;
     l_inv -= d.dt_u * (pa * r.na + pb * r.nb + (Q.q == 0 ? p0 * r.n0 : T(0)));
+}
+// FP32: the outer node's terms of kneq into the FP64 sum, once psi is on its way.
+// (The conversions and FP64 additions within adj_psi: reverse sweep of 160 steps
+// of the 2588-node patch, n = 96, 101 ms instead of 94; an FP32 sum of the three
+// products: 90.5.)
+template <typename T>
+__device__ __forceinline__ void adj_kneq(const ANode<T>& N, double& l_kneq) {
+    if constexpr (sizeof(T) == 4) {
+        if (N.kind != HLBM_NODE_OUTER) return;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) l_kneq += double(N.kq[j]);
+    }
 }
 
 }  // namespace hk

@@ -2975,6 +2975,8 @@ __device__ __forceinline__ ANode<T> adj_node(const Dev<T>& d, const AQuad<T>& Q,
     for (int j = 0; j < 6; ++j) N.s0[j] = N.s1[j] = T(0);
 #pragma unroll
     for (int j = 0; j < 4; ++j) N.g0[j] = N.g1[j] = T(0);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) N.kq[j] = T(0);
     if (N.kind == HLBM_NODE_OUTER) {
         const int64_t no = d.n_outer;
         const T* p = d.snap + d.outer_of[N.k];
@@ -3155,6 +3157,7 @@ __global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const 
             const T* l = lPn + 9 * (int64_t)N.k;
             adj_psi(d, Q, N, r, th, U, V, l[1 + Q.ia], l[1 + Q.ib], Q.q == 0 ? l[0] : T(0), pa, pb, p0, l_inv, l_kneq, l_v);
             if (N.valid) adj_send(at(N.k, 0), Q.q, pa, pb, p0, tag0);
+            adj_kneq(N, l_kneq);
             add_v(ns - 1, l_v);
         }
         bool ok = true;
@@ -3192,6 +3195,7 @@ __global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const 
             if (m > 0) {
                 adj_psi(d, Q, N, r, th, U, V, la, lb, l0, pa, pb, p0, l_inv, l_kneq, l_v);
                 if (N.valid && ok) adj_send(at(N.k, i + 1), Q.q, pa, pb, p0, tag0 + i + 1);
+                adj_kneq(N, l_kneq);
                 add_v(m - 1, l_v);
             } else if (N.valid) {
                 put_out(N.k, la, lb, l0);
@@ -3208,6 +3212,7 @@ __global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const 
             adj_psi(d, Q, N, adj_rec(d, Q, N, rec, ns - 1), th, U, V, l[1 + Q.ia], l[1 + Q.ib], Q.q == 0 ? l[0] : T(0), pa,
                     pb, p0, l_inv, l_kneq, l_v);
             adj_put(Q, N, x0, pa, pb, p0);
+            adj_kneq(N, l_kneq);
             adj_node_out(d, Q, N, lsnap);
         }
         add_v(ns - 1, l_v);
@@ -3241,6 +3246,7 @@ __global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const 
                     T pa, pb, p0;
                     adj_psi(d, Q, N, adj_rec(d, Q, N, rec, m - 1), th, U, V, la, lb, l0, pa, pb, p0, l_inv, l_kneq, l_v);
                     adj_put(Q, N, nxt, pa, pb, p0);
+                    adj_kneq(N, l_kneq);
                     adj_node_out(d, Q, N, lsnap);
                 } else if (N.valid) {
                     put_out(N.k, la, lb, l0);
@@ -3418,13 +3424,14 @@ __global__ void k_adj_stream(Dev<T> d, StepArgs a, const T* lfB, const T* lSn, T
         T dr, rho, ux, uy;
         mom_d(f, T(d.rho0), dr, rho, ux, uy);
         const T om = 1.0 / T(d.tau_s);
+        const T k0 = T(1.0 - double(om)), k1 = T(1.0 - double(om) - double(k0));  // 1 - omega
         const int64_t s = (int64_t)y * d.pitch + x;
         T lam[9], mu[9], eq[9];
         feq_all(dr, rho, ux, uy, eq);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             lam[i] = lfB[i * d.plane + s];
-            mu[i] = (T(1) - om) * lam[i];
+            mu[i] = sizeof(T) == 8 ? k0 * lam[i] : fma_rn(lam[i], k0, lam[i] * k1);
             l_om -= lam[i] * (f[i] - eq[i]);
         }
         jfeqT_add(ux, uy, lam, om, mu);
