@@ -401,7 +401,10 @@ int hlbm_sweep_fv_time(hlbm_sweep_t* w, int64_t nsteps, double* fv_ms);
  * tiles neither can hold even with more, smaller tiles stays unpacked.  enable = 0 undoes it (the tuner's tiling,
  * or the default one before hlbm_sweep_tune).  n_packs (may be NULL) receives
  * the number of packs.  Results do not change: a node's arithmetic does not
- * depend on its tile or launch.  hlbm_sweep_tune after this call undoes it. */
+ * depend on its tile or launch.  hlbm_sweep_tune after this call undoes it.
+ * After hlbm_set_fv_depth on a packed solver the solvers of its pack are
+ * launched one by one, until the next call of this, unless their new tiles
+ * still take one block per SM of one kernel. */
 int hlbm_sweep_pack(hlbm_sweep_t* w, int32_t enable, int32_t* n_packs);
 const char* hlbm_sweep_last_error(const hlbm_sweep_t* w);
 void hlbm_sweep_destroy(hlbm_sweep_t* w);

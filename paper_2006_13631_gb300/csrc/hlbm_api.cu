@@ -1841,6 +1841,7 @@ struct hlbm_sweep {
     std::vector<int32_t> tile_nodes;    // target nodes per FV tile chosen by the tuner (0: default)
     std::vector<std::vector<int>> packs; // instances whose FV sub-steps share one launch
     std::vector<int> pack_of;           // instance -> pack index, -1 when launched alone
+    int sms = 0;                        // blocks a pack may have
     std::vector<cudaEvent_t> ev_pack;   // one per pack: its launch is done
     std::string err;
 };
@@ -1864,6 +1865,19 @@ int inst_retile(hlbm* h, int tiles, int kind = HLBM_FV_AUTO) {
 int tuned_tiles(const hlbm_sweep* w, int i) {
     const int c = w->tile_nodes[i];
     return c > 0 ? (w->inst[i]->patch.n_nodes + c - 1) / c : 0;
+}
+
+// Whether pack p still has the tiles of one launch: hlbm_set_fv_depth rebuilds
+// an instance's tiles as for a launch of its own, perhaps of another kernel, and
+// the pack's instances are then launched one by one
+bool pack_whole(const hlbm_sweep* w, size_t p) {
+    const int kind = w->inst[w->packs[p][0]]->fv_kind;
+    int blocks = 0;
+    for (int i : w->packs[p]) {
+        if (w->inst[i]->fv_kind != kind) return false;
+        blocks += w->inst[i]->n_tiles;
+    }
+    return (kind == HLBM_FV_DEEP || kind == HLBM_FV_TMEM) && blocks <= w->sms;
 }
 
 // The FV sub-steps of pack p's instances in one cooperative launch on the
@@ -1919,14 +1933,19 @@ int sweep_one_step(hlbm_sweep* w, bool time_fv) {
         }
         cudaEventRecord(w->ev_lat[i], w->streams[i]);
     }
+    std::vector<char> done(n, 0);  // stepped by its pack's launch
     for (size_t p = 0; p < w->packs.size(); ++p) {
-        for (int i : w->packs[p]) cudaStreamWaitEvent(w->fv, w->ev_lat[i], 0);
+        if (!pack_whole(w, p)) continue;
+        for (int i : w->packs[p]) {
+            cudaStreamWaitEvent(w->fv, w->ev_lat[i], 0);
+            done[i] = 1;
+        }
         int rc = w->inst[w->packs[p][0]]->dtype != HLBM_F64 ? pack_fv<float>(w, p, ps) : pack_fv<double>(w, p, ps);
         if (rc != HLBM_OK) return rc;
         cudaEventRecord(w->ev_pack[p], w->fv);
     }
     for (size_t i = 0; i < n; ++i) {
-        if (w->pack_of.size() == n && w->pack_of[i] >= 0) {
+        if (done[i]) {
             cudaEventRecord(w->ev_fv[i], w->fv);  // after its pack's launch on the same stream
             continue;
         }
@@ -3150,6 +3169,7 @@ int hlbm_sweep_pack(hlbm_sweep_t* w, int32_t enable, int32_t* n_packs) {
         int sms = 0, dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        w->sms = sms;
         std::vector<int> order;
         for (int i = 0; i < n; ++i)
             if (w->inst[i]->patch.outer_fv == 0 && w->inst[i]->patch.fv_kernel == HLBM_FV_AUTO) order.push_back(i);
