@@ -328,7 +328,8 @@ int hlbm_info(hlbm_t* h, hlbm_info_t* info);
  * layers cost redundant work and shared memory.  The tiles are rebuilt
  * with the largest interval up to `depth` (1 .. HLBM_FV_MAX_DEPTH) that
  * fits on the device (default 2; 1 for FP64 tiles of more than 18 nodes,
- * without outer_fv); the results do not change, bit for bit.
+ * without outer_fv, and for FP64 solvers in a pack); the results do not
+ * change, bit for bit.
  * Synchronises the stream.  HLBM_EINVAL for another depth. */
 #define HLBM_FV_MAX_DEPTH 4
 int hlbm_set_fv_depth(hlbm_t* h, int32_t depth);

@@ -856,9 +856,9 @@ int build_tiles(hlbm* h, int n_tiles_req, int kind = HLBM_FV_AUTO) {
     int deep_quads = 0;
     if ((want == HLBM_FV_AUTO || (want == HLBM_FV_DEEP && h->patch.outer_fv == 0)) && max_row - 1 <= 7) {
         // a pack of FP64 solvers fills the SMs' FP64 pipes, as large tiles do
-        const int depth = kind != HLBM_FV_AUTO && sizeof(T) == 8 ? 1
-                          : h->fv_depth > 0                      ? std::min(h->fv_depth, kDeepMaxK)
-                                                                 : default_depth<T>(tile_cap, h->patch.outer_fv);
+        const int depth = h->fv_depth > 0                          ? std::min(h->fv_depth, kDeepMaxK)
+                          : kind != HLBM_FV_AUTO && sizeof(T) == 8 ? 1
+                                                                   : default_depth<T>(tile_cap, h->patch.outer_fv);
         for (int K = depth; K >= 1 && !deep_ok; --K) {
             if (!build_deep_tables(h, tile_start, owner, K, fv_deep_tmem_slots<T>(), fv_deep_early<T>(), deep)) continue;
             // FP64, few computed slots: four lanes per node

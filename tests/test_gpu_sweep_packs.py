@@ -63,6 +63,26 @@ def test_depth_set_on_packed_solvers(dtype, changed):
     sw.close()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_packs_take_the_depth_asked_for(dtype):
+    from paper_2006_13631_gb300 import Solver, Sweep, hlbm_set_fv_depth
+
+    ws = _workloads(dtype)
+    packed, alone = [Solver(w) for w in ws], [Solver(w) for w in ws]
+    for s in packed:
+        hlbm_set_fv_depth(s.h, 3)
+    sw = Sweep(packed)
+    assert sw.pack() == 1
+    assert [s.info()["fv_depth"] for s in packed] == [3, 3]
+    sw.step(3)
+    for s in alone:
+        s.step(3)
+    torch.cuda.synchronize()
+    for a, b in zip(packed, alone):
+        _same(a, b)
+    sw.close()
+
+
 def test_depth_set_on_one_solver_of_a_tensor_memory_pack():
     """Five solvers whose tiles are too large for the deep kernel: the changed one
     has the deep kernel's tables afterwards and the others do not."""
