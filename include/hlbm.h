@@ -390,7 +390,8 @@ int hlbm_sweep_step(hlbm_sweep_t* w, int64_t nsteps);
  * fastest.  The trial steps advance the solvers like hlbm_sweep_step.
  * tile_nodes (may be NULL) receives the chosen size per instance. */
 int hlbm_sweep_tune(hlbm_sweep_t* w, int32_t trial_steps, int32_t* tile_nodes);
-/* nsteps sweep steps with the FV time of each instance summed into fv_ms[n]. */
+/* nsteps sweep steps with the FV time of each instance summed into fv_ms[n]
+ * (of an instance in a pack: the time of the pack's launches). */
 int hlbm_sweep_fv_time(hlbm_sweep_t* w, int64_t nsteps, double* fv_ms);
 /* Packs the sweep's solvers into shared FV launches (enable = 1): solvers of
  * the same precision whose sub-step counts lie within 25 % of each other,

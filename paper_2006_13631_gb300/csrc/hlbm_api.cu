@@ -1933,15 +1933,20 @@ int sweep_one_step(hlbm_sweep* w, bool time_fv) {
         }
         cudaEventRecord(w->ev_lat[i], w->streams[i]);
     }
+    std::vector<int> timed(n);  // the instance whose events time the launch that steps i
     std::vector<char> done(n, 0);  // stepped by its pack's launch
+    for (size_t i = 0; i < n; ++i) timed[i] = (int)i;
     for (size_t p = 0; p < w->packs.size(); ++p) {
         if (!pack_whole(w, p)) continue;
         for (int i : w->packs[p]) {
             cudaStreamWaitEvent(w->fv, w->ev_lat[i], 0);
             done[i] = 1;
+            timed[i] = w->packs[p][0];
         }
+        if (time_fv) cudaEventRecord(w->fv_t0[w->packs[p][0]], w->fv);
         int rc = w->inst[w->packs[p][0]]->dtype != HLBM_F64 ? pack_fv<float>(w, p, ps) : pack_fv<double>(w, p, ps);
         if (rc != HLBM_OK) return rc;
+        if (time_fv) cudaEventRecord(w->fv_t1[w->packs[p][0]], w->fv);
         cudaEventRecord(w->ev_pack[p], w->fv);
     }
     for (size_t i = 0; i < n; ++i) {
@@ -1967,9 +1972,9 @@ int sweep_one_step(hlbm_sweep* w, bool time_fv) {
     }
     if (time_fv) {
         for (size_t i = 0; i < n; ++i) {
-            cudaEventSynchronize(w->fv_t1[i]);
+            cudaEventSynchronize(w->fv_t1[timed[i]]);
             float ms = 0.f;
-            if (cudaEventElapsedTime(&ms, w->fv_t0[i], w->fv_t1[i]) == cudaSuccess) w->fv_ms[i] += ms;
+            if (cudaEventElapsedTime(&ms, w->fv_t0[timed[i]], w->fv_t1[timed[i]]) == cudaSuccess) w->fv_ms[i] += ms;
         }
     }
     return HLBM_OK;

@@ -83,6 +83,20 @@ def test_packs_take_the_depth_asked_for(dtype):
     sw.close()
 
 
+def test_fv_time_of_a_pack():
+    """Several timed steps of a packed sweep: every solver of the pack gets the
+    time of the shared launches."""
+    from paper_2006_13631_gb300 import Solver, Sweep
+
+    solvers = [Solver(w) for w in _workloads("f32")]
+    sw = Sweep(solvers)
+    assert sw.pack() == 1
+    ms = sw.fv_time(3)
+    assert ms[0] > 0 and ms[0] == ms[1]
+    assert all(s.status == 0 and s.info()["time"] == 3 for s in solvers)
+    sw.close()
+
+
 def test_depth_set_on_one_solver_of_a_tensor_memory_pack():
     """Five solvers whose tiles are too large for the deep kernel: the changed one
     has the deep kernel's tables afterwards and the others do not."""
