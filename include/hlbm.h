@@ -340,8 +340,8 @@ int hlbm_set_fv_depth(hlbm_t* h, int32_t depth);
  * every lattice node outside step t+1's window and the nodes pulling from it
  * (the only nodes that step t+1's relocation, classification and eq. 178
  * feed change), on warps of its own, or where the patch leaves SMs without
- * a tile, on those; step t+1's stream-collide then covers that rectangle
- * alone.  The results are the same bits either way.  Across
+ * a tile, on those, when they are expected to end in time; step t+1's
+ * stream-collide then covers that rectangle alone.  The results are the same bits either way.  Across
  * hlbm_step calls the precomputed part is kept (hlbm_load, hlbm_clear_status
  * and an injected lattice fault drop it).  enable = 0 runs each step's
  * stream-collide whole, before its FV launch. */

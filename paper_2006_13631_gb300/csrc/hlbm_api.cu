@@ -458,6 +458,21 @@ int step_lattice(hlbm* h, cudaStream_t s, PendingStep& ps) {
     return HLBM_OK;
 }
 
+// Whether `idle` SMs without a tile, on which the two-lane FV launch can run the
+// next step's stream-collide, end before the FV sub-steps and a stream-collide
+// of its own would have: 72 bytes a node at 40 GB/s per SM (measured with 55 to
+// 135 of them), or as little as 2 TB/s in all where many SMs share a large
+// lattice (from 391e3 = 135 SMs x 2896 on; 332e3 = 81 x 4096 keeps the 40 GB/s;
+// the cause is not known), against 1.6 us a sub-step and 6.7 TB/s.  Step us with / without:
+// 4096^2 beside 1048 nodes, n = 64: 641 / 317, 4544 nodes 397 / 321, with
+// n = 150 398 / 446; 2896^2 beside 2516 nodes, n = 24: 192 / 178, n = 64:
+// 192 / 237; 2048^2 beside 6204 nodes, n = 24: 184 / 133, n = 64: 184 / 189.
+bool far_pays(int idle, double nodes, int n_sub) {
+    const double bytes = 72.0 * nodes;
+    const double per_us = idle * std::sqrt(nodes) <= 3.5e5 ? 40e3 * idle : 2e6;
+    return idle > 0 && bytes / per_us < 1.6 * n_sub + bytes / 6.7e6;
+}
+
 // FarArgs of the next step's stream-collide outside its near rectangle, when
 // the spare warps of the FV kernel can run it: FP32 lattice, deep-tile FV,
 // one lattice level, a prescribed motion (the next window is known)
@@ -468,8 +483,8 @@ bool far_args(hlbm* h, const PendingStep& ps, FarArgs<T>& far) {
         h->motion.kind == HLBM_MOTION_INDUCED)
         return false;
     // with two lanes per node the FV blocks have no lattice warps: the SMs
-    // without a tile run the lattice, when they are enough to end before the FV
-    if (d.deep_duo && 4 * (d.deep_sms - h->n_tiles) < d.deep_sms) return false;
+    // without a tile run the lattice
+    if (d.deep_duo && !far_pays(d.deep_sms - h->n_tiles, (double)d.nx * d.ny, d.n_sub)) return false;
     double X, Y;
     motion_pos(h->motion, ps.a.t + 1, &X, &Y);
     int bx0, by0;
