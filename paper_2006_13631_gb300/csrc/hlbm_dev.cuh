@@ -67,10 +67,11 @@ __device__ __forceinline__ T cdot(int i, T x, T y) {
 
 enum : int8_t { CLS_DISC = 0, CLS_INTERP = 1, CLS_UNUSED = 2 };
 
-// Polls of a neighbour tile's progress counter before an FV wait gives up
-// (with the kernels' short sleeps between polls: well under a second), sets
-// HLBM_ST_SYNC_TIMEOUT and the abort flag, and returns.
-constexpr long kSpinLimit = 1L << 23;
+// Polls of a neighbour tile's packet or progress counter before an FV wait gives
+// up, sets HLBM_ST_SYNC_TIMEOUT and the abort flag, and returns: about a second.
+// A poll takes 0.24 us in the deep kernel, which does not sleep in between, 0.38
+// in the tensor- and shared-memory kernels and 0.53 in the global-memory one.
+constexpr long kSpinLimit = 1L << 21;
 
 // patch node record: f'[9], q[6], pad
 constexpr int kRec = 16;
@@ -241,7 +242,7 @@ struct Dev {
     const int32_t* tile_nb;
     unsigned long long* progress;
     unsigned* abort_flag;
-    long spin_limit;   // polls of a neighbour's counter before the wait gives up
+    long spin_limit;   // polls of a neighbour's packet or counter before the wait gives up
     int stall_tile;    // fault injection: this tile never releases its counter (-1: none)
     // deep tiles (HLBM_FV_DEEP): each tile holds its own nodes and deep_k
     // layers of ghost nodes as local slots and exchanges records with its

@@ -3176,7 +3176,7 @@ __global__ void __launch_bounds__(128) k_adj_fv_rev(Dev<T> d, StepArgs a, const 
                 for (int e = 0; e < E; ++e) have = adj_recv(at(ecol[e], i), Q.q, fa[e], fb[e], f0[e], tag0 + i) && have;
                 if (__all_sync(0xffffffffu, have || !N.valid)) break;
                 if ((spins & 63) == 63) ok = !*(volatile unsigned*)d.abort_flag;
-                if (spins > d.spin_limit) {
+                if (spins > d.spin_limit / E) {  // E packets a turn
                     atomicOr(d.status, HLBM_ST_SYNC_TIMEOUT);
                     atomicExch(d.abort_flag, 1u);
                     ok = false;
