@@ -458,19 +458,23 @@ int step_lattice(hlbm* h, cudaStream_t s, PendingStep& ps) {
     return HLBM_OK;
 }
 
-// Whether `idle` SMs without a tile, on which the two-lane FV launch can run the
-// next step's stream-collide, end before the FV sub-steps and a stream-collide
-// of its own would have: 72 bytes a node at 40 GB/s per SM (measured with 55 to
-// 135 of them), or as little as 2 TB/s in all where many SMs share a large
-// lattice (from 391e3 = 135 SMs x 2896 on; 332e3 = 81 x 4096 keeps the 40 GB/s;
-// the cause is not known), against 1.6 us a sub-step and 6.7 TB/s.  Step us with / without:
-// 4096^2 beside 1048 nodes, n = 64: 641 / 317, 4544 nodes 397 / 321, with
-// n = 150 398 / 446; 2896^2 beside 2516 nodes, n = 24: 192 / 178, n = 64:
-// 192 / 237; 2048^2 beside 6204 nodes, n = 24: 184 / 133, n = 64: 184 / 189.
-bool far_pays(int idle, double nodes, int n_sub) {
-    const double bytes = 72.0 * nodes;
-    const double per_us = idle * std::sqrt(nodes) <= 3.5e5 ? 40e3 * idle : 2e6;
-    return idle > 0 && bytes / per_us < 1.6 * n_sub + bytes / 6.7e6;
+// How many of the `idle` SMs without a tile the two-lane FV launch takes for the
+// next step's stream-collide: none when that would end later than the FV
+// sub-steps and a stream-collide of its own would; at 72 bytes a node, 40 GB/s
+// per SM (measured with 55 to 112 of them), 1.6 us a sub-step and 6.7 TB/s.  No
+// more than end with half of the sub-steps' time to spare: the launch is
+// cooperative, and blocks it has no use for keep the launches of other solvers,
+// on other streams, waiting for it (eight solvers on 203^2 lattices stepped
+// together: 145 us a step, 327 with a block on every SM).  No more than
+// 3e5 / sqrt(nodes): above, many SMs on a large lattice can get as little as
+// 2 TB/s in all (120 x 2896 and 112 x 4096 did; the cause is not known).
+// Step us with / without: 4096^2 beside 1048 nodes, n = 64: 641 / 317, 4544 nodes
+// 397 / 321, with n = 150 398 / 446; 2896^2 beside 2516 nodes, n = 24: 192 / 178,
+// n = 64: 192 / 237; 2048^2 beside 6204 nodes, n = 24: 184 / 133, n = 64: 184 / 189.
+int far_blocks(int idle, double nodes, int n_sub) {
+    const double bytes = 72.0 * nodes, sm = 40e3, fv = 1.6 * n_sub;  // bytes, bytes per us, us
+    const double m = std::min({(double)idle, std::floor(3e5 / std::sqrt(nodes)), std::ceil(1.5 * bytes / (sm * fv))});
+    return m >= 1.0 && bytes / (sm * m) < fv + bytes / 6.7e6 ? (int)m : 0;
 }
 
 // FarArgs of the next step's stream-collide outside its near rectangle, when
@@ -484,7 +488,8 @@ bool far_args(hlbm* h, const PendingStep& ps, FarArgs<T>& far) {
         return false;
     // with two lanes per node the FV blocks have no lattice warps: the SMs
     // without a tile run the lattice
-    if (d.deep_duo && !far_pays(d.deep_sms - h->n_tiles, (double)d.nx * d.ny, d.n_sub)) return false;
+    far.blocks = d.deep_duo ? far_blocks(d.deep_sms - h->n_tiles, (double)d.nx * d.ny, d.n_sub) : 0;
+    if (d.deep_duo && far.blocks < 1) return false;
     double X, Y;
     motion_pos(h->motion, ps.a.t + 1, &X, &Y);
     int bx0, by0;

@@ -195,6 +195,7 @@ struct FarArgs {
     int n_seg;      // chunks per row
     int n_chunks;   // 0: no lattice work
     unsigned* next; // zero at the launch
+    int blocks;     // two lanes per node: blocks of the launch that run the chunks
 };
 
 template <typename T>

@@ -2614,7 +2614,7 @@ cudaError_t launch_fv_deep(const Dev<T>& d, const StepArgs& a, const FarArgs<T>*
                  : d.fv_rec ? (const void*)k_fv_duo<true, false>
                             : (const void*)k_fv_duo<false, false>;
             threads = kDuoThreads;
-            if (fa.n_chunks > 0) blocks = std::max(blocks, d.deep_sms);  // the other SMs run the lattice
+            if (fa.n_chunks > 0) blocks += fa.blocks;  // on SMs without a tile
         }
     }
     return cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(threads), args, smem, s);
