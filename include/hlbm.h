@@ -307,7 +307,7 @@ typedef struct {
     int64_t n_struct_disc; /* discretization nodes in the last step       */
     int32_t n_nodes, n_tris, nnz, n_outer, n_wall_segments;
     int32_t box_w, box_h;  /* lattice window that follows the patch       */
-    int32_t launches_per_step; /* kernels per step (with levels: the most)     */
+    int32_t launches_per_step; /* kernels per step, at most (no absorbing layer) */
     int32_t dtype;
     int32_t fv_kernel; /* HLBM_FV_* in use                                */
     int32_t n_tiles;   /* FV tiles (blocks of the FV launch)               */
@@ -387,7 +387,9 @@ int hlbm_sweep_step(hlbm_sweep_t* w, int64_t nsteps);
 /* Tile-size autotuner for the FV kernels: for each candidate size (256,
  * 512, 1024, 1536 nodes per tile) every instance is re-tiled and
  * trial_steps sweep steps are timed per instance; each instance keeps the
- * fastest.  The trial steps advance the solvers like hlbm_sweep_step.
+ * fastest.  The default tiling, one tile per SM of at least 64 nodes (FP64:
+ * 16), is not among them; small patches run faster with it, or in a pack.  The
+ * trial steps advance the solvers like hlbm_sweep_step.
  * tile_nodes (may be NULL) receives the chosen size per instance. */
 int hlbm_sweep_tune(hlbm_sweep_t* w, int32_t trial_steps, int32_t* tile_nodes);
 /* nsteps sweep steps with the FV time of each instance summed into fv_ms[n]
@@ -440,7 +442,7 @@ int hlbm_theta_gradient(const hlbm_grid_t* grid, const hlbm_patch_t* patch, doub
  * segments between checkpoints from the last to the first: each is stepped
  * again from its checkpoint keeping what every step's reverse needs, and
  * the steps are reversed one by one -- force, the n FV sub-steps of eq. ulbe
- * (recomputed), the outer-node feed (eq. postcollision2_u), stream-collide
+ * (their sums recorded as they are stepped again), the outer-node feed (eq. postcollision2_u), stream-collide
  * (eq. LBE), the eq. postcollision2_s fill and the refill of Sec. 4 -- with
  * every decision of the forward step held fixed (node classes, refill types,
  * donor cells and triangles; Theta is smooth in the parameters between
@@ -452,8 +454,10 @@ int hlbm_theta_gradient(const hlbm_grid_t* grid, const hlbm_patch_t* patch, doub
  * of the reverse sweep.  HARMONIC motion, one lattice level, outer_fv = 0,
  * no absorbing layer (sponge_rows = 0), FP64 or FP32 populations (adjoints
  * in the population type, the parameter sums in FP64).  Device memory: one lattice
- * copy per checkpoint and per step of a segment, released before the call
- * returns.  Errors as for hlbm_create (message: hlbm_last_error(NULL)). */
+ * copy per checkpoint and per step of a segment, and the FV records of a segment's
+ * steps, 16 values per node and sub-step, when the device has room for them and
+ * they take no more than 8 GiB (otherwise those of one step, made again step by
+ * step); released before the call returns.  Errors as for hlbm_create (message: hlbm_last_error(NULL)). */
 int hlbm_theta_adjoint(const hlbm_grid_t* grid, const hlbm_patch_t* patch, double tau_s, const hlbm_motion_t* motion,
                        int64_t nsteps, double discard_periods, double fit_periods, double w_re, double w_im,
                        int32_t checkpoint_every, void* cuda_stream, double* theta, double* grad, double* fwd_ms,

@@ -84,8 +84,8 @@ struct hlbm {
     // with this tile never releasing its counter and this spin limit
     int inject_stall_tile = -1;
     long inject_spin_limit = 0;
-    // the next step's stream-collide away from the patch, run by the spare
-    // warps of the FP32 deep-tile FV kernel (FarArgs): far_ready when the
+    // the next step's stream-collide away from the patch, run by warps or blocks
+    // of the FP32 deep-tile FV launch that step no node (FarArgs): far_ready when the
     // current post-collision buffer's successor already holds it outside
     // far_rect, which the next stream-collide then covers alone
     int overlap = 1;
@@ -478,8 +478,8 @@ int far_blocks(int idle, double nodes, int n_sub) {
 }
 
 // FarArgs of the next step's stream-collide outside its near rectangle, when
-// the spare warps of the FV kernel can run it: FP32 lattice, deep-tile FV,
-// one lattice level, a prescribed motion (the next window is known)
+// the FV launch can run it beside the patch: FP32 lattice, deep-tile FV, one
+// lattice level, a prescribed motion (the next window is known)
 template <typename T>
 bool far_args(hlbm* h, const PendingStep& ps, FarArgs<T>& far) {
     Dev<T>& d = dev_of<T>(h);
@@ -2987,9 +2987,10 @@ int hlbm_info(hlbm_t* h, hlbm_info_t* info) {
     info->n_wall_segments = h->nseg;
     info->box_w = bw;
     info->box_h = bh;
-    // refill, classify, fill, stream-collide, feed, FV sub-steps, force (2)
-    // with levels: + one coupling launch and one stream-collide per level
-    // at a step where all of them start (every 2^n_levels steps)
+    // at most: refill (with classification), fill, stream-collide (two under the
+    // overlap), feed, FV sub-steps, force (2); with levels: + one coupling launch
+    // and one stream-collide per level at a step where all of them start (every
+    // 2^n_levels steps)
     info->launches_per_step = 8 + 2 * (int32_t)h->lv.size();
     info->n_levels = (int32_t)h->lv.size();
     info->n_coarse = 0;

@@ -181,8 +181,8 @@ struct StepArgs {
     unsigned xtag;  // deep tiles: exchange b of this step's FV launch carries the tag xtag + b
 };
 
-// The next lattice step's stream-collide outside a rectangle, run by the
-// spare warps of the FV kernel while the FV sub-steps of this step run:
+// The next lattice step's stream-collide outside a rectangle, run by warps or
+// blocks of the FV launch that step no node while the FV sub-steps of this step run:
 // the nodes outside [ex0, ex1) x [ey0, ey1) (the next step's window with the
 // pull margin; ex0, ex1 multiples of 4) pull from src (the post-collision
 // state at t+1, written by this step's stream-collide) and write dst, in

@@ -1381,8 +1381,9 @@ size_t fv_deep_packet_bytes(int n) {
     return (size_t)2 * n * kPkts<T> * 16;
 }
 
-// Quads (FP64, small tiles; rows in shared memory instead of tensor memory):
-// one row is 7 entries (g.c of the four axes, C, column) and a header
+// Quads (FP64, small tiles): rows in shared memory, one is 7 entries (g.c of the
+// four axes, C, column) and a header.  They are a branch of the kernel that keeps
+// a node per lane's rows in tensor memory, which is allocated all the same.
 struct alignas(16) QuadEntry {
     double k[4];  // gx, gy, gx + gy, gx - gy
     double c;
@@ -2954,7 +2955,7 @@ __global__ void k_adj_force(Dev<T> d, double lamF, T* lP) {
 //   psi_k + sum_P [ dt (c_j . g_Pk) psi_P,j - dt / tau_u C_Pk psi_P,j ]
 //         + dt / tau_u (J_feq(k)^T sum_P C_Pk psi_P)_j
 // over the rows P that read k.  psi of the sub-step before it is formed from
-// that at the node itself, so a sub-step is one pass and one grid barrier.
+// that at the node itself, so a sub-step is one pass and one exchange.
 // It needs only what the forward sub-step recorded (adj_record): its collision
 // sums, velocities and the wall moments; J_feq needs u alone, since its B
 // terms carry the rho they are divided by.  Four lanes share a node as in the
@@ -2964,7 +2965,7 @@ __global__ void k_adj_force(Dev<T> d, double lamF, T* lP) {
 // Reverse sweep of 48 steps on the 3008-node FP64 patch (n = 50): 404 ms with
 // a node per thread on 24 SMs, three grid barriers per sub-step and the sums
 // formed again, 62 ms so; 160 steps of the 2588-node FP32 patch (n = 96):
-// 664 ms and 115 ms.
+// 664 ms and 94 ms.
 template <typename T>
 __device__ __forceinline__ ANode<T> adj_node(const Dev<T>& d, const AQuad<T>& Q, int k, bool valid) {
     ANode<T> N;
