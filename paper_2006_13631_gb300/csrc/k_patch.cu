@@ -2032,8 +2032,7 @@ __device__ __forceinline__ void take_packet_duo(float* buf, int cap, int x, int 
     }
 }
 
-// One chunk of the next lattice step's stream-collide (FarArgs, FP32'''
-
+// One chunk of the next lattice step's stream-collide (FarArgs, FP32
 // storage) on the lattice warps: row y = c / n_seg, nodes [64 seg,
 // 64 seg + 64), two per lane.  The pull and BGK arithmetic of a node is that
 // of k_stream_collide (the same pulled values through bgk_dev; edge nodes
